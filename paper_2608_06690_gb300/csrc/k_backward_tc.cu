@@ -546,52 +546,79 @@ __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams 
 
 // ------------------------------------------------------------- wgrad
 
+// On CTA pairs (tc_ptx.cuh): a tile is 256 rows of M (2I or H) x up to 256
+// columns of N; each CTA stages its 128 rows of A and its half of B's columns
+// (32 KB a stage at N = 256) and drains its own 128 rows.  What bounds it is
+// the FP32 gradients: 604 MB written and 210 MB of operands read at Qwen3
+// prefill (16,384 private rows) are 120 us at the measured copy rate.  The
+// epilogue must keep up with short K loops (8 steps, about 4,300 clocks, at
+// 512 rows an expert): boxes of 4 KB, three in flight a warp, take it out of
+// the way (2 KB boxes, two in flight: 5,600 clocks a tile).  Training step at
+// Qwen3 T = 4096 1184 -> 1177 us, at the DeepSeek shape T = 3000 1559 -> 1542
+// us against single-CTA 128 x 256 tiles.
+constexpr int kWgStages = 5;
+constexpr int kWgStageBytes = 2 * kABytes;
+constexpr int kWgLoaders = 2;
+constexpr int kWgOutBufs = 3;              // per epilogue warp, boxes of 32 rows x 32 FP32 columns
+constexpr int kWgOutBoxBytes = 32 * 128;
+constexpr int kWgDynSmem = kWgStages * kWgStageBytes + 4 * kWgOutBufs * kWgOutBoxBytes + 1024;
+
 struct WgParams {
     int E_pub, E_priv, H, I, R;
     // the group table's groups (the private experts alone, g0 = E_pub, or all
     // routed experts, g0 = 0, whose padded layout the operands then use) and
     // the table index of private expert 0
     int g0, G, q_off;
-    int bn_a, bn_b;  // output columns per tile: [dW_gate; dW_up] (N = H), dW_down (N = I)
     const uint32_t *offsets;
     uint32_t *status;
-    uint32_t idesc_a, idesc_b;
+    uint32_t idesc;  // M = 256, both operands MN-major, N = 0 (added per tile)
 };
 
 struct WgMaps {
-    // 3-D maps, boxes of 64 rows (K) x 64-element MN blocks (encode_3d_blocks)
-    CUtensorMap dgu;        // [padded rows][2I], 2 blocks per box (MN-major A)
-    CUtensorMap a_perm;     // [R][H], bn_a / 128 blocks per box (MN-major B)
-    CUtensorMap dout_rows;  // [R + 64][H], 2 blocks per box (MN-major A)
-    CUtensorMap wact;       // [padded rows][I], bn_b / 128 blocks per box (MN-major B)
-    CUtensorMap d_gate, d_up, d_down;  // FP32 outputs, 16 x 32 boxes, 64-byte swizzle
+    // 3-D maps, boxes of 64 rows (K) x 64-element MN blocks (encode_3d_blocks):
+    // A: a CTA's 128 rows of M, 2 blocks; B [0]: its half of 256 columns, 2
+    // blocks, [1]: of a last tile of 128 columns, 1 block
+    CUtensorMap dgu;         // [padded rows][2I] (A)
+    CUtensorMap a_perm[2];   // [R][H] (B)
+    CUtensorMap dout_rows;   // [R + 64][H] (A)
+    CUtensorMap wact[2];     // [padded rows][I] (B)
+    CUtensorMap d_gate, d_up, d_down;  // FP32 outputs, 32 x 32 boxes, 128-byte swizzle
 };
 
 struct WgTile {
     int prob, q, m0, n0, bn, nkb;
 };
 
+// M blocks of 256 and N blocks of at most 256 (H and I are multiples of 128;
+// 2I is one of 256).
+__device__ __forceinline__ int wg_blocks(int n) { return (n + 255) / 256; }
+
+__device__ __forceinline__ int wg_total(const WgParams &p)
+{
+    return p.E_priv * (p.I / 128 * wg_blocks(p.H) + wg_blocks(p.H) * wg_blocks(p.I));
+}
+
 __device__ __forceinline__ WgTile decode_wg(const WgParams &p, const GroupTable &gt, int tile)
 {
     WgTile t;
-    const int na = p.H / p.bn_a, nta = (2 * p.I / BM) * na;
-    const int nb = p.I / p.bn_b, ntb = (p.H / BM) * nb;
+    const int na = wg_blocks(p.H), nta = p.I / 128 * na;
+    const int nb = wg_blocks(p.I), ntb = wg_blocks(p.H) * nb;
     int local;
     if (tile < p.E_priv * nta) {
         t.prob = 0;
         t.q = tile / nta;
         local = tile - t.q * nta;
-        t.m0 = (local / na) * BM;
-        t.n0 = (local % na) * p.bn_a;
-        t.bn = p.bn_a;
+        t.m0 = (local / na) * 256;
+        t.n0 = (local % na) * 256;
+        t.bn = min(256, p.H - t.n0);
     } else {
         tile -= p.E_priv * nta;
         t.prob = 1;
         t.q = tile / ntb;
         local = tile - t.q * ntb;
-        t.m0 = (local / nb) * BM;
-        t.n0 = (local % nb) * p.bn_b;
-        t.bn = p.bn_b;
+        t.m0 = (local / nb) * 256;
+        t.n0 = (local % nb) * 256;
+        t.bn = min(256, p.I - t.n0);
     }
     t.nkb = (gt.rows[t.q + p.q_off] + BK - 1) / BK;
     return t;
@@ -601,80 +628,83 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
 {
     extern __shared__ uint8_t dsmem[];
     __shared__ GroupTable gt;
-    __shared__ __align__(8) uint64_t bars[2 * kStages + 5];
+    __shared__ __align__(8) uint64_t bars[2 * kWgStages + 5];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_ctarank();  // 0: the leader, whose thread issues the pair's MMAs
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const uint32_t sbase = (smem_u32(dsmem) + 1023u) & ~1023u;
     const uint32_t bar0 = smem_u32(bars);
+    // full (both CTAs' copies) and tempty (both CTAs' epilogues) are the
+    // leader's; empty and tfull are signalled in both CTAs by the commits
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
-    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
-    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kStages + 2 + b); };
-    const uint32_t done_bar = bar0 + 8u * (2 * kStages + 4);
+    auto empty_bar = [&](int s) { return bar0 + 8u * (kWgStages + s); };
+    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kWgStages + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kWgStages + 2 + b); };
+    const uint32_t done_bar = bar0 + 8u * (2 * kWgStages + 4);
 
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), kLoaders); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 4); }
+        for (int s = 0; s < kWgStages; ++s) { mbar_init(full_bar(s), kWgLoaders); mbar_init(empty_bar(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
         mbar_init(done_bar, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
+    if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
     build_groups(gt, p.offsets, p.g0, p.G, p.R, 0, 0, 0);
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();  // both CTAs' barriers and TMEM are ready
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
-    const int total = p.E_priv * ((2 * p.I / BM) * (p.H / p.bn_a) + (p.H / BM) * (p.I / p.bn_b));
+    const int total = wg_total(p);
     const int p0 = (int)min(p.offsets[p.g0], (uint32_t)p.R);
 
-    if (warp == 0 && lane < kLoaders) {
+    if (warp == 0 && lane < kWgLoaders) {
         // ------------------------------------------------ TMA producers
-        // lane 0: the two 64-element MN blocks of A; lanes 1-2: half of B's
-        // bn / 64 blocks each; one 3-D box per lane (64 MN elements x 64 rows of
-        // K per block).
+        // lane 0: this CTA's two 64-element MN blocks of A; lane 1: its half of
+        // B's bn / 64 blocks; one 3-D box per lane (64 MN elements x 64 rows of
+        // K per block).  Every copy completes on the leader's barrier, where
+        // the leader's lanes announce both CTAs' bytes.
         int stage = 0;
         uint32_t phase = 0, filled = 0, last_parity = 0;
-        for (int tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x) {
+        for (int tile = pair; tile < total && !s_abort; tile += pairs) {
             const WgTile t = decode_wg(p, gt, tile);
-            const int nbox = t.bn / 64, half = nbox / 2;
+            const int half = t.bn / 128;  // MN blocks of B per CTA
             const int gq = t.q + p.q_off;  // the expert's entry in the group table
             const int rowA = t.prob == 0 ? gt.pad[gq] : gt.off[gq];
             const int rowB = t.prob == 0 ? p0 + gt.off[gq] : gt.pad[gq];
             const CUtensorMap *amap = t.prob == 0 ? &maps.dgu : &maps.dout_rows;
-            const CUtensorMap *bmap = t.prob == 0 ? &maps.a_perm : &maps.wact;
+            const CUtensorMap *bmap = t.prob == 0 ? &maps.a_perm[2 - half] : &maps.wact[2 - half];
             bool ok = true;
             for (int kb = 0; kb < t.nkb; ++kb) {
                 if (!mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status)) { ok = false; break; }
-                const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
+                const uint32_t sA = sbase + stage * kWgStageBytes, sB = sA + kABytes;
+                const uint32_t fb = dsmem_addr(full_bar(stage), 0);
                 const int ky = kb * BK;
-                mbar_expect_tx(full_bar(stage), lane == 0 ? (uint32_t)kABytes : (uint32_t)(half * kMnBlockBytes));
-                if (lane == 0) {
-                    tma_load_3d(sA, amap, full_bar(stage), 0, rowA + ky, t.m0 / 64);
-                } else {
-                    const int b0 = (lane - 1) * half;
-                    tma_load_3d(sB + b0 * kMnBlockBytes, bmap, full_bar(stage), 0, rowB + ky, t.n0 / 64 + b0);
-                }
+                if (rank == 0)
+                    mbar_expect_tx(full_bar(stage), 2u * (lane == 0 ? (uint32_t)kABytes : (uint32_t)(half * kMnBlockBytes)));
+                if (lane == 0) tma_load_3d_pair(sA, amap, fb, 0, rowA + ky, t.m0 / 64 + 2 * rank);
+                else tma_load_3d_pair(sB, bmap, fb, 0, rowB + ky, t.n0 / 64 + half * rank);
                 filled |= 1u << stage;
                 last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                if (++stage == kWgStages) { stage = 0; phase ^= 1u; }
             }
             if (!ok) break;
         }
-        drain_stages(bar0, kStages, filled, last_parity);
+        if (rank == 0) drain_stages(bar0, kWgStages, filled, last_parity);  // both CTAs' copies
     } else if (warp == 1 && lane == 0) {
         // ------------------------------------------------ MMA issuer
-        // two 128 x 256 FP32 accumulators: the epilogue of one tile overlaps the
+        // two 256-column FP32 accumulators: the epilogue of one tile overlaps the
         // MMAs of the next.  A tile of an expert without rows issues no MMA;
         // its epilogue writes zeros.
         int stage = 0, it = 0;
         uint32_t phase = 0;
-        for (int tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x, ++it) {
+        for (int tile = pair; rank == 0 && tile < total && !s_abort; tile += pairs, ++it) {
             const WgTile t = decode_wg(p, gt, tile);
-            const uint32_t idesc = t.prob == 0 ? p.idesc_a : p.idesc_b;
+            const uint32_t idesc = p.idesc | ((uint32_t)(t.bn >> 3) << 17);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
             if (!mbar_wait(tempty_bar(buf), use ^ 1u, &s_abort, p.status)) break;
@@ -684,27 +714,29 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
             for (int kb = 0; kb < t.nkb; ++kb) {
                 if (!mbar_wait(full_bar(stage), phase, &s_abort, p.status)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
+                const uint32_t sA = sbase + stage * kWgStageBytes, sB = sA + kABytes;
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    tc_mma(d_tmem, mn_sw128_desc(sA + k * 2048, kMnBlockBytes), mn_sw128_desc(sB + k * 2048, kMnBlockBytes),
-                           idesc, (kb | k) != 0);
-                tc_commit(empty_bar(stage));
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                    tc_mma_pair(d_tmem, mn_sw128_desc(sA + k * 2048, kMnBlockBytes),
+                                mn_sw128_desc(sB + k * 2048, kMnBlockBytes), idesc, (kb | k) != 0);
+                tc_commit_pair(empty_bar(stage));
+                if (++stage == kWgStages) { stage = 0; phase ^= 1u; }
             }
             if (!ok) break;
-            tc_commit(tfull_bar(buf));
+            tc_commit_pair(tfull_bar(buf));
         }
-        tc_commit(done_bar);
+        // the leader's last commit: its MMAs and every commit before (whose
+        // arrivals reach both CTAs) are done before either CTA exits
+        if (rank == 0) tc_commit_pair(done_bar);
         const unsigned long long t0 = globaltimer_ns();
         while (!mbar_try_wait(done_bar, 0))
             if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     } else if (warp >= 2) {
         // ------------------------------------------------ epilogue
         const int quarter = warp & 3;
-        OutStager out{sbase + kStages * kStageBytes + (uint32_t)((warp - 2) * kOutBufs * kOutBoxBytes), 0};
-        int it = 0;
-        for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++it) {
+        const uint32_t out0 = sbase + kWgStages * kWgStageBytes + (uint32_t)((warp - 2) * kWgOutBufs * kWgOutBoxBytes);
+        int it = 0, ob = 0;
+        for (int tile = pair; tile < total; tile += pairs, ++it) {
             const WgTile t = decode_wg(p, gt, tile);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
@@ -714,19 +746,21 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
             if (!ok) break;
             __syncwarp();
             tc_fence_after();
+            const int m0 = t.m0 + rank * BM;  // this CTA's 128 rows
+            const bool inside = m0 < (t.prob == 0 ? 2 * p.I : p.H);  // (H may end inside the pair's 256 rows)
             const CUtensorMap *omap;
             int orow;
             if (t.prob == 0) {
-                omap = t.m0 < p.I ? &maps.d_gate : &maps.d_up;
-                orow = t.q * p.I + (t.m0 < p.I ? t.m0 : t.m0 - p.I);
+                omap = m0 < p.I ? &maps.d_gate : &maps.d_up;
+                orow = t.q * p.I + (m0 < p.I ? m0 : m0 - p.I);
             } else {
                 omap = &maps.d_down;
-                orow = t.q * p.H + t.m0;
+                orow = t.q * p.H + m0;
             }
             orow += quarter * 32;
             const uint32_t tb = tmem_base + (uint32_t)(buf * 256) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-            for (int c = 0; c < t.bn / 32; ++c) {
+            for (int c = 0; inside && c < t.bn / 32; ++c) {
                 float v[32];
                 if (t.nkb > 0) {
                     tmem_ld32(tb + c * 32, v);
@@ -735,22 +769,40 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
 #pragma unroll
                     for (int i = 0; i < 32; ++i) v[i] = 0.f;
                 }
-                out.put(lane, reinterpret_cast<const uint32_t *>(v), omap, t.n0 + c * 32, orow);
-                out.put(lane, reinterpret_cast<const uint32_t *>(v + 16), omap, t.n0 + c * 32 + 16, orow);
+                // a box of 32 rows of 128 bytes, 16-byte chunk j of row r at chunk
+                // j ^ (r & 7): the TMA 128-byte swizzle, conflict-free here
+                const uint32_t sbuf = out0 + (uint32_t)(ob * kWgOutBoxBytes);
+                if (lane == 0) bulk_wait_read<kWgOutBufs - 1>();  // the store that used this buffer has read it
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(sbuf + lane * 128 + ((j ^ (lane & 7)) << 4)),
+                                 "f"(v[4 * j]), "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
+                                 : "memory");
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_2d(omap, sbuf, t.n0 + c * 32, orow);
+                    bulk_commit();
+                }
+                ob = ob == kWgOutBufs - 1 ? 0 : ob + 1;
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(buf));
+            if (lane == 0) {
+                if (rank == 0) mbar_arrive(tempty_bar(buf));
+                else mbar_arrive_remote(dsmem_addr(tempty_bar(buf), 0));
+            }
         }
         if (lane == 0) bulk_wait_all();
     }
 
     __syncwarp();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();  // the pair's MMAs, copies and barrier arrivals are done
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc_pair(tmem_base, kTmemCols);
     }
 }
 
@@ -903,26 +955,25 @@ cudaError_t launch_backward_wgrad(const Ctx &c, const bf16 *dout_rows, const bf1
     p.g0 = all ? 0 : s.E_pub;
     p.G = all ? s.E() : s.E_priv;
     p.q_off = all ? s.E_pub : 0;
-    p.bn_a = s.H % 256 == 0 ? 256 : 128;
-    p.bn_b = s.I % 256 == 0 ? 256 : 128;
     p.offsets = c.offsets;
     p.status = c.audit.status;
-    p.idesc_a = make_idesc_major(BM, p.bn_a, true, true);
-    p.idesc_b = make_idesc_major(BM, p.bn_b, true, true);
-    // A: both 64-element MN blocks in one box; B: half of its blocks per box
+    p.idesc = make_idesc_major(2 * BM, 0, true, true);
     bool ok = encode_3d_blocks(&maps.dgu, dgu, 2 * (uint64_t)s.I, RP, 64, 2);
-    ok &= encode_3d_blocks(&maps.a_perm, c.a_perm, s.H, R, 64, p.bn_a / 128);
     ok &= encode_3d_blocks(&maps.dout_rows, dout_rows, s.H, R + 64, 64, 2);
-    ok &= encode_3d_blocks(&maps.wact, wact, s.I, RP, 64, p.bn_b / 128);
-    const CUtensorMapSwizzle osw = CU_TENSOR_MAP_SWIZZLE_64B;
-    ok &= encode_2d_f32(&maps.d_gate, d_gate, s.H, (uint64_t)s.E_priv * s.I, 16, 32, osw);
-    ok &= encode_2d_f32(&maps.d_up, d_up, s.H, (uint64_t)s.E_priv * s.I, 16, 32, osw);
-    ok &= encode_2d_f32(&maps.d_down, d_down, s.I, (uint64_t)s.E_priv * s.H, 16, 32, osw);
+    for (int h = 0; h < 2; ++h) {  // full tiles of 256 columns; a last one of 128
+        ok &= encode_3d_blocks(&maps.a_perm[h], c.a_perm, s.H, R, 64, 2 - h);
+        ok &= encode_3d_blocks(&maps.wact[h], wact, s.I, RP, 64, 2 - h);
+    }
+    const CUtensorMapSwizzle osw = CU_TENSOR_MAP_SWIZZLE_128B;
+    ok &= encode_2d_f32(&maps.d_gate, d_gate, s.H, (uint64_t)s.E_priv * s.I, 32, 32, osw);
+    ok &= encode_2d_f32(&maps.d_up, d_up, s.H, (uint64_t)s.E_priv * s.I, 32, 32, osw);
+    ok &= encode_2d_f32(&maps.d_down, d_down, s.I, (uint64_t)s.E_priv * s.H, 32, 32, osw);
     if (!ok) return cudaErrorInvalidValue;
     static std::atomic<int> smem_limit[64];
-    cudaError_t err = ensure_dynamic_smem(bwd_wgrad_tc_kernel, kDynSmem, smem_limit);
+    cudaError_t err = ensure_dynamic_smem(bwd_wgrad_tc_kernel, kWgDynSmem, smem_limit);
     if (err != cudaSuccess) return err;
-    return launch_pdl(bwd_wgrad_tc_kernel, dim3(c.num_sms), dim3(kThreads), kDynSmem, c.stream, p, maps);
+    return launch_cluster_pdl(bwd_wgrad_tc_kernel, 2, dim3(c.num_sms / 2 * 2), dim3(kThreads), kWgDynSmem, c.stream, p,
+                              maps);
 }
 
 }  // namespace pmpe

@@ -647,22 +647,6 @@ static int cluster_router_smem(int P, int k, int nq)
     return (after > kCRingBytes ? after : kCRingBytes) + 1024;
 }
 
-__device__ __forceinline__ uint32_t cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ uint32_t dsmem_addr(uint32_t local, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(local), "r"(rank));
-    return r;
-}
 __device__ __forceinline__ uint32_t dsmem_ld_u32(uint32_t addr)
 {
     uint32_t v;
