@@ -341,8 +341,6 @@ int grid_for(long long work, int num_sms)
 
 }  // namespace
 
-int column_block(int H) { return H % 256 == 0 ? 256 : 128; }
-
 cudaError_t launch_permute(const Ctx &c)
 {
     const Shape &s = c.s;

@@ -8,54 +8,78 @@
 // Groups are the routed experts (rows of the dispatch order) plus, with
 // shared experts, one dense group over all T tokens (gate/up weights of the
 // E_sh experts side by side; the down projection sums the E_sh experts in
-// one accumulator).  A persistent grid (one CTA per SM) walks a tile list
-// built on the device from the dispatch offsets: no host sync, and empty
-// experts contribute no tile.  The list holds every gate/up tile, then every
-// down tile, group by group, n-tile major inside a group.  The CTAs take the
-// tiles in list order: in waves (CTA c: tiles c, c + grid, ...) when a group
-// has several 128-row blocks, so that the m-tiles sharing weights run
-// together, and otherwise dynamically, each CTA the next tile when its loader
-// is ready for one (an atomic counter), which evens out tiles of unequal
-// cost.  Warp 0 hands each tile index to the CTA's other roles through a
-// small queue in shared memory.  A down tile waits (bounded) until the
-// gate/up tiles of its activation rows have stored them; every one of those
-// was handed out earlier to a running CTA, and no gate/up tile ever waits,
-// so the wait ends.
+// one accumulator).
 //
-// The routed gate/up tiles read their A rows straight from the hidden states:
-// the row of dispatch slot r is hidden[tok_of_slot[r]], gathered into shared
-// memory by four warps with 16-byte cp.async copies (the hidden states, read
-// by every expert a token routes to, stay in L2), so the dispatched rows are
-// never written out.  The gather warps never wait for their own copies: each
-// thread's copies of a stage arrive on the stage's full barrier when they
-// complete (cp.async.mbarrier.arrive), and the MMA thread fences the async
-// proxy after that barrier, before the tensor cores read the rows.
+// The grid is persistent, one CTA per SM in CTA pairs (cta_group::2,
+// tc_ptx.cuh).  The weights are the MMA's M and the tokens its N: a pair's
+// tile is 256 weight rows (gate/up: each CTA 64 gate and the same 64 up
+// columns; down: 128 output columns each) x N tokens of one expert, N any
+// multiple of 32 up to 256, half of them staged by each CTA.  N follows the
+// expert's rows, so a tile computes at most 31 padding rows (128-row M tiles
+// computed 31 % padding at Qwen3 prefill), and a full tile stages 32 KB per CTA
+// and 64-wide K step for what a single CTA's 128 x 256 tile stages 48 KB.
+// The ring's stages are as large as the launch's largest N needs: 6 of 32 KB
+// at N = 256, 10 of 18 KB at N = 32 (decode), so that a batch of few rows per
+// expert keeps 160 KB of weights in flight per SM.
 //
-// CTA roles (320 threads):
-//   warp 0       three lanes issue the TMA loads of a 4-stage ring, one
-//                operand box each (A: 128 rows x 64 K of the activations or,
-//                for the shared group, of the hidden states; B: 256 rows x
-//                64 K, i.e. 128 gate + 128 up rows, or 256 / 128 output
-//                columns of the down projection in two halves)
-//   warp 1       allocates 512 TMEM columns (two 128 x 256 FP32
-//                accumulators, so the epilogue of one tile overlaps the MMAs
-//                of the next) and one thread issues tcgen05.mma M=128 N=256
-//                K=16, committing stage releases and accumulator-full events
-//   warps 2..5   epilogue: tcgen05.ld of the warp's 32 TMEM lanes (= 32 tile
-//                rows), SwiGLU or weight scaling, BF16 stores; in gate/up mode
-//                the tiles of N-tile 0 also write the execution audit, each
-//                row checked against the route log of its token
-//   warps 6..9   the A-row gather of the routed gate/up tiles (cp.async into
-//                the ring)
-// Expert weights stream through L2 once and are loaded with an evict-first
-// policy; the hidden states and activations, read again by other tiles of
-// the launch, with evict-last.
+// What bounds it: HBM (the weights) up to a few thousand tokens, then the rate
+// at which L2 delivers the operands (32 KB a stage and CTA in 512 clocks at the
+// full MMA rate).  Forward, against single-CTA tiles of 128 tokens x 256 weight
+// rows: Qwen3 shape T = 4096 437 -> 366 us, T = 16384 1229 -> 1037 us, T = 777
+// 271 -> 264 us, T = 64 213 -> 211 us; DeepSeek shape T = 8192 1020 -> 867 us.
+// Half of that is the roles' own time a stage (tc_ptx.cuh: the waits' timer, the
+// elected lane) and a tile (the queue below).
+//
+// The pairs walk a tile list built on the device from the dispatch offsets:
+// no host sync, and empty experts contribute no tile.  The list holds every
+// gate/up tile, then every down tile, group by group, weight-block major inside
+// a group, so that the tiles sharing weights are next to each other.  Each pair
+// takes the next tile when its loader is ready for one (an atomic counter);
+// the leader hands it to the roles of both CTAs through a small queue in
+// shared memory.  A down tile waits (bounded) until the gate/up tiles of its
+// activation rows have stored them; every one of those was handed out earlier
+// to a running pair, and no gate/up tile ever waits, so the wait ends.
+//
+// The routed gate/up tiles read their token rows straight from the hidden
+// states: the row of dispatch slot r is hidden[tok_of_slot[r]], gathered into
+// shared memory by eight warps with 16-byte cp.async copies (the hidden states,
+// read by every expert a token routes to, stay in L2), so the dispatched rows
+// are never written out.  The gather warps never wait for their own copies:
+// each thread's copies of a stage arrive on a barrier when they complete
+// (cp.async.mbarrier.arrive): the leader's on the stage's full barrier; the
+// other CTA's on one of its own, where its warp 0 waits, fences the async proxy
+// and arrives on the leader's.
+//
+// CTA roles (480 threads):
+//   warp 0       hands out the tiles (leader) and loads the token rows that
+//                come through TMA (activations or, for the shared group, hidden
+//                states), completing on the leader's barrier
+//   warp 1       allocates 512 TMEM columns (two accumulators of 256 columns,
+//                so the epilogue of one tile overlaps the MMAs of the next);
+//                the leader's issues tcgen05.mma M = 256, K = 16
+//   warps 2..5   epilogue: tcgen05.ld of the warp's 32 TMEM lanes (= 32 weight
+//                columns).  Gate/up: the gate columns sit in warps 0-1's lanes
+//                and the up columns in warps 2-3's; the two warps of a column
+//                swap half of each 32-token chunk through shared memory, so
+//                each computes the SwiGLU of 16 tokens.  Results are transposed
+//                through shared memory into row-major 64-byte runs.  In gate/up
+//                mode the tiles of weight block 0 also write the execution audit,
+//                each row checked against the route log of its token
+//   warps 6..13  the row gather of the routed gate/up tiles (cp.async), two
+//                groups of four warps taking turns
+//   warp 14      the weights through TMA, two 64-row boxes a stage
+// Warps 0, 1 and 14 run their loops as whole warps and issue TMA and MMA
+// instructions from one elected lane.
+// Expert weights that only one tile reads stream through L2 (evict first);
+// the hidden states and activations, read again by other tiles of the launch,
+// are kept (evict last).
 // Every wait is bounded in time: on expiry the CTA records
 // PMPE_STATUS_PIPELINE_TIMEOUT, stops issuing work, waits (bounded) for its
 // own copies and MMAs in flight, frees its TMEM and exits.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -65,19 +89,20 @@
 namespace pmpe {
 namespace {
 
-constexpr int BM = 128;                       // rows per tile (MMA M)
+constexpr int kMaxN = 256;                    // tokens per tile at most (MMA N; a multiple of 32)
+constexpr int kRowBlock = 128;                // rows per block of the execution audit's tile count
 constexpr int BK = 64;                        // K per stage: one 128-byte swizzle row
-constexpr int kStages = 4;
-constexpr int kABytes = BM * BK * 2;          // 16 KB
-constexpr int kBBytes = 256 * BK * 2;         // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kAccCols = 256;                 // FP32 TMEM columns per accumulator
+constexpr int kWBytes = 128 * BK * 2;         // a CTA's weight rows of a stage: 16 KB
+constexpr int kRingBytes = 6 * 2 * kWBytes;   // 6 stages at N = 256
+constexpr int kMaxStages = 10;                // at N = 32: 18 KB each
+constexpr int kAccCols = kMaxN;               // FP32 TMEM columns per accumulator
 constexpr int kTmemCols = 2 * kAccCols;
-constexpr int kGatherWarps = 4;               // warps 6..9
-constexpr int kThreads = 192 + 32 * kGatherWarps;
-constexpr int kLoaders = 3;                   // TMA-issuing lanes of warp 0
-constexpr int kGatherThreads = 32 * kGatherWarps;
-constexpr int kFullArrivals = kLoaders + kGatherThreads;  // per ring stage
+constexpr int kGatherGroups = 2;              // the row gather: groups of four warps, every other stage each
+constexpr int kGatherWarps = 4 * kGatherGroups;  // warps 6..13
+constexpr int kWeightWarp = 6 + kGatherWarps;
+constexpr int kThreads = 192 + 32 * kGatherWarps + 32;
+constexpr int kGatherThreads = 128;           // of a group: the arrivals of a gathered stage
+constexpr int kFullArrivals = 3 + kGatherThreads;  // the leader's token and weight loaders and gather, the other CTA's gather
 constexpr int kMaxGroups = 2 * kMaxPool + 1;
 constexpr int kPrefetchTiles = 96;            // gate/up tiles (1 MB of weights each) prefetched into L2 at small batches
 // Large batches, the launch following the router: the gate and up weights of
@@ -87,21 +112,18 @@ constexpr int kPrefetchTiles = 96;            // gate/up tiles (1 MB of weights 
 constexpr size_t kPrefillPrefetchBytes = 96ull << 20;
 constexpr int kPrefillPrefetchExperts = 16;
 constexpr unsigned long long kPrefillPrefetchDelayNs = 14000;
-constexpr int kTQ = 8;                        // tile queue entries (tile indices handed to the CTA's roles)
-constexpr int kTailWaves = 2;                 // waves of tiles at the list's end handed out dynamically
-constexpr int kTQConsumers = 1 + 4 + kGatherWarps;  // MMA thread, epilogue warps, gather warps (one lane each)
-constexpr int kOutBox = 32;                   // output staged and stored as 32 x 32 BF16 boxes (2 KB)
-constexpr int kOutBufBytes = kOutBox * kOutBox * 2;
-constexpr int kOutBytes = 4 * 2 * kOutBufBytes;  // 4 epilogue warps x 2 buffers
-constexpr int kDynSmem = kStages * kStageBytes + kOutBytes + 1024 /* alignment slack */;
+constexpr int kTQ = 8;                        // tile queue entries (tile indices handed to the pair's roles)
+constexpr int kHandOutStages = 8;             // K steps before a tile's last at which the next tile is handed out
+constexpr int kTQConsumers = 2 + 4 + kGatherWarps       // leader: MMA, weight, epilogue and gather warps (one lane each)
+                             + 2 + 4 + kGatherWarps;    // other CTA: both loaders, epilogue, gather
+constexpr int kStageOutBytes = 4096;          // per epilogue warp: two 2 KB exchange / transpose buffers
+constexpr int kRowWBytes = kMaxN * 4;         // per epilogue warp: the tile's routing weights
+constexpr int kDynSmem = kRingBytes + 4 * (kStageOutBytes + kRowWBytes) + 1024 /* alignment slack */;
+constexpr int kTokBoxes = 4;                  // token row boxes: 128, 64, 32, 16 rows
 
 enum { kGateUp = 0, kDown = 1 };
-enum { kTileGU = 0, kTileDown = 1 };
 
-// One GEMM of the layer: gate/up (SwiGLU fused) or down (routing weight fused).
 struct TcPhase {
-    int bn;           // output columns per tile (gate/up: 128 activation columns; down: 256 or 128)
-    uint32_t idesc;   // tcgen05 instruction descriptor (BF16 x BF16 -> FP32, M = 128, N = MMA width)
     bf16 *C_routed, *C_shared;
 };
 
@@ -109,16 +131,17 @@ struct TcParams {
     // which GEMMs this launch runs: the gate/up tiles, the down tiles
     int has_gu, has_down;
     TcPhase ph[2];    // [kGateUp], [kDown]
+    uint32_t idesc;   // tcgen05 instruction descriptor (BF16 x BF16 -> FP32, M = 256, N added per tile)
     int E, E_pub, E_sh, T, H, I, R, k;
     const uint32_t *offsets;
     const float *w_of_slot;
     const int32_t *tok_of_slot;
     const int32_t *topk_idx;  // [T, k] the route log, read back by the execution audit
     const bf16 *hidden;       // the gather source of the routed gate/up tiles
-    // has_gu && has_down: per (group, 128-row block), the gate/up epilogue
-    // warps whose activations are stored (zeroed before the launch)
+    // has_gu && has_down: per (group, row tile), the gate/up epilogue warps
+    // whose activations are stored (zeroed before the launch)
     uint32_t *ready;
-    // the next tile of the list to hand out (zeroed before the launch): CTAs
+    // the next tile of the list to hand out (zeroed before the launch): pairs
     // take tiles in list order, each when it is ready for one
     uint32_t *tile_ctr;
     uint32_t *exec_rows, *exec_tiles, *exec_priv_rows, *shared_rows, *status;
@@ -157,46 +180,63 @@ struct TcParams {
     int fuse_combine;
     uint32_t *bar_d;
     bf16 *out;                       // [T, H]
-    // small batches (every expert at most one 128-row block): the first
+    // small batches (at most 128 tokens: every expert one row tile): the first
     // `prefetch_tiles` gate/up tiles of the list of all experts have their
     // weights prefetched into L2 by the CTA of the same index, before the
     // launch waits for the routing (the weights are inputs, not results of
     // the kernels before); 0 = off
     int prefetch_tiles;
     int prefetch_experts;      // large batches: CTA e < this prefetches expert e's gate and up rows
+    uint8_t up_first[3];      // the box holds the up rows before the gate rows
+    uint8_t gu_two_boxes[3];
     const bf16 *gate_w[2], *up_w[2];  // [E_pool * I, H] public / private
     // optional FP32: the gate and up accumulators saved for the backward,
     // [R][2I] G | U of the routed rows, then [T][2 E_sh I] of the shared
-    // experts (gu_save / gu_save_sh maps for whole 32-row blocks)
+    // experts
     float *saved_gu;
 };
 
-struct TcMaps {  // [phase]
-    CUtensorMap c_routed[2], c_shared[2];  // outputs, 32 x 32 boxes, 64-byte swizzle
-    CUtensorMap a_routed[2], a_shared[2];
-    CUtensorMap b0[2][3];  // per pool [pub, priv, shared]: gate (gate/up) or down
-    CUtensorMap b1[2][3];  // up (gate/up)
-    CUtensorMap gu_save;   // saved_gu, routed rows [R][2I], 16 x 32 FP32 boxes, 64-byte swizzle
-    CUtensorMap gu_save_sh;  // saved_gu's shared part [T][2 E_sh I], the same boxes
+struct TcMaps {
+    // per pool [pub, priv, shared]: the gate and up rows of 64 columns as one
+    // 3-D box of both tensors (one dimension steps from one to the other), or
+    // (p.gu_two_boxes) 64-row boxes of each; down, 128-row boxes
+    CUtensorMap gu[3], gate[3], up[3], down[3];
+    CUtensorMap tok[2][kTokBoxes];     // per GEMM, by box rows: the shared group's hidden states; the activations
+    CUtensorMap tok_sh[kTokBoxes];     // the shared group's activations
 };
 
 // ------------------------------------------------------------- tile list
 
-struct Tile {
-    int kind, ph, bn, g, m_tile, m0, n0, rows, row_base, nkb, cb;
-    bool shared;
+// A tile as the queue carries it: two 16-byte words of shared memory.
+enum { kTileDown = 1, kTileShared = 2, kTileManyRows = 4, kTileEnd = 8 };
+struct __align__(16) Tile {
+    int flags;      // kTile...: the GEMM, the shared group, several row tiles read its weights, the list's end
+    int g, m_tile, m0, n0, rows, row_base, nkb;
+    __device__ __forceinline__ bool down() const { return flags & kTileDown; }
+    __device__ __forceinline__ bool shared() const { return flags & kTileShared; }
+    __device__ __forceinline__ bool gather() const { return (flags & (kTileDown | kTileShared)) == 0; }
+    __device__ __forceinline__ int n() const { return (rows + 31) & ~31; }
 };
 
 struct TileTable {
     int prefix[2][kMaxGroups + 1];  // tiles of the groups before g, per GEMM
-    int mpre[kMaxGroups + 1];       // 128-row blocks of the groups before g
+    int mpre[kMaxGroups + 1];       // row tiles of the groups before g
     int rows[kMaxGroups];
     int base[kMaxGroups];
 };
 
-__device__ __forceinline__ int group_n(const TcParams &p, int mode, bool shared)
+// Row tiles of a group of n rows: the fewest that hold 256 rows, of equal size
+// up to a multiple of 32 (equal tiles cost the same MMA time as full ones and a
+// remainder, and end together).
+__device__ __forceinline__ int row_tiles(int n) { return (n + kMaxN - 1) / kMaxN; }
+__device__ __forceinline__ int round32(int n) { return (n + 31) & ~31; }
+__device__ __forceinline__ int row_tile_size(int n, int mt) { return round32((n + mt - 1) / mt); }
+
+// Weight blocks of a group: 128 activation columns (gate and up rows) or 256
+// output columns (the last block of an H of 128 mod 256 half empty).
+__device__ __forceinline__ int group_blocks(const TcParams &p, int mode, bool shared)
 {
-    return mode == kGateUp ? (shared ? p.E_sh * p.I : p.I) : p.H;
+    return mode == kGateUp ? (shared ? p.E_sh * p.I : p.I) / 128 : (p.H + 255) / 256;
 }
 __device__ __forceinline__ int group_k(const TcParams &p, int mode, bool shared)
 {
@@ -228,44 +268,45 @@ __device__ __forceinline__ int down_place(const TcParams &p, int g)
     return g < h ? g : (g == p.E ? h : g + 1);
 }
 
-// Tile `tile` of the list: the gate/up tiles (when this launch runs them),
-// then the down tiles; inside a GEMM, group by group (the down GEMM in
-// down_group order), n-tile major.
-__device__ __forceinline__ Tile decode_tile(const TcParams &p, const TileTable &tt, int G, int tile)
+// Tile `tile` of the list (the end at `total`): the gate/up tiles (when this
+// launch runs them), then the down tiles; inside a GEMM, group by group (the
+// down GEMM in down_group order), weight-block major.  By a whole warp.
+__device__ __forceinline__ Tile decode_tile(const TcParams &p, const TileTable &tt, int G, int tile, int total, int lane)
 {
     Tile t;
-    const int n_gu = p.has_gu ? tt.prefix[kGateUp][G] : 0;
-    t.ph = tile < n_gu ? kGateUp : kDown;
-    t.kind = t.ph == kGateUp ? kTileGU : kTileDown;
-    const int local_all = tile - (t.ph == kDown ? n_gu : 0);
-    const int *pre = tt.prefix[t.ph];
-    int lo = 0, hi = G - 1;  // last group with prefix <= local_all
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pre[mid] <= local_all) lo = mid; else hi = mid - 1;
+    if (tile >= total) {
+        t.flags = kTileEnd;
+        t.g = t.m_tile = t.m0 = t.n0 = t.rows = t.row_base = t.nkb = 0;
+        return t;
     }
-    t.bn = p.ph[t.ph].bn;
-    const int g = t.ph == kDown ? down_group(p, lo) : lo;
-    t.g = g;
-    t.shared = g >= p.E;
-    const int rows = tt.rows[g];
-    const int mt = (rows + BM - 1) / BM;
+    const int n_gu = p.has_gu ? tt.prefix[kGateUp][G] : 0;
+    const int ph = tile < n_gu ? kGateUp : kDown;
+    const int local_all = tile - (ph == kDown ? n_gu : 0);
+    const int *pre = tt.prefix[ph];
+    int n = 0;  // groups with prefix <= local_all; the last of them holds the tile
+    for (int b = 0; b < G; b += 32) n += __popc(__ballot_sync(~0u, b + lane < G && pre[b + lane] <= local_all));
+    const int lo = n - 1;
+    const int g = ph == kDown ? down_group(p, lo) : lo;
+    const bool shared = g >= p.E;
+    const int rows = tt.rows[g], mt = row_tiles(rows);
     const int local = local_all - pre[lo];
-    const int n_tile = local / mt;
-    t.m_tile = local - n_tile * mt;
-    t.m0 = t.m_tile * BM;
-    t.n0 = n_tile * t.bn;
-    t.cb = n_tile;
-    t.rows = min(BM, rows - t.m0);
+    const int block = local / mt;
+    const int bm = row_tile_size(rows, mt);
+    t.flags = (ph == kDown ? kTileDown : 0) | (shared ? kTileShared : 0) | (mt > 1 ? kTileManyRows : 0);
+    t.g = g;
+    t.m_tile = local - block * mt;
+    t.m0 = t.m_tile * bm;
+    t.n0 = block * (ph == kGateUp ? 128 : 256);
+    t.rows = min(bm, rows - t.m0);
     t.row_base = tt.base[g];
-    t.nkb = group_k(p, t.ph == kGateUp ? kGateUp : kDown, t.shared) / BK;
+    t.nkb = group_k(p, ph, shared) / BK;
     return t;
 }
 
 // ---------------------------------------------------------------- kernel
 
 // Weights of gate/up tile blockIdx.x of the list of all experts (the first
-// wave when every expert has at most one 128-row block): 128 gate rows and
+// wave when every expert has one row tile): 128 gate rows and
 // 128 up rows, each block contiguous, prefetched into L2 by one thread.
 __device__ __forceinline__ void prefetch_first_wave(const TcParams &p)
 {
@@ -610,66 +651,75 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
 {
     extern __shared__ uint8_t dsmem[];
     __shared__ TileTable tt;
-    __shared__ __align__(8) uint64_t bars[2 * kStages + 5 + 2 * kTQ];
+    __shared__ __align__(8) uint64_t bars[3 * kMaxStages + 5 + 2 * kTQ];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
-    __shared__ volatile int s_tq[kTQ];
+    __shared__ Tile s_tq[kTQ];
     __shared__ volatile int s_pdl_done;  // thread 0 has passed griddepcontrol.wait
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(~0u, tid >> 5, 0), lane = tid & 31;
+    const int rank = (int)cluster_ctarank();  // 0: the pair's leader, whose thread issues the MMAs
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const uint32_t sbase = (smem_u32(dsmem) + 1023u) & ~1023u;
     const uint32_t bar0 = smem_u32(bars);
+    // The leader's: full (a stage's TMA bytes and gathered rows of both CTAs),
+    // tempty (both CTAs' epilogues), tq_empty.  The other CTA's: gfull (its
+    // gathered rows, which it reports to full).  Each CTA's own: empty, tfull (the commits' arrivals) and
+    // tq_full, which the leader signals in both.
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
-    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
-    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kStages + 2 + b); };
-    const uint32_t done_bar = bar0 + 8u * (2 * kStages + 4);
-    auto tq_full_bar = [&](int i) { return bar0 + 8u * (2 * kStages + 5 + i); };
-    auto tq_empty_bar = [&](int i) { return bar0 + 8u * (2 * kStages + 5 + kTQ + i); };
-    // Entry i of the CTA's tile sequence, for a consumer role (one thread):
-    // -1 at the end of the list or after an abort.  In wave order every role
-    // computes it; dynamically, warp 0 hands it out through the tile queue.
-    // The list's tiles [0, tail) go out in waves (CTA c: c, c + grid, ...,
-    // n_wave of them), the rest [tail, total) dynamically, through the queue.
-    int total = 0, tail = 0, n_wave = 0;
-    auto next_tile = [&](int i) -> int {
-        if (i < n_wave) return s_abort ? -1 : (int)blockIdx.x + i * (int)gridDim.x;
-        const int d = i - n_wave, slot = d % kTQ;
-        if (!mbar_wait(tq_full_bar(slot), (uint32_t)(d / kTQ) & 1u, &s_abort, p.status)) return -1;
-        const int t = s_tq[slot];
-        mbar_arrive(tq_empty_bar(slot));
-        return t;
+    auto empty_bar = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
+    auto gfull_bar = [&](int s) { return bar0 + 8u * (2 * kMaxStages + s); };
+    auto tfull_bar = [&](int b) { return bar0 + 8u * (3 * kMaxStages + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (3 * kMaxStages + 2 + b); };
+    const uint32_t done_bar = bar0 + 8u * (3 * kMaxStages + 4);
+    auto tq_full_bar = [&](int i) { return bar0 + 8u * (3 * kMaxStages + 5 + i); };
+    auto tq_empty_bar = [&](int i) { return bar0 + 8u * (3 * kMaxStages + 5 + kTQ + i); };
+    // Entry i of the pair's tile sequence, for a consumer role (a whole warp).
+    // False at the end of the list or after an abort.
+    auto next_tile = [&](int i, Tile &t) -> bool {
+        const int slot = i % kTQ;
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait(tq_full_bar(slot), (uint32_t)(i / kTQ) & 1u, &s_abort, p.status) ? 1 : 0;
+        if (!__shfl_sync(~0u, ok, 0)) return false;
+        const uint32_t a = smem_u32(&s_tq[slot]);
+        const uint4 x = ld_shared_v4(a), y = ld_shared_v4(a + 16);
+        t.flags = (int)x.x; t.g = (int)x.y; t.m_tile = (int)x.z; t.m0 = (int)x.w;
+        t.n0 = (int)y.x; t.rows = (int)y.y; t.row_base = (int)y.z; t.nkb = (int)y.w;
+        // (the vote needs every lane's entry: it is read before its slot is handed back)
+        const bool live = !__any_sync(~0u, t.flags & kTileEnd) && __all_sync(~0u, t.rows > 0 && t.nkb > 0);
+        if (lane == 0) {
+            if (rank == 0) mbar_arrive(tq_empty_bar(slot));
+            else mbar_arrive_remote(dsmem_addr(tq_empty_bar(slot), 0));
+        }
+        return live;
     };
 
     const int G = p.E + (p.E_sh > 0 ? 1 : 0);
-    // expert weights stream through L2 once (evict first); the hidden states,
-    // activations and per-row outputs are read again by other tiles of this
-    // launch (evict last)
+    // expert weights that one tile reads stream through L2 (evict first); the
+    // hidden states, activations and per-row outputs are read again by other
+    // tiles of this launch (evict last)
     const uint64_t pol_stream = l2_policy_evict_first(), pol_keep = l2_policy_evict_last();
+    const uint64_t pol_normal = l2_policy_evict_normal();
     if (warp == 0 && lane < 2) {  // the weight maps of this launch's GEMMs, ahead of their first loads
-        const int ph = lane == 0 ? kGateUp : kDown;
-        if (ph == kGateUp ? p.has_gu : p.has_down)
-            for (int q = 0; q < (p.E_sh > 0 ? 3 : 2); ++q) {
-                prefetch_tmap(&maps.b0[ph][q]);
-                if (ph == kGateUp) prefetch_tmap(&maps.b1[ph][q]);
-            }
+        if (lane == 0 ? p.has_gu : p.has_down)
+            for (int q = 0; q < (p.E_sh > 0 ? 3 : 2); ++q) prefetch_tmap(lane == 0 ? &maps.gu[q] : &maps.down[q]);
     }
     pdl_trigger();
 
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), kFullArrivals); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 4); }
+        for (int s = 0; s < kMaxStages; ++s) {
+            mbar_init(full_bar(s), kFullArrivals);
+            mbar_init(empty_bar(s), 1);
+            mbar_init(gfull_bar(s), kGatherThreads);
+        }
+        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
         mbar_init(done_bar, 1);
         for (int i = 0; i < kTQ; ++i) { mbar_init(tq_full_bar(i), 1); mbar_init(tq_empty_bar(i), kTQConsumers); }
         s_abort = 0;
         s_pdl_done = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
-                     "r"(kTmemCols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
-    }
+    if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
     __syncthreads();  // s_pdl_done and s_abort are initialised
     // weights of the first wave into L2 while the routing is computed (in
     // this launch: after this CTA's router rows have landed, which the
@@ -787,7 +837,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
         return true;
     };
     // tile list: rows and tiles per group, prefixes over groups
-    int multi = 0;  // some group has more than one 128-row block
+    int nmax = 0;  // bit b: some row tile has N = 32 (b + 1)
     for (int g = tid; g < G; g += kThreads) {
         const bool shared = g >= p.E;
         int rows, base;
@@ -802,16 +852,19 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
             rows = e - b;
             base = b;
         }
-        const int mt = (rows + BM - 1) / BM;
-        multi |= mt > 1 ? 1 : 0;
+        const int mt = row_tiles(rows);
+        if (mt > 0) nmax |= 1 << (row_tile_size(rows, mt) / 32 - 1);
         tt.rows[g] = rows;
         tt.base[g] = base;
         tt.mpre[g + 1] = mt;
-        tt.prefix[kGateUp][g + 1] = mt * (group_n(p, kGateUp, shared) / p.ph[kGateUp].bn);
-        tt.prefix[kDown][down_place(p, g) + 1] = mt * (group_n(p, kDown, shared) / p.ph[kDown].bn);
+        tt.prefix[kGateUp][g + 1] = mt * group_blocks(p, kGateUp, shared);
+        tt.prefix[kDown][down_place(p, g) + 1] = mt * group_blocks(p, kDown, shared);
     }
     // the same value in every thread of every CTA (all read the same offsets)
-    multi = __syncthreads_or(multi);
+    nmax = __reduce_or_sync(~0u, nmax);
+    __shared__ int s_nmax[kThreads / 32];
+    if (lane == 0) s_nmax[warp] = nmax;
+    __syncthreads();
     if (warp < 3) {  // three inclusive scans, one per warp: tiles of each GEMM, row blocks
         int *arr = warp == 2 ? tt.mpre : tt.prefix[warp];
         int carry = 0;
@@ -829,91 +882,96 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
         if (lane == 0) arr[0] = 0;
     }
     __syncwarp();
+    for (int w = 0; w < kThreads / 32; ++w) nmax |= s_nmax[w];
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();  // both CTAs' barriers, TMEM and tables are ready
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
-    total = total_tiles(p, tt, G);
-    // waves keep an expert's m-tiles (which share weights) running together;
-    // the last kTailWaves waves, and every tile when no group has a second
-    // 128-row block (nothing to share), go out dynamically, so that the CTAs
-    // finish together
-    tail = multi == 0 ? 0 : max(0, total - kTailWaves * (int)gridDim.x);
-    n_wave = (int)blockIdx.x < tail ? (tail - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int total = total_tiles(p, tt, G);
+    // the ring: stages of 16 KB of weights and half of the launch's largest
+    // N of token rows
+    const int stage_bytes = kWBytes + (nmax ? 32 - __clz(nmax) : 1) * (16 * BK * 2);
+    const int nst = min(kMaxStages, kRingBytes / stage_bytes);
 
-    if (warp == 0 && lane < kLoaders) {
-        // ------------------------------------------------ TMA producers
-        // Three lanes, one operand box each: a single thread's TMA boxes are
-        // processed one after another, so spreading a stage's boxes over
-        // three issuing threads triples the ring's fill rate.
-        //   lane 0: the A tile (128 rows x 64 K) when A comes through TMA (the
-        //           activations, or the hidden states of the shared group), and
-        //           then also the arrivals of the gather warps, which have
-        //           nothing to copy; in a routed gate/up tile the gather warps
-        //           fill A and lane 0 only arrives
-        //   lane 1: gate rows (gate/up) or B rows [0, bn/2) (down)
-        //   lane 2: up rows (gate/up)   or B rows [bn/2, bn) (down)
+    // A barrier wait by a whole warp: every lane waits, and the vote keeps the
+    // warp together (a lane left behind could be lapped) and gives one answer.
+    auto warp_wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        return __all_sync(~0u, mbar_wait(bar, parity, &s_abort, p.status));
+    };
+
+    if (warp == 0) {
+        // ------------------------------------------------ tile hand-out, token rows through TMA
+        // This CTA's half of the tile's token rows when they come through TMA
+        // (the activations, or the hidden states of the shared group; at most
+        // three boxes, of 128 to 16 rows); every copy completes on the leader's
+        // barrier, where the leader announces both CTAs' bytes.  In a gathered
+        // tile the other CTA's warp waits for its CTA's rows, fences the async
+        // proxy and arrives there for them.  (Each of these warps holds up
+        // every stage until it has passed it: a warp that only followed the
+        // ring could be lapped, which a parity wait cannot see.)  The leader
+        // picks the tiles (the first one by the pair's index, so that its
+        // weights load before the dispatch is final) and hands each to both
+        // CTAs' other roles.
         int stage = 0;
         uint32_t phase = 0;
-        uint32_t filled = 0, last_parity = 0;  // per-stage bits, for the drain below
-        // Lane 0 picks the tiles and hands each to the CTA's other roles
-        // through the tile queue.  When a group has several 128-row blocks,
-        // its m-tiles share weights: they sit next to each other in the list
-        // and the CTAs take the list in waves (CTA c: tiles c, c + grid, ...),
-        // so those m-tiles run at the same moment and one DRAM read of the
-        // weights serves them all.  When no group has (decode), nothing is
-        // shared, and the tiles go out dynamically, the next one to whichever
-        // CTA is ready (an atomic counter, taken one tile ahead), which
-        // evens out tiles of unequal cost.
-        uint32_t ahead = 0u;  // lane 0: the next dynamic tile, taken one ahead
+        int issued = 0;       // stages passed, for the drain below
+        uint32_t ahead = 0u;  // leader, lane 0: the next tile
         bool synced = false;  // lane 0: wait_dispatch has returned
-        for (int qi = 0;; ++qi) {
-            int tile = -1;
-            if (qi < n_wave) {
-                tile = next_tile(qi);
-            } else {
-                if (lane == 0) {
-                    const int d = qi - n_wave, slot = d % kTQ;
-                    if (d == 0) {
-                        if (!synced) synced = wait_dispatch();
-                        ahead = synced ? (uint32_t)tail + atomicAdd(p.tile_ctr, 1u) : (uint32_t)total;
-                    }
-                    if (mbar_wait(tq_empty_bar(slot), ((uint32_t)(d / kTQ) & 1u) ^ 1u, &s_abort, p.status) &&
-                        !s_abort && ahead < (uint32_t)total) {
-                        tile = (int)ahead;
-                        ahead = (uint32_t)tail + atomicAdd(p.tile_ctr, 1u);
-                    }
-                    s_tq[slot] = tile;
-                    mbar_arrive(tq_full_bar(slot));
-                }
-                tile = __shfl_sync((1u << kLoaders) - 1u, tile, 0);
+        // Leader: the next tile is taken when a tile starts and handed out
+        // kHandOutStages before its last stage (handed out after the last stage,
+        // every tile began with 1.4 us in which nothing was loaded; taken a tile
+        // earlier, the CTAs ended less evenly, 212 -> 216 us a decode step).
+        Tile t, next;
+        auto push = [&](int i, Tile &e) {
+            const int slot = i % kTQ;
+            if (lane == 0) {
+                if (!mbar_wait(tq_empty_bar(slot), ((uint32_t)(i / kTQ) & 1u) ^ 1u, &s_abort, p.status) || s_abort)
+                    e.flags |= kTileEnd;
+                const uint4 x = make_uint4((uint32_t)e.flags, (uint32_t)e.g, (uint32_t)e.m_tile, (uint32_t)e.m0);
+                const uint4 y = make_uint4((uint32_t)e.n0, (uint32_t)e.rows, (uint32_t)e.row_base, (uint32_t)e.nkb);
+                const uint32_t a = smem_u32(&s_tq[slot]);
+                st_shared_v4(a, x);
+                st_shared_v4(a + 16, y);
+                mbar_arrive(tq_full_bar(slot));
+                st_async_32(dsmem_addr(a, 1), x, y, dsmem_addr(tq_full_bar(slot), 1));
             }
-            if (tile < 0) break;
-            const Tile t = decode_tile(p, tt, G, tile);
-            const bool gather = t.kind == kTileGU && !t.shared;
-            const int q = t.shared ? 2 : (t.g < p.E_pub ? 0 : 1);
-            const int ei = t.shared ? 0 : (q == 0 ? t.g : t.g - p.E_pub);
-            const CUtensorMap *amap = t.shared ? &maps.a_shared[t.ph] : &maps.a_routed[t.ph];
-            const int arow = t.row_base + t.m0;
-            const uint32_t my_tx = lane == 0 ? (gather ? 0u : (uint32_t)kABytes)
-                                             : (t.ph == kGateUp ? (uint32_t)(BM * 128) : (uint32_t)(t.bn / 2 * 128));
-            bool ok = true;
-            if (t.kind == kTileDown && p.has_gu && lane == 0) {
+            e.flags = __shfl_sync(~0u, e.flags, 0);
+        };
+        if (rank == 0) {
+            t = decode_tile(p, tt, G, pair, total, lane);
+            push(0, t);
+        }
+        for (int qi = 0;; ++qi) {
+            if (rank == 0) {
+                if (t.flags & kTileEnd) break;
+                if (lane == 0) {
+                    if (!synced) synced = wait_dispatch();
+                    ahead = synced ? (uint32_t)pairs + atomicAdd(p.tile_ctr, 1u) : (uint32_t)total;
+                }
+            } else if (!next_tile(qi, t)) {
+                break;
+            }
+            const bool gather = t.gather();
+            const CUtensorMap *tmap = !t.down() ? maps.tok[kGateUp] : (t.shared() ? maps.tok_sh : maps.tok[kDown]);
+            const int tn = t.n(), trows = tn / 2;  // this CTA's token rows
+            const int trow = t.row_base + t.m0 + rank * trows;
+            int ok = 1;
+            if (t.down() && p.has_gu && lane == 0) {
                 // a down tile after the gate/up tiles of the same launch: its
                 // activation rows are complete once every gate/up epilogue
-                // warp of their row block has stored its part (bounded wait;
+                // warp of their row tile has stored its part (bounded wait;
                 // the weights are loaded meanwhile)
-                const uint32_t need = 4u * (uint32_t)(group_n(p, kGateUp, t.shared) / p.ph[kGateUp].bn);
+                const uint32_t need = 8u * (uint32_t)group_blocks(p, kGateUp, t.shared());
                 const uint32_t *rp = p.ready + tt.mpre[t.g] + t.m_tile;
                 if (!synced) synced = wait_dispatch();
-                if (!synced) ok = false;
+                if (!synced) ok = 0;
                 const unsigned long long t0 = globaltimer_ns();
                 while (ok && ld_acquire_gpu(rp) < need) {
-                    if (s_abort) { ok = false; break; }
+                    if (s_abort) { ok = 0; break; }
                     if (globaltimer_ns() - t0 > kWaitLimitNs) {
                         s_abort = 1;
                         if (p.status) atomicOr(p.status, PMPE_STATUS_PIPELINE_TIMEOUT);
-                        ok = false;
+                        ok = 0;
                         break;
                     }
                     __nanosleep(128);
@@ -921,81 +979,154 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
                 // the async proxy (TMA) reads what the generic acquire observed
                 asm volatile("fence.proxy.async.global;\n" ::: "memory");
             }
-            for (int kb = 0; kb < t.nkb && ok; ++kb) {
-                if (!mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status)) { ok = false; break; }
-                const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
-                mbar_expect_tx(full_bar(stage), my_tx);
-                const int kx = kb * BK;
-                if (lane == 0) {
-                    if (!gather) {
-                        tma_load_2d_hint(sA, amap, full_bar(stage), kx, arow, pol_keep);
-                        mbar_arrive_count(full_bar(stage), kGatherThreads);
+            ok = __all_sync(~0u, ok);
+            if (!ok) break;
+            auto advance = [&]() {
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+            };
+            // the boxes of this CTA's rows, largest first (1 to 3)
+            const int b0 = __clz(trows) - 24, r0 = 128 >> b0;  // trows is 16 .. 128
+            const int b1 = trows > r0 ? __clz(trows - r0) - 24 : -1, r1 = b1 < 0 ? 0 : r0 + (128 >> b1);
+            const int b2 = b1 >= 0 && trows > r1 ? __clz(trows - r1) - 24 : -1;
+            const int hand_out = max(t.nkb - kHandOutStages, 1);
+            int kb = 0;
+#pragma unroll 1
+            for (int part = 0; part < 2 && ok; ++part) {
+                const int end = part == 0 ? hand_out : t.nkb;
+                if (part == 1 && rank == 0) {
+                    next = decode_tile(p, tt, G, (int)min(__shfl_sync(~0u, ahead, 0), (uint32_t)total), total, lane);
+                    push(qi + 1, next);
+                }
+                if (gather && rank == 1) {
+                    for (; kb < end; ++kb, advance()) {
+                        if (!warp_wait(gfull_bar(stage), phase)) { ok = 0; break; }
+                        if (elect_one()) {
+                            fence_proxy_async_smem();
+                            mbar_arrive_remote(dsmem_addr(full_bar(stage), 0));
+                        }
                     }
-                } else if (t.ph == kGateUp) {
-                    const int brow = ei * p.I + t.n0;  // shared: n0 spans E_sh * I rows
-                    tma_load_2d_hint(sB + (lane - 1) * BM * 128, lane == 1 ? &maps.b0[t.ph][q] : &maps.b1[t.ph][q],
-                                     full_bar(stage), kx, brow, pol_stream);
+                } else if (gather) {
+                    for (; kb < end; ++kb, advance()) {
+                        if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = 0; break; }
+                        if (elect_one()) mbar_arrive(full_bar(stage));
+                    }
                 } else {
-                    const int half = (lane - 1) * (t.bn / 2);
-                    if (t.shared) {
-                        const int sidx = kx / p.I;
-                        tma_load_2d_hint(sB + half * 128, &maps.b0[t.ph][2], full_bar(stage), kx - sidx * p.I,
-                                         sidx * p.H + t.n0 + half, pol_stream);
-                    } else {
-                        tma_load_2d_hint(sB + half * 128, &maps.b0[t.ph][q], full_bar(stage), kx,
-                                         ei * p.H + t.n0 + half, pol_stream);
+                    for (; kb < end; ++kb, advance()) {
+                        if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = 0; break; }
+                        if (elect_one()) {
+                            const uint32_t sT = sbase + stage * stage_bytes + kWBytes;
+                            const uint32_t fb = dsmem_addr(full_bar(stage), 0);
+                            if (rank == 0) {
+                                mbar_expect_tx(full_bar(stage), (uint32_t)(tn * BK * 2));
+                                mbar_arrive_count(full_bar(stage), 1 + kGatherThreads);  // nothing is gathered
+                            }
+                            tma_load_2d_pair_hint(sT, &tmap[b0], fb, kb * BK, trow, pol_keep);
+                            if (b1 >= 0) tma_load_2d_pair_hint(sT + r0 * 128, &tmap[b1], fb, kb * BK, trow + r0, pol_keep);
+                            if (b2 >= 0) tma_load_2d_pair_hint(sT + r1 * 128, &tmap[b2], fb, kb * BK, trow + r1, pol_keep);
+                        }
                     }
                 }
-                filled |= 1u << stage;
-                last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            }
+            issued += t.nkb;
+            if (!ok) break;
+            if (rank == 0) t = next;
+        }
+        // drain: every copy of the pair has landed before its CTAs exit (the
+        // last use of each stage)
+        for (int s = 0; s < nst && rank == 0 && issued > 0; ++s) {
+            if (issued < nst && s >= stage) break;
+            const uint32_t last = s < stage ? phase : phase ^ 1u;
+            const unsigned long long t0 = globaltimer_ns();
+            while (!mbar_try_wait(full_bar(s), last))
+                if (globaltimer_ns() - t0 > kWaitLimitNs) break;
+        }
+    } else if (warp == kWeightWarp) {
+        // ------------------------------------------------ weights through TMA
+        // One 16 KB box a stage: 64 gate and 64 up rows, or 128 output columns'
+        // rows.  (A box costs the TMA unit about 180 clocks whatever its rows:
+        // as two boxes beside the tokens' one, a stage took 540 clocks even
+        // with every operand in L2.  The drain above covers these copies.)
+        int stage = 0;
+        uint32_t phase = 0;
+        int ok = 1;
+        Tile t;
+        for (int qi = 0; next_tile(qi, t); ++qi) {
+            const int q = t.shared() ? 2 : (t.g < p.E_pub ? 0 : 1);
+            const int ei = t.shared() ? 0 : (q == 0 ? t.g : t.g - p.E_pub);
+            const bool gu = !t.down(), two = p.gu_two_boxes[q];
+            const uint64_t wpol = (t.flags & kTileManyRows) ? pol_normal : pol_stream;
+            // shared gate/up: n0 spans E_sh * I rows; shared down: the experts
+            // one after another along K
+            int y = gu ? ei * p.I + t.n0 + rank * 64 : ei * p.H + t.n0 + rank * 128;
+            const int kend = gu ? p.H : p.I;
+            int x = 0;
+            for (int kb = 0; kb < t.nkb; ++kb) {
+                if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = 0; break; }
+                if (elect_one()) {
+                    const uint32_t sW = sbase + stage * stage_bytes;
+                    const uint32_t fb = dsmem_addr(full_bar(stage), 0);
+                    if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * kWBytes);
+                    if (!gu) {
+                        tma_load_2d_pair_hint(sW, &maps.down[q], fb, x, y, wpol);
+                    } else if (!two) {
+                        tma_load_3d_pair_hint(sW, &maps.gu[q], fb, x, y, 0, wpol);
+                    } else {
+                        tma_load_2d_pair_hint(sW, &maps.gate[q], fb, x, y, wpol);
+                        tma_load_2d_pair_hint(sW + kWBytes / 2, &maps.up[q], fb, x, y, wpol);
+                    }
+                }
+                x += BK;
+                if (x == kend) { x = 0; y += p.H; }
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
             }
             if (!ok) break;
         }
-        // drain: every copy this thread issued has landed before the CTA exits
-        for (int s = 0; s < kStages; ++s)
-            if ((filled >> s) & 1u) {
-                const unsigned long long t0 = globaltimer_ns();
-                while (!mbar_try_wait(full_bar(s), (last_parity >> s) & 1u))
-                    if (globaltimer_ns() - t0 > kWaitLimitNs) break;
-            }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         int stage = 0, it = 0;
         uint32_t phase = 0;
-        for (int qi = 0;; ++qi) {
-            const int tile = next_tile(qi);
-            if (tile < 0) break;
-            const Tile t = decode_tile(p, tt, G, tile);
-            const uint32_t idesc = p.ph[t.ph].idesc;
+        Tile t;
+        for (int qi = 0; rank == 0 && next_tile(qi, t); ++qi) {
+            const bool gather = t.gather();
+            const uint32_t idesc = p.idesc | ((uint32_t)(t.n() >> 3) << 17);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
             ++it;
-            if (!mbar_wait(tempty_bar(buf), use ^ 1u, &s_abort, p.status)) break;
+            if (!warp_wait(tempty_bar(buf), use ^ 1u)) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * kAccCols);
-            bool ok = true;
+            // The warp's own work per stage must stay below the 512 clocks of
+            // four full MMAs: the next stage's barrier is tested (without
+            // waiting) before this stage's MMAs are issued.
+            int ok = 1;
+            bool ready = false;
             for (int kb = 0; kb < t.nkb; ++kb) {
-                if (!mbar_wait(full_bar(stage), phase, &s_abort, p.status)) { ok = false; break; }
+                if (!__all_sync(~0u, ready || mbar_wait(full_bar(stage), phase, &s_abort, p.status))) { ok = 0; break; }
+                // rows this CTA's gather warps copied (generic proxy, complete
+                // when the barrier's phase completed) are read by the tensor
+                // cores through the async proxy
+                if (gather) fence_proxy_async_smem();
                 tc_fence_after();
-                // rows the gather warps copied (generic proxy, complete when
-                // the barrier's phase completed) are read by the tensor cores
-                // through the async proxy
-                fence_proxy_async_smem();
-                const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
-                const uint64_t ad = sw128_desc(sA), bd = sw128_desc(sB);
+                const uint32_t eb = empty_bar(stage);
+                const uint32_t sW = sbase + stage * stage_bytes;
+                const uint64_t ad = sw128_desc(sW), bd = sw128_desc(sW + kWBytes);
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+                ready = mbar_test_wait(full_bar(stage), phase);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)  // +32 bytes of K per step inside the swizzle row
-                    tc_mma(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0);
-                tc_commit(empty_bar(stage));
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                    for (int k = 0; k < BK / 16; ++k)  // +32 bytes of K per step inside the swizzle row
+                        tc_mma_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0);
+                    tc_commit_pair(eb);
+                    if (kb == t.nkb - 1) tc_commit_pair(tfull_bar(buf));
+                }
+                __syncwarp();
             }
             if (!ok) break;
-            tc_commit(tfull_bar(buf));
         }
-        // every MMA this thread issued has completed before TMEM is freed
-        tc_commit(done_bar);
-        {
+        // the leader's last commit: its MMAs and every commit before (whose
+        // arrivals reach both CTAs) are done before either CTA exits
+        if (elect_one()) {
+            if (rank == 0) tc_commit_pair(done_bar);
             const unsigned long long t0 = globaltimer_ns();
             while (!mbar_try_wait(done_bar, 0))
                 if (globaltimer_ns() - t0 > kWaitLimitNs) break;
@@ -1003,280 +1134,293 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
     } else if (warp >= 2 && warp < 6) {
         // ------------------------------------------------ epilogue
         const int quarter = warp & 3;  // TMEM lanes this warp may access
-        const uint32_t out_base = sbase + kStages * kStageBytes + (uint32_t)((warp - 2) * 2 * kOutBufBytes);
-        int out_parity = 0;
+        const uint32_t stage0 = sbase + kRingBytes;
+        const uint32_t own = stage0 + quarter * kStageOutBytes;            // this warp's two 2 KB buffers
+        const uint32_t partner = stage0 + (quarter ^ 2) * kStageOutBytes;  // those of the warp of the same columns
+        const uint32_t roww = stage0 + 4 * kStageOutBytes + quarter * kRowWBytes;
         int it = 0;
         bool synced = false;  // wait_dispatch has returned (every lane acquires)
         for (int qi = 0;; ++qi) {
-            int tile = 0;
-            if (lane == 0) tile = next_tile(qi);
-            tile = __shfl_sync(~0u, tile, 0);
-            if (tile < 0) break;
-            const Tile t = decode_tile(p, tt, G, tile);
+            Tile t;
+            int ok = next_tile(qi, t);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
             ++it;
-            // one lane waits, the warp follows: tcgen05.ld below is warp-collective
-            int ok = 1;
-            if (lane == 0) ok = mbar_wait(tfull_bar(buf), use, &s_abort, p.status) ? 1 : 0;
-            ok = __shfl_sync(~0u, ok, 0);
-            if (!ok) break;
-            if (!synced && !(synced = wait_dispatch())) break;
-            __syncwarp();
+            if (ok && !synced) ok = synced = __all_sync(~0u, wait_dispatch());
+            if (ok) {
+                if (t.down() && !t.shared()) {  // the rows' routing weights, ahead of the accumulator
+                    float w[kMaxN / 32];
+#pragma unroll
+                    for (int c = 0; c < kMaxN / 32; ++c) {
+                        const int r = c * 32 + lane;
+                        w[c] = r < t.rows ? p.w_of_slot[t.row_base + t.m0 + r] : 0.f;
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < kMaxN / 32; ++c) st_shared_f32(roww + (c * 32 + lane) * 4, w[c]);
+                    __syncwarp();
+                }
+                // one lane waits, the warp follows: tcgen05.ld below is warp-collective
+                if (lane == 0) ok = mbar_wait(tfull_bar(buf), use, &s_abort, p.status) ? 1 : 0;
+                ok = __shfl_sync(~0u, ok, 0);
+            }
+            // the four warps go on together (they meet at barriers inside a tile) or stop together
+            if (!named_barrier_all(3, 128, ok)) break;
             tc_fence_after();
-            const TcPhase &ph = p.ph[t.ph];
-            const bool gu = t.kind == kTileGU;
-            const int r = quarter * 32 + lane;  // tile row of this thread
-            const bool valid = r < t.rows;
-            const int grow = t.row_base + t.m0 + r;
+            const bool gu = !t.down(), shared = t.shared();
+            const TcPhase &ph = p.ph[gu ? kGateUp : kDown];
+            const int nch = t.n() / 32;
+            const int row0 = t.row_base + t.m0;  // slot (shared: token) of the tile's first token row
             const uint32_t taddr = tmem_base + (uint32_t)(buf * kAccCols) + ((uint32_t)(quarter * 32) << 16);
+            // Each chunk of 32 tokens is read as two 16-lane fragments (tmem_frag16):
+            // v[h][4 j + q] is column 16 h + 8 (q / 2) + lane / 4, token
+            // 8 j + 2 (lane & 3) + (q & 1).  stmatrix.trans turns packed pairs of
+            // tokens into rows of columns: half the shared-memory instructions of a
+            // transpose by 32-bit stores from one column per thread.
+            const int srow = lane & 7, scol = lane >> 3;  // stmatrix: this lane's row of matrix scol
             if (gu) {
-                // Whole 32-row blocks go out through shared memory and TMA
-                // stores; the block holding a tile's last rows is written row
-                // by row so that it never touches the next expert's rows.
-                const bool full_block = (t.rows - quarter * 32) >= 32;
-                const int ldc = t.shared ? p.E_sh * p.I : p.I;
-                bf16 *crow = (t.shared ? ph.C_shared : ph.C_routed) + (size_t)grow * ldc + t.n0;
-                const CUtensorMap *cmap = t.shared ? &maps.c_shared[t.ph] : &maps.c_routed[t.ph];
+                const bool first = quarter < 2;  // this warp computes tokens 0-15 of a chunk, its partner 16-31
+                const bool gate = first != (p.up_first[shared ? 2 : (t.g < p.E_pub ? 0 : 1)] != 0);
+                const int col = t.n0 + rank * 64 + (quarter & 1) * 32;  // this warp's columns
+                const int ldc = shared ? p.E_sh * p.I : p.I;
+                bf16 *crow = (shared ? ph.C_shared : ph.C_routed) + (size_t)row0 * ldc + col + (lane & 3) * 8;
+                const int ld2 = 2 * ldc;  // saved G | U: floats per row
+                float *saved = p.saved_gu ? p.saved_gu + (shared ? (size_t)p.R * 2 * p.I : 0) + (size_t)row0 * ld2 +
+                                                (gate ? 0 : ldc) + col + (lane & 7) * 4
+                                          : nullptr;
 #pragma unroll 1
-                for (int c = 0; c < BM / 32; ++c) {
-                    uint32_t pk[16];
-                    float gv[32], uv[32];
-                    tmem_ld32(taddr + c * 32, gv);
-                    tmem_ld32(taddr + 128 + c * 32, uv);
+                for (int c = 0; c < nch; ++c) {
+                    const uint32_t xo = own + (uint32_t)((c & 1) * 2048), xp = partner + (uint32_t)((c & 1) * 2048);
+                    float v[2][16];
+                    tmem_frag16(taddr + c * 32, v[0]);
+                    tmem_frag16(taddr + c * 32 + (16u << 16), v[1]);
                     tmem_ld_wait();
+                    if (saved) {  // the FP32 accumulators for the backward, 16 tokens at a time
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        pk[i] = pack_bf16x2(silu_mul(gv[2 * i], uv[2 * i]), silu_mul(gv[2 * i + 1], uv[2 * i + 1]));
-                    if (p.saved_gu) {
-                        // G and U of these 32 columns, as FP32, for the backward
-                        const int y0 = t.row_base + t.m0 + quarter * 32;
-                        const int ld2 = t.shared ? 2 * p.E_sh * p.I : 2 * p.I;  // floats per saved row
-                        const int uoff = ld2 / 2;                                // U follows G
-                        const CUtensorMap *smap = t.shared ? &maps.gu_save_sh : &maps.gu_save;
-                        if (full_block) {
+                        for (int hh = 0; hh < 2; ++hh) {
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {  // G lo, G hi, U lo, U hi: 16 columns each
-                                const float *src = (b < 2 ? gv : uv) + (b & 1) * 16;
-                                const uint32_t sbuf = out_base + (uint32_t)(out_parity * kOutBufBytes);
-                                if (lane == 0) bulk_wait_read<1>();
-                                __syncwarp();
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) {
-                                    const uint32_t addr = sbuf + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4);
-                                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr),
-                                                 "f"(src[4 * j]), "f"(src[4 * j + 1]), "f"(src[4 * j + 2]),
-                                                 "f"(src[4 * j + 3])
-                                                 : "memory");
-                                }
-                                fence_proxy_async_smem();
-                                __syncwarp();
-                                if (lane == 0) {
-                                    tma_store_2d(smap, sbuf, (b < 2 ? 0 : uoff) + t.n0 + c * 32 + (b & 1) * 16, y0);
-                                    bulk_commit();
-                                }
-                                out_parity ^= 1;
+                            for (int i = 0; i < 16; ++i) {  // h = i / 8, j = 2 hh + (i / 4) % 2, q = i % 4
+                                const int tok = 8 * ((i >> 2) & 1) + 2 * (lane & 3) + (i & 1);
+                                const int cc = 16 * (i >> 3) + 8 * ((i >> 1) & 1) + (lane >> 2);
+                                st_shared_f32(xo + (tok * 32 + (cc ^ ((lane & 3) << 3))) * 4,
+                                              v[i >> 3][8 * hh + (i & 7)]);
                             }
-                        } else if (valid) {
-                            float *sbase = t.shared ? p.saved_gu + (size_t)p.R * 2 * p.I : p.saved_gu;
-                            float4 *gd = reinterpret_cast<float4 *>(sbase + (size_t)grow * ld2 + t.n0 + c * 32);
-                            float4 *ud = gd + uoff / 4;
+                            __syncwarp();
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                gd[i] = make_float4(gv[4 * i], gv[4 * i + 1], gv[4 * i + 2], gv[4 * i + 3]);
-                                ud[i] = make_float4(uv[4 * i], uv[4 * i + 1], uv[4 * i + 2], uv[4 * i + 3]);
+                            for (int j = 0; j < 4; ++j) {
+                                const int r = j * 4 + (lane >> 3), tok = c * 32 + hh * 16 + r;
+                                const uint4 f = ld_shared_v4(xo + r * 128 + ((((lane & 7) * 4) ^ (((r >> 1) & 3) << 3)) * 4));
+                                if (tok < t.rows) *reinterpret_cast<uint4 *>(saved + (size_t)tok * ld2) = f;
                             }
+                            __syncwarp();
                         }
                     }
-                    if (full_block) {
-                        const uint32_t sbuf = out_base + (uint32_t)(out_parity * kOutBufBytes);
-                        if (lane == 0) bulk_wait_read<1>();  // the store that used this buffer has read it
-                        __syncwarp();
-                        // 64-byte rows, 16-byte chunk j of row r at chunk j ^ ((r >> 1) & 3): the
-                        // TMA 64-byte swizzle, and conflict-free for these 16-byte writes
+                    // each warp of the pair gives the other its values of the
+                    // tokens that the other computes
+                    float mine[16], other[16];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint32_t addr = sbuf + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4);
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(pk[4 * j]),
-                                         "r"(pk[4 * j + 1]), "r"(pk[4 * j + 2]), "r"(pk[4 * j + 3])
-                                         : "memory");
-                        }
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) {
-                            tma_store_2d_hint(cmap, sbuf, t.n0 + c * 32, t.row_base + t.m0 + quarter * 32, pol_keep);
-                            bulk_commit();
-                        }
-                        out_parity ^= 1;
-                    } else if (valid) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(crow + c * 32);
+                    for (int i = 0; i < 4; ++i) {
+                        const float *s = &v[i >> 1][(i & 1) * 4];  // tokens 0-15; + 8: tokens 16-31
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                        for (int q = 0; q < 4; ++q) mine[4 * i + q] = first ? s[q] : s[8 + q];
+                        st_shared_v4(xo + i * 512 + lane * 16,
+                                     make_uint4(__float_as_uint(first ? s[8] : s[0]), __float_as_uint(first ? s[9] : s[1]),
+                                                __float_as_uint(first ? s[10] : s[2]), __float_as_uint(first ? s[11] : s[3])));
+                    }
+                    named_barrier_sync(1 + (quarter & 1), 64);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint4 f = ld_shared_v4(xp + i * 512 + lane * 16);
+                        other[4 * i] = __uint_as_float(f.x); other[4 * i + 1] = __uint_as_float(f.y);
+                        other[4 * i + 2] = __uint_as_float(f.z); other[4 * i + 3] = __uint_as_float(f.w);
+                    }
+                    uint32_t pk[8];  // [h][j][q / 2]
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float a0 = silu_mul(gate ? mine[2 * i] : other[2 * i], gate ? other[2 * i] : mine[2 * i]);
+                        const float a1 = silu_mul(gate ? mine[2 * i + 1] : other[2 * i + 1],
+                                                  gate ? other[2 * i + 1] : mine[2 * i + 1]);
+                        pk[i] = pack_bf16x2(a0, a1);
+                    }
+                    __syncwarp();
+                    // transposed through the partner's buffer, which this warp has read
+                    // and the partner fills again only after their next barrier
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int r = 8 * j + srow;
+                        stmatrix_x4_trans(xp + r * 64 + ((scol ^ ((r >> 1) & 3)) << 4), pk[2 * j], pk[2 * j + 1], pk[4 + 2 * j],
+                                          pk[5 + 2 * j]);
+                    }
+                    __syncwarp();
+                    uint4 f[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int r = 8 * h + (lane >> 2);
+                        f[h] = ld_shared_v4(xp + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int tok = c * 32 + (first ? 0 : 16) + 8 * h + (lane >> 2);
+                        if (tok < t.rows) st_global_hint(crow + (size_t)tok * ldc, f[h], pol_keep);
                     }
                 }
             } else {
-                // ---- down: y = w * (act W_down^T), BF16, one row per thread;
-                // whole 32-row blocks through shared memory and TMA stores, a
-                // tile's last partial block row by row
-                const bool full_block = (t.rows - quarter * 32) >= 32;
-                bf16 *crow = (t.shared ? ph.C_shared : ph.C_routed) + (size_t)grow * p.H + t.n0;
-                const CUtensorMap *cmap = t.shared ? &maps.c_shared[t.ph] : &maps.c_routed[t.ph];
-                const float sc = t.shared ? 1.f : (valid ? p.w_of_slot[grow] : 0.f);
+                // ---- down: y = w * (act W_down^T), BF16
+                const int col = t.n0 + rank * 128 + quarter * 32;
+                bf16 *crow = (shared ? ph.C_shared : ph.C_routed) + (size_t)row0 * p.H + col + (lane & 3) * 8;
 #pragma unroll 1
-                for (int c = 0; c < t.bn / 32; ++c) {
-                    uint32_t pk[16];
-                    float v[32];
-                    tmem_ld32(taddr + c * 32, v);
+                for (int c = 0; c < nch && col < p.H; ++c) {  // (a last block's second half may lie past H)
+                    const uint32_t xo = own + (uint32_t)((c & 1) * 2048);
+                    float v[2][16];
+                    tmem_frag16(taddr + c * 32, v[0]);
+                    tmem_frag16(taddr + c * 32 + (16u << 16), v[1]);
+                    float2 w[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        w[j] = shared ? make_float2(1.f, 1.f) : ld_shared_f32x2(roww + (c * 32 + 8 * j + 2 * (lane & 3)) * 4);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(v[2 * i] * sc, v[2 * i + 1] * sc);
-                    if (full_block) {
-                        const uint32_t sbuf = out_base + (uint32_t)(out_parity * kOutBufBytes);
-                        if (lane == 0) bulk_wait_read<1>();  // the store that used this buffer has read it
-                        __syncwarp();
+                    for (int j = 0; j < 4; ++j) {
+                        const int r = 8 * j + srow;
+                        stmatrix_x4_trans(xo + r * 64 + ((scol ^ ((r >> 1) & 3)) << 4),
+                                          pack_bf16x2(v[0][4 * j] * w[j].x, v[0][4 * j + 1] * w[j].y),
+                                          pack_bf16x2(v[0][4 * j + 2] * w[j].x, v[0][4 * j + 3] * w[j].y),
+                                          pack_bf16x2(v[1][4 * j] * w[j].x, v[1][4 * j + 1] * w[j].y),
+                                          pack_bf16x2(v[1][4 * j + 2] * w[j].x, v[1][4 * j + 3] * w[j].y));
+                    }
+                    __syncwarp();
+                    uint4 f[4];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint32_t addr = sbuf + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4);
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(pk[4 * j]),
-                                         "r"(pk[4 * j + 1]), "r"(pk[4 * j + 2]), "r"(pk[4 * j + 3])
-                                         : "memory");
-                        }
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) {
-                            tma_store_2d(cmap, sbuf, t.n0 + c * 32, t.row_base + t.m0 + quarter * 32);
-                            bulk_commit();
-                        }
-                        out_parity ^= 1;
-                    } else if (valid) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(crow + c * 32);
+                    for (int h = 0; h < 4; ++h) {
+                        const int r = 8 * h + (lane >> 2);
+                        f[h] = ld_shared_v4(xo + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
+                    }
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                    for (int h = 0; h < 4; ++h) {
+                        const int tok = c * 32 + 8 * h + (lane >> 2);
+                        if (tok < t.rows) *reinterpret_cast<uint4 *>(crow + (size_t)tok * p.H) = f[h];
                     }
                 }
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(buf));
+            if (lane == 0) {
+                if (rank == 0) mbar_arrive(tempty_bar(buf));
+                else mbar_arrive_remote(dsmem_addr(tempty_bar(buf), 0));
+            }
             // execution audit: rows this tile processed, counted where they
-            // ran.  A row counts for its expert only if its token's route
-            // names this expert (the route log is read back and checked, row
-            // by row); a row that fails the check is a dispatch mismatch.
-            // The per-token private count follows the rows physically run.
-            if (gu) {
-                const unsigned vm = __ballot_sync(~0u, valid);
-                if (!t.shared && t.n0 == 0) {
-                    const int tok = valid ? p.tok_of_slot[grow] : -1;
-                    bool routed = false;
-                    if ((unsigned)tok < (unsigned)p.T) {
-                        const int32_t *ti = p.topk_idx + (size_t)tok * p.k;
-                        for (int j = 0; j < p.k; ++j) routed |= ti[j] == t.g;
+            // ran (by the leader of the pair, which runs them in weight block 0).
+            // A row counts for its expert only if its token's route names this
+            // expert (the route log is read back and checked, row by row); a
+            // row that fails the check is a dispatch mismatch.  The per-token
+            // private count follows the rows physically run.
+            if (gu && rank == 0 && p.status) {
+                if (!shared && t.n0 == 0) {
+                    for (int c = quarter; c < nch; c += 4) {
+                        const bool valid = c * 32 + lane < t.rows;
+                        const int tok = valid ? p.tok_of_slot[row0 + c * 32 + lane] : -1;
+                        bool routed = false;
+                        if ((unsigned)tok < (unsigned)p.T) {
+                            const int32_t *ti = p.topk_idx + (size_t)tok * p.k;
+                            for (int j = 0; j < p.k; ++j) routed |= ti[j] == t.g;
+                        }
+                        if (valid && !routed) atomicOr(p.status, PMPE_STATUS_DISPATCH_MISMATCH);
+                        const unsigned ok_rows = __ballot_sync(~0u, valid && routed);
+                        if (lane == 0 && ok_rows) atomicAdd(&p.exec_rows[t.g], (unsigned)__popc(ok_rows));
+                        if ((unsigned)tok < (unsigned)p.T && t.g >= p.E_pub) atomicAdd(&p.exec_priv_rows[tok], 1u);
                     }
-                    if (valid && !routed && p.status) atomicOr(p.status, PMPE_STATUS_DISPATCH_MISMATCH);
-                    const unsigned ok_rows = __ballot_sync(~0u, valid && routed);
-                    if (lane == 0 && p.exec_rows && ok_rows) atomicAdd(&p.exec_rows[t.g], (unsigned)__popc(ok_rows));
-                    if (lane == 0 && quarter == 0 && p.exec_tiles) atomicAdd(&p.exec_tiles[t.g], 1u);
-                    if ((unsigned)tok < (unsigned)p.T && t.g >= p.E_pub && p.exec_priv_rows)
-                        atomicAdd(&p.exec_priv_rows[tok], 1u);
+                    // 128-row blocks of the expert that start in this row tile
+                    if (lane == 0 && quarter == 0)
+                        atomicAdd(&p.exec_tiles[t.g], (unsigned)((t.m0 + t.rows + kRowBlock - 1) / kRowBlock -
+                                                                 (t.m0 + kRowBlock - 1) / kRowBlock));
                 }
-                if (t.shared && p.shared_rows && lane == 0 && vm && (t.n0 % p.I) == 0)
-                    atomicAdd(p.shared_rows, (unsigned)__popc(vm));
+                if (shared && lane == 0 && quarter == 0 && (t.n0 % p.I) == 0)
+                    atomicAdd(p.shared_rows, (unsigned)t.rows);
             }
             if (gu && p.has_down) {
-                // release this warp's activation rows to the down tiles that
-                // read them: the row stores (generic) and the TMA stores (async
-                // proxy, complete after wait_group 0) are ordered before the count
+                // release this warp's activation columns to the down tiles
+                // that read them (through TMA, after an acquire and a proxy fence)
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) {
-                    bulk_wait_all();
                     asm volatile("fence.proxy.async.global;\n" ::: "memory");
-                    __threadfence();
                     atomicAdd(p.ready + tt.mpre[t.g] + t.m_tile, 1u);
                 }
                 __syncwarp();
             }
         }
-        if (lane == 0) bulk_wait_all();  // this warp's TMA stores are complete before the CTA exits
-    } else if (warp >= 6) {
-        // ------------------------------------------------ A-row gather
-        // Gather: thread i of the 128 copies 16-byte chunk (i & 7) of tile rows
-        // (i >> 3) + 16 j, j = 0..7, every stage, into the 128-byte-swizzled A
-        // slot of the stage (chunk c of row r at chunk c ^ (r & 7)); a warp
-        // instruction covers four whole 128-byte rows.  Rows past the tile's
-        // rows are zero-filled.  Each thread's copies of a stage arrive on the
-        // stage's full barrier when they complete (cp.async.mbarrier.arrive),
-        // so the threads never wait for their own copies: up to the whole ring
-        // is in flight.  The MMA thread fences the async proxy after the
-        // barrier before the tensor cores read the rows.
-        const int gi = tid - 192;            // 0 .. 127
+    } else if (warp >= 6 && warp < kWeightWarp) {
+        // ------------------------------------------------ token row gather
+        // This CTA's half of a routed gate/up tile's token rows: thread i of
+        // a group's 128 copies 16-byte chunk (i & 7) of rows (i >> 3) + 16 j of
+        // the group's stages (every other one: a stage costs a thread about
+        // 600 clocks whatever its rows, more than its MMAs) into the 128-byte-swizzled token slot of the stage (chunk c of
+        // row r at chunk c ^ (r & 7)); a warp instruction covers four whole
+        // 128-byte rows.  Rows past the tile's rows are zero-filled.  Each
+        // thread's copies of a stage arrive on the leader's full barrier, or the
+        // other CTA's gfull barrier, when they complete (cp.async.mbarrier.arrive), so the threads never wait for
+        // their own copies: up to the whole ring is in flight.
+        const int gi = (tid - 192) & 127, group = (warp - 6) >> 2;
         const int chunk = gi & 7, row0 = gi >> 3;
-        uint32_t sc = 0;                     // ring stages passed so far (the ring position)
+        int stage = 0;
+        uint32_t phase = 0;
+        int turn = 0;                        // the group whose stage is next
+        auto gbar = [&](int s) { return rank == 0 ? full_bar(s) : gfull_bar(s); };
         bool ok = true;
         bool synced = false;                 // wait_dispatch has returned (every lane acquires)
-        auto drain = [&]() { cp_async_wait<0>(); };
-        for (int qi = 0; ok; ++qi) {
-            int tile = 0;
-            if (lane == 0) tile = next_tile(qi);
-            tile = __shfl_sync(~0u, tile, 0);
-            if (tile < 0) break;
-            const Tile t = decode_tile(p, tt, G, tile);
-            if (t.kind != kTileGU || t.shared) {  // A comes through TMA: only follow the ring
-                sc += (uint32_t)t.nkb;
-                continue;
-            }
-            if (!synced && !(synced = wait_dispatch())) break;
-            // this thread's 8 rows: their token rows in the hidden states
+        Tile t;
+        for (int qi = 0; ok && next_tile(qi, t); ++qi) {
+            if (!t.gather()) continue;  // rows through TMA; no gathered tile follows one
+            if (!synced && !(synced = __all_sync(~0u, wait_dispatch()))) break;
+            // this thread's rows: their token rows in the hidden states
+            const int nj = t.n() / 32, first = rank * (t.n() / 2);
             const bf16 *src[8];
             uint32_t nbytes[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int r = row0 + 16 * j;
-                const int tok = r < t.rows ? p.tok_of_slot[t.row_base + t.m0 + r] : -1;
+                const int r = first + row0 + 16 * j;
+                const int tok = j < nj && r < t.rows ? p.tok_of_slot[t.row_base + t.m0 + r] : -1;
                 const bool in = (unsigned)tok < (unsigned)p.T;
                 src[j] = p.hidden + (in ? (size_t)tok * p.H : 0) + chunk * 8;
                 nbytes[j] = in ? 16u : 0u;
             }
-            for (int kb = 0; kb < t.nkb; ++kb, ++sc) {
-                const int stage = (int)(sc % kStages);
-                const uint32_t phase = (sc / kStages) & 1u;
-                int free_ = 1;
-                if (lane == 0) free_ = mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status) ? 1 : 0;
-                free_ = __shfl_sync(~0u, free_, 0);
-                if (!free_) { ok = false; break; }
-                const uint32_t sA = sbase + stage * kStageBytes;
+            for (int kb = 0; kb < t.nkb; ++kb) {
+                if (turn == group) {
+                    int free_ = 1;
+                    if (lane == 0) free_ = mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status) ? 1 : 0;
+                    free_ = __shfl_sync(~0u, free_, 0);
+                    if (!free_) { ok = false; break; }
+                    const uint32_t sT = sbase + stage * stage_bytes + kWBytes;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int r = row0 + 16 * j;
-                    cp_async16_zfill(sA + r * 128 + ((chunk ^ (r & 7)) << 4), src[j] + kb * BK, nbytes[j], pol_keep);
+                    for (int j = 0; j < 8; ++j) {
+                        const int r = row0 + 16 * j;
+                        if (j < nj)
+                            cp_async16_zfill(sT + r * 128 + ((chunk ^ (r & 7)) << 4), src[j] + kb * BK, nbytes[j],
+                                             pol_keep);
+                    }
+                    cp_async_arrive_noinc(gbar(stage));
                 }
-                cp_async_arrive_noinc(full_bar(stage));
+                turn = turn == kGatherGroups - 1 ? 0 : turn + 1;
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
             }
         }
-        drain();
+        cp_async_wait<0>();
     }
 
-    // every warp reconverges before the block barrier: __syncthreads is a
-    // warp-aligned barrier, and the single-thread roles above diverge from
-    // their warps; TMEM is freed only after all epilogue reads completed
+    // every warp reconverges before the cluster barrier (a warp-aligned
+    // barrier; the single-thread roles above diverge from their warps): the
+    // pair's MMAs, copies, barrier arrivals and TMEM reads are done
     __syncwarp();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(kTmemCols));
+        tmem_dealloc_pair(tmem_base, kTmemCols);
     }
     if (kRoute && p.fuse_combine) {
         // ---- the weighted combine (Sec. 3.1), as combine_kernel sums it:
-        // j ascending, then the shared experts, in FP32.  Every epilogue
-        // warp's stores are complete (wait_group 0 above); they are made
-        // visible, then every CTA meets at the last grid barrier.
-        if (warp >= 2 && warp < 6 && lane == 0) {
-            asm volatile("fence.proxy.async.global;\n" ::: "memory");
-            __threadfence();
-        }
+        // j ascending, then the shared experts, in FP32, once every CTA has met
+        // at the last grid barrier (whose release covers the epilogues' stores).
         if (grid_barrier(p.bar_d, gridDim.x, &s_abort, p.status)) {
             const bf16 *y = p.ph[kDown].C_routed;
             const bf16 *y_sh = p.E_sh > 0 ? p.ph[kDown].C_shared : nullptr;
@@ -1322,48 +1466,44 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
 
 // ------------------------------------------------------------ host side
 
-// Parameters and tensor maps of one GEMM (`mode`) of a launch.
+// Tensor maps of the token rows at `ptr` [rows, cols], by box rows.
+bool encode_tokens(CUtensorMap *m, const bf16 *ptr, int cols, uint64_t rows)
+{
+    bool ok = true;
+    for (int b = 0; b < kTokBoxes; ++b) ok &= encode_2d(&m[b], ptr, cols, rows, 128u >> b);
+    return ok;
+}
+
+// Outputs and tensor maps of one GEMM (`mode`) of a launch.
 bool fill_phase(const Ctx &c, int mode, TcParams &p, TcMaps &maps)
 {
     const Shape &s = c.s;
     const uint64_t R = (uint64_t)s.T * s.k, T = (uint64_t)s.T;
+    const bool gu = mode == kGateUp;
     bool ok = true;
-    if (mode == kGateUp) {
-        TcPhase &f = p.ph[mode];
-        f.C_routed = c.act;
-        f.C_shared = c.act_sh;
-        ok &= encode_2d_box(&maps.c_routed[mode], c.act, s.I, R, kOutBox, kOutBox, CU_TENSOR_MAP_SWIZZLE_64B);
-        if (s.E_sh > 0)
-            ok &= encode_2d_box(&maps.c_shared[mode], c.act_sh, (uint64_t)s.E_sh * s.I, T, kOutBox, kOutBox,
-                                CU_TENSOR_MAP_SWIZZLE_64B);
-        for (int q = 0; q < 2; ++q) {
-            const uint64_t n = (uint64_t)(q ? s.E_priv : s.E_pub) * s.I;
-            ok &= encode_2d(&maps.b0[mode][q], c.gate[q], s.H, n, 128);
-            ok &= encode_2d(&maps.b1[mode][q], c.up[q], s.H, n, 128);
+    p.ph[mode].C_routed = gu ? c.act : c.y;
+    p.ph[mode].C_shared = gu ? c.act_sh : c.y_sh;
+    for (int q = 0; q < (s.E_sh > 0 ? 3 : 2); ++q) {
+        const uint64_t n = (uint64_t)(q == 0 ? s.E_pub : q == 1 ? s.E_priv : s.E_sh);
+        if (!gu) {
+            ok &= encode_2d(&maps.down[q], c.down[q], s.I, n * s.H, 128);
+            continue;
         }
-        if (s.E_sh > 0) {
-            ok &= encode_2d(&maps.a_shared[mode], c.hidden, s.H, T, BM);
-            ok &= encode_2d(&maps.b0[mode][2], c.gate[2], s.H, (uint64_t)s.E_sh * s.I, 128);
-            ok &= encode_2d(&maps.b1[mode][2], c.up[2], s.H, (uint64_t)s.E_sh * s.I, 128);
-        }
-    } else {
-        const int bn = p.ph[mode].bn;
-        TcPhase &f = p.ph[mode];
-        f.C_routed = c.y;
-        f.C_shared = c.y_sh;
-        ok &= encode_2d_box(&maps.c_routed[mode], c.y, s.H, R, kOutBox, kOutBox, CU_TENSOR_MAP_SWIZZLE_64B);
-        if (s.E_sh > 0)
-            ok &= encode_2d_box(&maps.c_shared[mode], c.y_sh, s.H, T, kOutBox, kOutBox, CU_TENSOR_MAP_SWIZZLE_64B);
-        ok &= encode_2d(&maps.a_routed[mode], c.act, s.I, R, BM);
-        for (int q = 0; q < 2; ++q) {
-            const uint64_t n = (uint64_t)(q ? s.E_priv : s.E_pub) * s.H;
-            ok &= encode_2d(&maps.b0[mode][q], c.down[q], s.I, n, bn / 2);
-        }
-        if (s.E_sh > 0) {
-            ok &= encode_2d(&maps.a_shared[mode], c.act_sh, (uint64_t)s.E_sh * s.I, T, BM);
-            ok &= encode_2d(&maps.b0[mode][2], c.down[2], s.I, (uint64_t)s.E_sh * s.H, bn / 2);
+        p.up_first[q] = c.up[q] < c.gate[q];
+        const bf16 *lo = p.up_first[q] ? c.up[q] : c.gate[q], *hi = p.up_first[q] ? c.gate[q] : c.up[q];
+        const uint64_t apart = (uint64_t)((uintptr_t)hi - (uintptr_t)lo);
+        // a tensor map's strides are below 2^40 bytes (one tensor as both: two boxes)
+        p.gu_two_boxes[q] = apart == 0 || apart >= (1ull << 40) ||
+                            !encode_3d_two(&maps.gu[q], lo, s.H, n * s.I, apart, 64);
+        if (p.gu_two_boxes[q]) {
+            p.up_first[q] = 0;
+            ok &= encode_2d(&maps.gate[q], c.gate[q], s.H, n * s.I, 64);
+            ok &= encode_2d(&maps.up[q], c.up[q], s.H, n * s.I, 64);
         }
     }
+    if (gu && s.E_sh > 0) ok &= encode_tokens(maps.tok[kGateUp], c.hidden, s.H, T);
+    if (!gu) ok &= encode_tokens(maps.tok[kDown], c.act, s.I, R);
+    if (!gu && s.E_sh > 0) ok &= encode_tokens(maps.tok_sh, c.act_sh, s.E_sh * s.I, T);
     return ok;
 }
 
@@ -1374,6 +1514,9 @@ cudaError_t ensure_tc_smem()
     static std::atomic<int> smem_limit[64];
     return ensure_dynamic_smem(expert_gemm_tc_kernel<kRoute>, kDynSmem, smem_limit);
 }
+
+// CTAs of the launch: one pair for every two SMs.
+int tc_grid(const Ctx &c) { return c.num_sms / 2 * 2; }
 
 // One persistent launch of the gate/up tiles, the down tiles, or both (and,
 // with fuse_dispatch, the dispatch before them).
@@ -1388,19 +1531,15 @@ cudaError_t launch_tc(const Ctx &c, bool gu, bool down, bool fuse_dispatch = fal
     p.has_gu = gu;
     p.has_down = down;
     p.E = s.E(); p.E_pub = s.E_pub; p.E_sh = s.E_sh; p.T = s.T; p.H = s.H; p.I = s.I; p.R = s.T * s.k; p.k = s.k;
-    p.ph[kGateUp].bn = 128;
-    p.ph[kGateUp].idesc = make_idesc(BM, 256);
-    p.ph[kDown].bn = column_block(s.H);
-    p.ph[kDown].idesc = make_idesc(BM, p.ph[kDown].bn);
+    p.idesc = make_idesc(256, 0);
     p.offsets = c.offsets;
     p.w_of_slot = c.w_of_slot;
     p.tok_of_slot = c.tok_of_slot;
     p.topk_idx = c.idx;
     p.hidden = c.hidden;
     p.ready = c.gemm_ready;
-    if (gu && s.T <= BM && s.I % 128 == 0 && (long long)s.H * s.I >= (1ll << 20)) {
-        // at most T rows per expert: no expert has a second 128-row block
-        // (small experts, as in the tiny layer: the launch is too short to
+    if (gu && s.T <= kRouteMaxTokens && (long long)s.H * s.I >= (1ll << 20)) {
+        // at most T rows per expert: one row tile each (small experts, as in the tiny layer: the launch is too short to
         // gain from it)
         p.prefetch_tiles = std::min(s.E() * (s.I / 128), kPrefetchTiles);
         for (int q = 0; q < 2; ++q) {
@@ -1471,38 +1610,46 @@ cudaError_t launch_tc(const Ctx &c, bool gu, bool down, bool fuse_dispatch = fal
     bool ok = true;
     if (gu) ok &= fill_phase(c, kGateUp, p, maps);
     if (down) ok &= fill_phase(c, kDown, p, maps);
-    if (c.saved_gu && gu) {
-        p.saved_gu = c.saved_gu;
-        ok &= encode_2d_f32(&maps.gu_save, c.saved_gu, 2 * (uint64_t)s.I, (uint64_t)s.T * s.k, 16, 32,
-                            CU_TENSOR_MAP_SWIZZLE_64B);
-        if (s.E_sh > 0)
-            ok &= encode_2d_f32(&maps.gu_save_sh, c.saved_gu + (size_t)s.T * s.k * 2 * s.I,
-                                2 * (uint64_t)s.E_sh * s.I, (uint64_t)s.T, 16, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    }
+    if (gu) p.saved_gu = c.saved_gu;
     if (!ok) return cudaErrorInvalidValue;
     const cudaError_t err = fuse_route ? ensure_tc_smem<true>() : ensure_tc_smem<false>();
     if (err != cudaSuccess) return err;
     if (fuse_route)
-        return launch_pdl(expert_gemm_tc_kernel<true>, dim3(c.num_sms), dim3(kThreads), kDynSmem, c.stream, p, maps);
-    return launch_pdl(expert_gemm_tc_kernel<false>, dim3(c.num_sms), dim3(kThreads), kDynSmem, c.stream, p, maps);
+        return launch_cluster_pdl(expert_gemm_tc_kernel<true>, 2, dim3(tc_grid(c)), dim3(kThreads), kDynSmem, c.stream, p,
+                                  maps);
+    return launch_cluster_pdl(expert_gemm_tc_kernel<false>, 2, dim3(tc_grid(c)), dim3(kThreads), kDynSmem, c.stream, p,
+                              maps);
 }
 
-// Whether the persistent grid (one CTA per SM) can be resident all at once:
-// the down tiles of the gate/up + down launch wait for gate/up tiles that
-// other CTAs own, so every CTA must run concurrently.  Cached per device.
+// Whether the persistent grid (one CTA per SM, in pairs) can be resident all
+// at once: the down tiles of the gate/up + down launch wait for gate/up tiles
+// that other pairs own, so every pair must run concurrently.  Cached per device.
+template <bool kRoute>
+bool pairs_fit(const Ctx &c)
+{
+    if (ensure_tc_smem<kRoute>() != cudaSuccess) return false;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(tc_grid(c));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kDynSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, expert_gemm_tc_kernel<kRoute>, &cfg) == cudaSuccess && 2 * n >= tc_grid(c);
+}
+
 static bool grid_fits(const Ctx &c)
 {
     static std::atomic<int> fits[64];  // 0 unknown, 1 yes, 2 no
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     if (dev >= 0 && dev < 64 && fits[dev].load() != 0) return fits[dev].load() == 1;
-    int per_sm = 0, per_sm_r = 0;
-    const bool ok = ensure_tc_smem<false>() == cudaSuccess && ensure_tc_smem<true>() == cudaSuccess &&
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expert_gemm_tc_kernel<false>, kThreads,
-                                                                  kDynSmem) == cudaSuccess &&
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_r, expert_gemm_tc_kernel<true>, kThreads,
-                                                                  kDynSmem) == cudaSuccess &&
-                    per_sm >= 1 && per_sm_r >= 1;
+    const bool ok = pairs_fit<false>(c) && pairs_fit<true>(c);
     if (dev >= 0 && dev < 64) fits[dev].store(ok ? 1 : 2);
     return ok;
 }
@@ -1531,7 +1678,7 @@ cudaError_t launch_down(const Ctx &c)
 bool experts_fuse_dispatch(const Ctx &c)
 {
     return (long long)c.s.H * c.s.I >= (1ll << 20) && grid_fits(c) &&
-           fused_dispatch_smem(c.s.E(), router_slots(c.s.T)) <= (size_t)(kStages * kStageBytes);
+           fused_dispatch_smem(c.s.E(), router_slots(c.s.T)) <= (size_t)kRingBytes;
 }
 
 // Routing in the expert launch: at most 128 tokens (one selection CTA each,
@@ -1543,8 +1690,8 @@ bool experts_fuse_dispatch(const Ctx &c)
 bool experts_fuse_route(const Ctx &c)
 {
     const Shape &s = c.s;
-    return s.T >= 1 && s.T <= kRouteMaxTokens && s.T <= c.num_sms && !c.unmasked && s.H <= kRouteMaxH &&
-           s.E_pub <= 256 && s.E_priv <= 256 && (size_t)s.E() * 24u <= (size_t)(kStages * kStageBytes) &&
+    return s.T >= 1 && s.T <= kRouteMaxTokens && s.T <= tc_grid(c) && !c.unmasked && s.H <= kRouteMaxH &&
+           s.E_pub <= 256 && s.E_priv <= 256 && (size_t)s.E() * 24u <= (size_t)kRingBytes &&
            grid_fits(c);
 }
 
@@ -1616,6 +1763,19 @@ bool encode_3d_blocks(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t r
     const cuuint64_t dims[3] = {64, rows, cols / 64};
     const cuuint64_t strides[2] = {cols * 2, 128};  // row pitch; 64-column blocks 128 bytes apart
     const cuuint32_t box[3] = {64, box_rows, nblocks};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool encode_3d_two(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows, uint64_t apart, uint32_t box_rows)
+{
+    auto fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {cols, rows, 2};
+    const cuuint64_t strides[2] = {cols * 2, apart};
+    const cuuint32_t box[3] = {64, box_rows, 2};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

@@ -74,8 +74,6 @@ int router_slots4(int T);
 // Readiness counters of the persistent expert GEMMs: one per (group, 128-row
 // block), an upper bound over all routings.
 size_t gemm_ready_words(const Shape &s);
-// Output columns per down tile: 256 when H allows, else 128.
-int column_block(int H);
 
 // Launchers (one per stage); each returns the launch's cudaError_t.
 // The router; with write_dispatch (only where route_writes_dispatch holds)

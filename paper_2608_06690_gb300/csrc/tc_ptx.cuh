@@ -1,5 +1,5 @@
 // Device-side wrappers of the Blackwell (sm_100 family) PTX this library
-// uses: mbarriers with bounded waits, TMA tile and gather4 loads, tcgen05 MMA,
+// uses: mbarriers with bounded waits, TMA tile loads, tcgen05 MMA,
 // commit, TMEM allocation and loads, and the shared-memory / instruction
 // descriptors.  Host-side tensor-map encoding is declared at the end.
 #pragma once
@@ -41,6 +41,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// The phase's state now, without waiting.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ unsigned long long globaltimer_ns()
 {
     unsigned long long t;
@@ -52,15 +63,24 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
 // (kWaitLimitNs for the layer's kernels) or until another role raised the
 // abort flag.  On expiry it raises the abort flag, records
 // PMPE_STATUS_PIPELINE_TIMEOUT and returns false.
+// The global timer is read only after kWaitTries failed tries: one read takes
+// about 350 clocks, and a wait that read it whenever its first try failed cost
+// every stage of every pipeline role one or two reads, 1,100 to 1,240 clocks a
+// stage in the thread that issues the MMAs whatever the tile's size.
+constexpr int kWaitTries = 32;
 __device__ __noinline__ static bool mbar_wait_for(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                                   uint32_t *status, unsigned long long limit_ns)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer_ns();
+    unsigned long long t0 = 0;
     for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
+        for (int i = 0; i < kWaitTries; ++i)
+            if (mbar_try_wait(bar, parity)) return true;
         if (*abort_flag) return false;
-        if (globaltimer_ns() - t0 > limit_ns) {
+        const unsigned long long now = globaltimer_ns();
+        if (t0 == 0) {
+            t0 = now;
+        } else if (now - t0 > limit_ns) {
             *abort_flag = 1;
             if (status) atomicOr(status, PMPE_STATUS_PIPELINE_TIMEOUT);
             return false;
@@ -70,7 +90,76 @@ __device__ __noinline__ static bool mbar_wait_for(uint32_t bar, uint32_t parity,
 __device__ __forceinline__ static bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                                  uint32_t *status)
 {
+    if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_for(bar, parity, abort_flag, status, kWaitLimitNs);
+}
+
+// Whether this is the elected lane of a converged warp (the same lane every
+// time).  Tested directly before TMA and tcgen05 instructions, in a loop that
+// the whole warp runs: with the loop inside the elected branch, or the result
+// kept in a variable, the operands' broadcasts made a stage of four MMAs and a
+// commit cost about 390 clocks instead of 60 to 190.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t pred;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(pred));
+    return pred != 0;
+}
+
+// Named CTA barriers of `threads` threads (whole warps): a plain one, and one
+// that tells every thread whether all of them passed `pred`.
+__device__ __forceinline__ void named_barrier_sync(int id, int threads)
+{
+    asm volatile("barrier.cta.sync.aligned %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ bool named_barrier_all(int id, int threads, int pred)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %3, 0;\n barrier.cta.red.and.aligned.pred q, %1, %2, p;\n selp.u32 %0, 1, "
+        "0, q;\n}\n"
+        : "=r"(r)
+        : "r"(id), "r"(threads), "r"(pred)
+        : "memory");
+    return r != 0;
+}
+
+// Shared-memory accesses by 32-bit shared address.
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, float v)
+{
+    asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, const uint4 &v)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ float2 ld_shared_f32x2(uint32_t addr)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+// Four 8 x 8 BF16 matrices in the mma fragment layout (thread i: row i / 4,
+// columns 2 (i & 3), + 1), each stored transposed: thread 8 m + r gives the
+// address of the 16-byte row r of (transposed) matrix m.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(a), "r"(b),
+                 "r"(c), "r"(d)
+                 : "memory");
+}
+// 16 bytes to global memory with an L2 cache policy.
+__device__ __forceinline__ void st_global_hint(void *ptr, const uint4 &v, uint64_t policy)
+{
+    asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;\n" ::"l"(ptr), "r"(v.x), "r"(v.y), "r"(v.z),
+                 "r"(v.w), "l"(policy)
+                 : "memory");
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y)
@@ -100,22 +189,17 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first()
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(p));
     return p;
 }
+__device__ __forceinline__ uint64_t l2_policy_evict_normal()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;\n" : "=l"(p));
+    return p;
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_last()
 {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;\n" : "=l"(p));
     return p;
-}
-
-// tma_load_2d with an L2 cache policy.
-__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y,
-                                                 uint64_t policy)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, "
-        "%4}], [%2], %5;\n" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "l"(policy)
-        : "memory");
 }
 
 // Untiled bulk copy of `bytes` (a multiple of 16; both addresses 16-byte
@@ -200,23 +284,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+// 16 TMEM lanes x 32 FP32 columns in the mma fragment layout: v[4 j + q] is
+// lane 8 (q / 2) + i / 4 (of the 16 from taddr's lane), column 8 j + 2 (i & 3) + (q & 1).
+__device__ __forceinline__ void tmem_frag16(uint32_t taddr, float *v)
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 
-
-// TMA gather4: four rows (y0..y3) of a 2-D tensor, `box width` columns from
-// x, into four consecutive 128-byte rows of shared memory (box height 1).
-__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y0, int y1,
-                                            int y2, int y3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
-        "%4, %5, %6, %7}], [%2];\n" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3)
-        : "memory");
-}
-
-// Make this thread's completed generic-proxy shared-memory writes (e.g. from
-// cp.async) visible to the async proxy that tcgen05.mma reads through.
 // Prefetch [ptr, ptr + bytes) into L2 (16-byte aligned, a multiple of 16 bytes).
 __device__ __forceinline__ void bulk_prefetch_l2(const void *ptr, uint32_t bytes)
 {
@@ -229,6 +311,8 @@ __device__ __forceinline__ void prefetch_tmap(const void *map)
 {
     asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
+// Make this thread's completed generic-proxy shared-memory writes (e.g. from
+// cp.async) visible to the async proxy that tcgen05.mma reads through.
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t slot_smem_addr, uint32_t ncols)
@@ -290,6 +374,38 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+// The same for a 2-D box with an L2 cache policy.
+__device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y,
+                                                      uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
+        "[%1, {%3, %4}], [%2], %5;\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "l"(policy)
+        : "memory");
+}
+// 32 bytes into another CTA's shared memory, handed over on that CTA's barrier
+// `remote_bar` (addresses from dsmem_addr): one arrival and the bytes' transaction.
+__device__ __forceinline__ void st_async_32(uint32_t remote_addr, const uint4 &x, const uint4 &y, uint32_t remote_bar)
+{
+    asm volatile(
+        "mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%1], 32;\n"
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.u32 [%0], {%2, %3, %4, %5}, [%1];\n"
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.u32 [%0 + 16], {%6, %7, %8, %9}, [%1];\n" ::"r"(remote_addr),
+        "r"(remote_bar), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(y.x), "r"(y.y), "r"(y.z), "r"(y.w)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d_pair_hint(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y,
+                                                      int z, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
+        "[%1, {%3, %4, %5}], [%2], %6;\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(policy)
+        : "memory");
+}
+
 // One warp of each CTA of the pair executes the allocation and the release.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem_addr, uint32_t ncols)
 {
@@ -330,14 +446,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t sr
                  "r"(src), "r"(x), "r"(y)
                  : "memory");
 }
-// tma_store_2d with an L2 cache policy.
-__device__ __forceinline__ void tma_store_2d_hint(const CUtensorMap *map, uint32_t src, int x, int y, uint64_t policy)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3}], [%1], %4;\n" ::"l"(
-                     reinterpret_cast<uint64_t>(map)),
-                 "r"(src), "r"(x), "r"(y), "l"(policy)
-                 : "memory");
-}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 // Wait until at most N committed bulk groups still read their shared-memory source.
 template <int N>
@@ -370,6 +478,10 @@ bool encode_2d_f32(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows
 // [box_rows][64] tiles one after another (the layout of an MN-major operand
 // whose MN blocks are box_rows * 128 bytes apart).
 bool encode_3d_blocks(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows, uint32_t box_rows, uint32_t nblocks);
+// 3-D BF16 tensor map over two row-major [rows, cols] matrices `apart` bytes
+// apart (the first at ptr): a box of 64 columns x box_rows rows of both, one
+// after the other, 128-byte swizzle.
+bool encode_3d_two(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows, uint64_t apart, uint32_t box_rows);
 // tcgen05 instruction descriptor: BF16 x BF16 -> FP32, both operands K-major.
 uint32_t make_idesc(int M, int N);
 // The same with either operand MN-major (transpose bits 15 for A, 16 for B).

@@ -1,0 +1,48 @@
+"""The expert GEMMs' row tiles (N of 32 to 256 tokens, tiles of equal size per
+expert) at the edges of their sizes, for a hidden size whose last 256-row weight
+block is half empty, and the ways the gate and up tensors can lie in memory."""
+import pytest
+import torch
+
+from paper_2608_06690_gb300.inputs import LayerShape
+from pmpe_testlib import check_against_oracle, check_audit, check_dispatch, make_layer, run_gpu_layer, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T", [1, 32, 33, 97, 224, 225, 256, 257, 289, 513, 800])
+@pytest.mark.parametrize("H, E_sh", [(256, 0), (384, 2)])
+def test_rows_of_one_expert(T, H, E_sh):
+    """k = 1 and one expert a pool: expert 0 gets every DENY token (all but
+    three), so its tiles split T - 3 rows, and the shared group's T."""
+    shape = LayerShape(T=T, H=H, I=128, E_pub=1, E_priv=1, E_sh=E_sh, k=1, renormalize=True)
+    w, h, _ = make_layer(shape, 60 + T)
+    pol = torch.zeros(T, dtype=torch.uint8)
+    pol[T // 2:T // 2 + 3] = 1
+    gpu = run_gpu_layer(shape, *to_device(w, h, pol))
+    check_against_oracle(shape, w, h, pol, gpu)
+    check_audit(shape, pol, gpu)
+    check_dispatch(shape, h, gpu)
+
+
+@pytest.mark.parametrize("layout", ["up_first", "same"])
+@pytest.mark.parametrize("T", [40, 300])
+def test_gate_and_up_tensors(layout, T):
+    """The gate and up rows come as one box of both tensors: the up tensor
+    below the gate tensor in memory, and one tensor as both (two boxes)."""
+    shape = LayerShape(T=T, H=256, I=256, E_pub=6, E_priv=4, E_sh=1, k=2, renormalize=True)
+    w, h, pol = make_layer(shape, 71)
+    for n in ("pub", "priv", "sh"):
+        if layout == "same":
+            w["up_" + n] = w["gate_" + n]
+    wd, hd, pd = to_device(w, h, pol)
+    for n in ("pub", "priv", "sh"):
+        if layout == "same":
+            wd["up_" + n] = wd["gate_" + n]
+        else:
+            both = torch.stack([wd["up_" + n], wd["gate_" + n]]).contiguous()
+            wd["up_" + n], wd["gate_" + n] = both[0], both[1]
+            assert wd["up_" + n].data_ptr() < wd["gate_" + n].data_ptr()
+    gpu = run_gpu_layer(shape, wd, hd, pd)
+    check_against_oracle(shape, w, h, pol, gpu)
+    check_audit(shape, pol, gpu)
