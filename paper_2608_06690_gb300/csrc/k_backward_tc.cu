@@ -28,9 +28,10 @@
 //
 // Every launch keeps four 48 KB operand stages in flight (a 128 x 256 x 64 MMA
 // block each) and two 128 x 256 FP32 accumulators, so the epilogue of one tile
-// overlaps the MMAs of the next.  CTA roles (192 threads), as in the forward:
-// warp 0 lanes 0-2 issue TMA loads, warp 1 allocates TMEM and one thread
-// issues the MMAs, warps 2-5 drain TMEM (one tile row per thread).  Every wait
+// overlaps the MMAs of the next.  CTA roles (224 threads): warps 0 and 6 issue
+// the TMA loads of the first and the second operand, warp 1 allocates TMEM and
+// issues the MMAs, warps 2-5 drain TMEM (one tile row per thread).  Warps 0, 1
+// and 6 run their loops as whole warps, with one elected lane issuing (elect_one).  Every wait
 // is bounded in time; on expiry the CTA records PMPE_STATUS_PIPELINE_TIMEOUT,
 // stops, waits (bounded) for its copies and MMAs in flight, frees TMEM and exits.
 #include <cuda.h>
@@ -50,8 +51,8 @@ constexpr int kABytes = BM * BK * 2;           // 16 KB
 constexpr int kBBytes = 256 * BK * 2;          // 32 KB
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kMnBlockBytes = 64 * BK * 2;     // one 64-element MN block of an MN-major operand: 8 KB
-constexpr int kThreads = 192;
-constexpr int kLoaders = 3;
+constexpr int kThreads = 224;
+constexpr int kLoaders = 2;                    // loader warps 0 and 6: one operand each
 constexpr int kPad = 128;                      // padded row layout: each expert starts at a multiple of 128
 
 // Four operand stages; outputs staged per epilogue warp in two 2 KB boxes of
@@ -154,15 +155,16 @@ struct OutStager {
     }
 };
 
-// Bounded wait for the drain at exit: every copy a loader issued has landed.
-__device__ __forceinline__ void drain_stages(uint32_t bar0, int stages, uint32_t filled, uint32_t last_parity)
+// Bounded wait for the drain at exit: every copy a loader issued has landed
+// (the last use of each stage, after `issued` stages up to `stage` in `phase`).
+__device__ __forceinline__ void drain_stages(uint32_t bar0, int stages, int issued, int stage, uint32_t phase)
 {
-    for (int s = 0; s < stages; ++s)
-        if ((filled >> s) & 1u) {
-            const unsigned long long t0 = globaltimer_ns();
-            while (!mbar_try_wait(bar0 + 8u * s, (last_parity >> s) & 1u))
-                if (globaltimer_ns() - t0 > kWaitLimitNs) break;
-        }
+    for (int s = 0; s < stages && issued > 0; ++s) {
+        if (issued < stages && s >= stage) break;
+        const unsigned long long t0 = globaltimer_ns();
+        while (!mbar_try_wait(bar0 + 8u * s, s < stage ? phase : phase ^ 1u))
+            if (globaltimer_ns() - t0 > kWaitLimitNs) break;
+    }
 }
 
 // ------------------------------------------------------------- rows
@@ -195,7 +197,7 @@ struct RowsParams {
 struct RowsMaps {
     CUtensorMap a;           // A rows, 64 x 128 box (K-major)
     CUtensorMap b0[2], b1[2];  // per weight pool (public, private; shared groups use [0]): MN mode:
-                             // 64 x 64 x bn/128 3-D boxes (MN-major); gate/up: gate, up, 64 x 128 (K-major)
+                             // 64 x 64 x bn/64 3-D boxes (MN-major); gate/up: gate, up, 64 x 128 (K-major)
     CUtensorMap out0;        // MN: C [RP][N]; gate/up: [dG | dU] [RP][2I]  (32 x 32 BF16 boxes, 64-byte swizzle)
     CUtensorMap out1;        // gate/up: w act [RP][I]
 };
@@ -204,14 +206,9 @@ struct RowsTile {
     int q, m0, n0, n_tile, rows;
 };
 
-__device__ __forceinline__ RowsTile decode_rows(const GroupTable &gt, int G, int nt, int bn, int tile, int reverse)
+// Tile `tile` of the list, given its group lo.
+__device__ __forceinline__ RowsTile rows_tile(const GroupTable &gt, int lo, int bn, int tile)
 {
-    if (reverse) tile = gt.tiles[G] - 1 - tile;
-    int lo = 0, hi = G - 1;  // last group whose tile prefix is <= tile (skips empty groups)
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (gt.tiles[mid] <= tile) lo = mid; else hi = mid - 1;
-    }
     RowsTile t;
     t.q = lo;
     const int mt = (gt.rows[lo] + BM - 1) / BM;
@@ -222,6 +219,28 @@ __device__ __forceinline__ RowsTile decode_rows(const GroupTable &gt, int G, int
     t.n0 = t.n_tile * bn;
     t.rows = min(BM, gt.rows[lo] - t.m0);
     return t;
+}
+
+// By a whole warp: the group is the last one whose tile prefix is <= tile
+// (empty groups are passed).
+__device__ __forceinline__ RowsTile decode_rows(const GroupTable &gt, int G, int bn, int tile, int reverse)
+{
+    const int lane = threadIdx.x & 31;
+    if (reverse) tile = gt.tiles[G] - 1 - tile;
+    int n = 0;
+    for (int b = 0; b < G; b += 32) n += __popc(__ballot_sync(~0u, b + lane < G && gt.tiles[b + lane] <= tile));
+    return rows_tile(gt, n - 1, bn, tile);
+}
+
+// By one thread (fewer instructions where every warp of a CTA decodes).
+__device__ __forceinline__ RowsTile decode_rows_thread(const GroupTable &gt, int G, int bn, int tile)
+{
+    int lo = 0, hi = G - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (gt.tiles[mid] <= tile) lo = mid; else hi = mid - 1;
+    }
+    return rows_tile(gt, lo, bn, tile);
 }
 
 // Weight pool (0 public or shared, 1 private) and index inside it of group q.
@@ -273,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(~0u, tid >> 5, 0), lane = tid & 31;
     const uint32_t sbase = (smem_u32(dsmem) + 1023u) & ~1023u;
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -301,88 +320,102 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
     const int nkb = p.K / BK;
     const int p0 = p.shared_T ? 0 : (int)min(p.offsets[p.g0], (uint32_t)p.R);
 
-    if (warp == 0 && lane < kLoaders) {
+    // A barrier wait by a whole warp: every lane waits, and the vote keeps the
+    // warp together and gives one answer.
+    auto warp_wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        return __all_sync(~0u, mbar_wait(bar, parity, &s_abort, p.status));
+    };
+
+    if (warp == 0 || warp == 6) {
         // ------------------------------------------------ TMA producers
-        // lane 0: the tile's 128 rows x 64 K of A (16 KB).  Gate/up: lane 1 the
-        // 128 gate rows, lane 2 the 128 up rows (16 KB each).  MN mode: lanes 1-2
-        // half of the bn / 64 MN blocks of B each, as one 3-D box (8 KB per block).
-        int stage = 0;
-        uint32_t phase = 0, filled = 0, last_parity = 0;
-        const int half = p.bn / 128;  // MN mode: MN blocks per loader lane
-        for (int tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x) {
-            const RowsTile t = decode_rows(gt, p.G, nt, p.bn, tile, p.reverse);
+        // warp 0: the tile's 128 rows x 64 K of A (16 KB).  Warp 6, gate/up: the
+        // 128 gate and the 128 up rows (16 KB each); MN mode: the bn / 64 MN
+        // blocks of B as one 3-D box (8 KB per block).
+        int stage = 0, issued = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+            const RowsTile t = decode_rows(gt, p.G, p.bn, tile, p.reverse);
             const int2 wq = group_weights(p, t.q);
             const int arow = (p.a_rows == kArowsPad ? gt.pad[t.q] : (p.a_rows == kArowsSlot ? p0 : 0) + gt.off[t.q]) + t.m0;
-            bool ok = true;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status)) { ok = false; break; }
+                if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = false; break; }
                 const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
                 const int kx = kb * BK;
-                if (lane == 0) {
-                    mbar_expect_tx(full_bar(stage), kABytes);
-                    tma_load_2d(sA, &maps.a, full_bar(stage), kx, arow);
+                if (warp == 0) {
+                    if (elect_one()) {
+                        mbar_expect_tx(full_bar(stage), kABytes);
+                        tma_load_2d(sA, &maps.a, full_bar(stage), kx, arow);
+                    }
                 } else if (kMode == kRowsGU) {
-                    mbar_expect_tx(full_bar(stage), kABytes);
-                    tma_load_2d(sB + (lane - 1) * kABytes, lane == 1 ? &maps.b0[wq.x] : &maps.b1[wq.x], full_bar(stage),
-                                kx, wq.y * p.I + t.n0);
+                    if (elect_one()) {
+                        mbar_expect_tx(full_bar(stage), 2 * kABytes);
+                        tma_load_2d(sB, &maps.b0[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
+                        tma_load_2d(sB + kABytes, &maps.b1[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
+                    }
                 } else {
-                    const int b0 = (lane - 1) * half;
                     const bool second = kb >= p.k_split;
                     const int krow = wq.y * p.kb_rows + (second ? kx - p.k_split * BK : kx);
-                    mbar_expect_tx(full_bar(stage), (uint32_t)(half * kMnBlockBytes));
-                    tma_load_3d(sB + b0 * kMnBlockBytes, second ? &maps.b1[wq.x] : &maps.b0[wq.x], full_bar(stage), 0,
-                                krow, t.n0 / 64 + b0);
+                    if (elect_one()) {
+                        mbar_expect_tx(full_bar(stage), (uint32_t)(p.bn / 64 * kMnBlockBytes));
+                        tma_load_3d(sB, second ? &maps.b1[wq.x] : &maps.b0[wq.x], full_bar(stage), 0, krow, t.n0 / 64);
+                    }
                 }
-                filled |= 1u << stage;
-                last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
+                ++issued;
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) break;
         }
-        drain_stages(bar0, kStages, filled, last_parity);
-    } else if (warp == 1 && lane == 0) {
+        drain_stages(bar0, kStages, issued, stage, phase);
+    } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         // gate/up: one N = 256 MMA over the gate and up rows, G in accumulator
         // columns [0, 128) and U in [128, 256); Z: N = bn, W_down MN-major.
         int stage = 0, it = 0;
         uint32_t phase = 0;
-        for (int tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x, ++it) {
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, ++it) {
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
-            if (!mbar_wait(tempty_bar(buf), use ^ 1u, &s_abort, p.status)) break;
+            if (!warp_wait(tempty_bar(buf), use ^ 1u)) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * kAccCols);
-            bool ok = true;
+            bool ready = false;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(full_bar(stage), phase, &s_abort, p.status)) { ok = false; break; }
+                if (!__all_sync(~0u, ready || mbar_wait(full_bar(stage), phase, &s_abort, p.status))) { ok = false; break; }
                 tc_fence_after();
+                const uint32_t eb = empty_bar(stage);
                 const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
                 const uint64_t ad = sw128_desc(sA);
-#pragma unroll
-                for (int k = 0; k < BK / 16; ++k) {
-                    // K-major: +32 bytes of K per step inside the swizzle row;
-                    // MN-major: 16 K rows = 2048 bytes per step
-                    const uint64_t bd = kMode == kRowsGU ? sw128_desc(sB) + 2 * k
-                                                         : mn_sw128_desc(sB + k * 2048, kMnBlockBytes);
-                    tc_mma(d_tmem, ad + 2 * k, bd, p.idesc, (kb | k) != 0);
-                }
-                tc_commit(empty_bar(stage));
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                ready = mbar_test_wait(full_bar(stage), phase);
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k) {
+                        // K-major: +32 bytes of K per step inside the swizzle row;
+                        // MN-major: 16 K rows = 2048 bytes per step
+                        const uint64_t bd = kMode == kRowsGU ? sw128_desc(sB) + 2 * k
+                                                             : mn_sw128_desc(sB + k * 2048, kMnBlockBytes);
+                        tc_mma(d_tmem, ad + 2 * k, bd, p.idesc, (kb | k) != 0);
+                    }
+                    tc_commit(eb);
+                    if (kb == nkb - 1) tc_commit(tfull_bar(buf));
+                }
+                __syncwarp();
             }
-            if (!ok) break;
-            tc_commit(tfull_bar(buf));
         }
-        tc_commit(done_bar);
-        const unsigned long long t0 = globaltimer_ns();
-        while (!mbar_try_wait(done_bar, 0))
-            if (globaltimer_ns() - t0 > kWaitLimitNs) break;
-    } else if (warp >= 2) {
+        if (elect_one()) {
+            tc_commit(done_bar);
+            const unsigned long long t0 = globaltimer_ns();
+            while (!mbar_try_wait(done_bar, 0))
+                if (globaltimer_ns() - t0 > kWaitLimitNs) break;
+        }
+    } else {
         // ------------------------------------------------ epilogue
         const int quarter = warp & 3;
         OutStager out{sbase + kStages * kStageBytes + (uint32_t)((warp - 2) * kOutBufs * kOutBoxBytes), 0};
         int it = 0;
         for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++it) {
-            const RowsTile t = decode_rows(gt, p.G, nt, p.bn, tile, p.reverse);
+            const RowsTile t = decode_rows(gt, p.G, p.bn, tile, p.reverse);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
             int ok = 1;
@@ -488,7 +521,7 @@ __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams 
     const float *sbase = p.shared_T ? saved_gu + (size_t)p.R * 2 * p.I : saved_gu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-        const RowsTile t = decode_rows(gt, p.G, nt, 128, tile, 0);
+        const RowsTile t = decode_rows_thread(gt, p.G, 128, tile);
         const bool wa_out = p.wact && !p.shared_T && p.g0 + t.q >= p.E_pub;
         const int gcol = p.shared_T ? t.q * p.I : 0;  // the group's G columns in its saved row
         for (int r = warp; r < BM; r += nwarps) {
@@ -558,7 +591,7 @@ __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams 
 // us against single-CTA 128 x 256 tiles.
 constexpr int kWgStages = 5;
 constexpr int kWgStageBytes = 2 * kABytes;
-constexpr int kWgLoaders = 2;
+constexpr int kWgLoaders = 2;               // loader warps 0 and 6
 constexpr int kWgOutBufs = 3;              // per epilogue warp, boxes of 32 rows x 32 FP32 columns
 constexpr int kWgOutBoxBytes = 32 * 128;
 constexpr int kWgDynSmem = kWgStages * kWgStageBytes + 4 * kWgOutBufs * kWgOutBoxBytes + 1024;
@@ -632,7 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(~0u, tid >> 5, 0), lane = tid & 31;
     const int rank = (int)cluster_ctarank();  // 0: the leader, whose thread issues the pair's MMAs
     const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const uint32_t sbase = (smem_u32(dsmem) + 1023u) & ~1023u;
@@ -662,76 +695,88 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
     const int total = wg_total(p);
     const int p0 = (int)min(p.offsets[p.g0], (uint32_t)p.R);
 
-    if (warp == 0 && lane < kWgLoaders) {
+    auto warp_wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        return __all_sync(~0u, mbar_wait(bar, parity, &s_abort, p.status));
+    };
+
+    if (warp == 0 || warp == 6) {
         // ------------------------------------------------ TMA producers
-        // lane 0: this CTA's two 64-element MN blocks of A; lane 1: its half of
-        // B's bn / 64 blocks; one 3-D box per lane (64 MN elements x 64 rows of
+        // warp 0: this CTA's two 64-element MN blocks of A; warp 6: its half of
+        // B's bn / 64 blocks; one 3-D box each (64 MN elements x 64 rows of
         // K per block).  Every copy completes on the leader's barrier, where
-        // the leader's lanes announce both CTAs' bytes.
-        int stage = 0;
-        uint32_t phase = 0, filled = 0, last_parity = 0;
-        for (int tile = pair; tile < total && !s_abort; tile += pairs) {
+        // the leader's warps announce both CTAs' bytes.
+        int stage = 0, issued = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = pair; tile < total && ok; tile += pairs) {
             const WgTile t = decode_wg(p, gt, tile);
             const int half = t.bn / 128;  // MN blocks of B per CTA
             const int gq = t.q + p.q_off;  // the expert's entry in the group table
             const int rowA = t.prob == 0 ? gt.pad[gq] : gt.off[gq];
             const int rowB = t.prob == 0 ? p0 + gt.off[gq] : gt.pad[gq];
-            const CUtensorMap *amap = t.prob == 0 ? &maps.dgu : &maps.dout_rows;
-            const CUtensorMap *bmap = t.prob == 0 ? &maps.a_perm[2 - half] : &maps.wact[2 - half];
-            bool ok = true;
+            const CUtensorMap *map = warp == 0 ? (t.prob == 0 ? &maps.dgu : &maps.dout_rows)
+                                               : (t.prob == 0 ? &maps.a_perm[2 - half] : &maps.wact[2 - half]);
+            const int row = warp == 0 ? rowA : rowB;
+            const int block = warp == 0 ? t.m0 / 64 + 2 * rank : t.n0 / 64 + half * rank;
+            const uint32_t bytes = 2u * (warp == 0 ? (uint32_t)kABytes : (uint32_t)(half * kMnBlockBytes));
             for (int kb = 0; kb < t.nkb; ++kb) {
-                if (!mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status)) { ok = false; break; }
-                const uint32_t sA = sbase + stage * kWgStageBytes, sB = sA + kABytes;
-                const uint32_t fb = dsmem_addr(full_bar(stage), 0);
-                const int ky = kb * BK;
-                if (rank == 0)
-                    mbar_expect_tx(full_bar(stage), 2u * (lane == 0 ? (uint32_t)kABytes : (uint32_t)(half * kMnBlockBytes)));
-                if (lane == 0) tma_load_3d_pair(sA, amap, fb, 0, rowA + ky, t.m0 / 64 + 2 * rank);
-                else tma_load_3d_pair(sB, bmap, fb, 0, rowB + ky, t.n0 / 64 + half * rank);
-                filled |= 1u << stage;
-                last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
+                if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = false; break; }
+                if (elect_one()) {
+                    const uint32_t dst = sbase + stage * kWgStageBytes + (warp == 0 ? 0 : kABytes);
+                    const uint32_t fb = dsmem_addr(full_bar(stage), 0);
+                    if (rank == 0) mbar_expect_tx(full_bar(stage), bytes);
+                    tma_load_3d_pair(dst, map, fb, 0, row + kb * BK, block);
+                }
+                ++issued;
                 if (++stage == kWgStages) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) break;
         }
-        if (rank == 0) drain_stages(bar0, kWgStages, filled, last_parity);  // both CTAs' copies
-    } else if (warp == 1 && lane == 0) {
+        if (rank == 0) drain_stages(bar0, kWgStages, issued, stage, phase);  // both CTAs' copies
+    } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         // two 256-column FP32 accumulators: the epilogue of one tile overlaps the
         // MMAs of the next.  A tile of an expert without rows issues no MMA;
         // its epilogue writes zeros.
         int stage = 0, it = 0;
         uint32_t phase = 0;
-        for (int tile = pair; rank == 0 && tile < total && !s_abort; tile += pairs, ++it) {
+        bool ok = true;
+        for (int tile = pair; rank == 0 && tile < total && ok; tile += pairs, ++it) {
             const WgTile t = decode_wg(p, gt, tile);
             const uint32_t idesc = p.idesc | ((uint32_t)(t.bn >> 3) << 17);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
-            if (!mbar_wait(tempty_bar(buf), use ^ 1u, &s_abort, p.status)) break;
+            if (!warp_wait(tempty_bar(buf), use ^ 1u)) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
-            bool ok = true;
+            bool ready = false;
             for (int kb = 0; kb < t.nkb; ++kb) {
-                if (!mbar_wait(full_bar(stage), phase, &s_abort, p.status)) { ok = false; break; }
+                if (!__all_sync(~0u, ready || mbar_wait(full_bar(stage), phase, &s_abort, p.status))) { ok = false; break; }
                 tc_fence_after();
+                const uint32_t eb = empty_bar(stage);
                 const uint32_t sA = sbase + stage * kWgStageBytes, sB = sA + kABytes;
-#pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_pair(d_tmem, mn_sw128_desc(sA + k * 2048, kMnBlockBytes),
-                                mn_sw128_desc(sB + k * 2048, kMnBlockBytes), idesc, (kb | k) != 0);
-                tc_commit_pair(empty_bar(stage));
                 if (++stage == kWgStages) { stage = 0; phase ^= 1u; }
+                ready = mbar_test_wait(full_bar(stage), phase);
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_pair(d_tmem, mn_sw128_desc(sA + k * 2048, kMnBlockBytes),
+                                    mn_sw128_desc(sB + k * 2048, kMnBlockBytes), idesc, (kb | k) != 0);
+                    tc_commit_pair(eb);
+                }
+                __syncwarp();
             }
-            if (!ok) break;
-            tc_commit_pair(tfull_bar(buf));
+            if (ok && elect_one()) tc_commit_pair(tfull_bar(buf));
+            __syncwarp();
         }
         // the leader's last commit: its MMAs and every commit before (whose
         // arrivals reach both CTAs) are done before either CTA exits
-        if (rank == 0) tc_commit_pair(done_bar);
-        const unsigned long long t0 = globaltimer_ns();
-        while (!mbar_try_wait(done_bar, 0))
-            if (globaltimer_ns() - t0 > kWaitLimitNs) break;
-    } else if (warp >= 2) {
+        if (elect_one()) {
+            if (rank == 0) tc_commit_pair(done_bar);
+            const unsigned long long t0 = globaltimer_ns();
+            while (!mbar_try_wait(done_bar, 0))
+                if (globaltimer_ns() - t0 > kWaitLimitNs) break;
+        }
+    } else {
         // ------------------------------------------------ epilogue
         const int quarter = warp & 3;
         const uint32_t out0 = sbase + kWgStages * kWgStageBytes + (uint32_t)((warp - 2) * kWgOutBufs * kWgOutBoxBytes);
@@ -863,7 +908,7 @@ cudaError_t launch_rows_z(const Ctx &c, const RowsGroups &g, const bf16 *d, uint
     for (int q = 0; q < (g.shared_T ? 1 : 2); ++q) {
         uint64_t rows;
         const bf16 *w = pool_tensor(c, g, c.down, q, s.H, &rows);
-        ok &= encode_3d_blocks(&maps.b0[q], w, s.I, rows, 64, p.bn / 128);
+        ok &= encode_3d_blocks(&maps.b0[q], w, s.I, rows, 64, p.bn / 64);
     }
     ok &= encode_2d_box(&maps.out0, zpad, s.I, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     if (!ok) return cudaErrorInvalidValue;
@@ -924,8 +969,8 @@ cudaError_t launch_rows_da(const Ctx &c, const RowsGroups &g, const bf16 *dgu, b
         uint64_t rows;
         const bf16 *wg = pool_tensor(c, g, c.gate, q, s.I, &rows);
         const bf16 *wu = pool_tensor(c, g, c.up, q, s.I, &rows);
-        ok &= encode_3d_blocks(&maps.b0[q], wg, s.H, rows, 64, p.bn / 128);
-        ok &= encode_3d_blocks(&maps.b1[q], wu, s.H, rows, 64, p.bn / 128);
+        ok &= encode_3d_blocks(&maps.b0[q], wg, s.H, rows, 64, p.bn / 64);
+        ok &= encode_3d_blocks(&maps.b1[q], wu, s.H, rows, 64, p.bn / 64);
     }
     ok &= encode_2d_box(&maps.out0, da, s.H, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     if (!ok) return cudaErrorInvalidValue;
