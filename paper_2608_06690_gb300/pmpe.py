@@ -76,7 +76,8 @@ def kernels_per_backward_private(shape) -> int:
 
 
 def kernels_per_backward_input(shape) -> int:
-    """Kernels one input-gradient backward launches: the dispatched rows, the
+    """Kernels one input-gradient backward launches (one less after a forward
+    that saved its accumulators: no dispatched rows): the dispatched rows, the
     dout row gather, Z,
     the gate/up recompute with the SwiGLU backward and dA over the routed
     experts (the same three again over the shared experts, if any), the
