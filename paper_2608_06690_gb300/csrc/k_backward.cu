@@ -30,6 +30,8 @@ __global__ void __launch_bounds__(256) bwd_gather_kernel(const bf16 *dout, const
                                                          const uint32_t *offsets, int g0, int g1, int R, int H,
                                                          bf16 *dout_rows)
 {
+    pdl_trigger();
+    pdl_wait();
     const uint32_t p0 = min(offsets[g0], (uint32_t)R), p1 = min(max(offsets[g1], p0), (uint32_t)R);
     const int nv = H / 8;
     const int rows = (int)(p1 - p0);
@@ -251,6 +253,7 @@ __global__ void bwd_router_kernel(const uint8_t *tau, const int32_t *idx, const 
                                   const float *gw_part, int n_part, int T, int E_pub, int E_priv, int k, int renorm,
                                   int both_pools, int ld, const float *logit_part, int ksplit, float *dz)
 {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
     for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += warps) {
@@ -320,6 +323,7 @@ __global__ void __launch_bounds__(256) bwd_router_wgrad_kernel(const float *dz, 
                                                                const uint8_t *tau, int T, int H, int E_priv,
                                                                int tok_per_split, float *part, int *active)
 {
+    pdl_wait();
     __shared__ float s_dz[32][33];
     __shared__ __align__(16) float s_h[32][128];
     const int e0 = blockIdx.y * 32, c0 = blockIdx.x * 128;
@@ -384,6 +388,8 @@ __global__ void __launch_bounds__(256) bwd_router_wgrad_kernel(const float *dz, 
 // contributes exact zeros).
 __global__ void bwd_router_reduce_kernel(const float *part, const int *active, int nsplit, int n, float *d_router)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ int s_list[kMaxRouterSplits];
     __shared__ int s_n;
     if (threadIdx.x == 0) {
@@ -427,10 +433,10 @@ int router_splits(const Shape &s, int num_sms, int *tok_per_split)
 // w act in the padded row layout ([RP][I], [RP][2I], [RP][I], BF16), the dL/dw
 // partials [R][I / 128], dz [T][E_priv] and the router weight-gradient
 // partials [splits][E_priv][H] (FP32).
-void launch_gather_rows(const bf16 *dout, const int32_t *tok_of_slot, const uint32_t *offsets, int g0, int g1, int R,
+cudaError_t launch_gather_rows(const bf16 *dout, const int32_t *tok_of_slot, const uint32_t *offsets, int g0, int g1, int R,
                         int H, bf16 *rows, int num_sms, cudaStream_t st)
 {
-    bwd_gather_kernel<<<num_sms * 8, 256, 0, st>>>(dout, tok_of_slot, offsets, g0, g1, R, H, rows);
+    return launch_pdl(bwd_gather_kernel, dim3(num_sms * 8), dim3(256), 0, st, dout, tok_of_slot, offsets, g0, g1, R, H, rows);
 }
 
 int router_logit_splits(const Shape &s)
@@ -448,19 +454,18 @@ cudaError_t launch_router_dz(const Ctx &c, const float *gw_part, int both_pools,
     cudaError_t err;
     const int ksplit = router_logit_splits(s);
     if (!s.renorm) {  // the pool softmax needs every logit of the token's pool: tiled GEMMs per pool
-        bwd_pool_tokens_kernel<<<1, 1024, 0, c.stream>>>(c.tau, s.T, pool_tok, pool_n);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+        err = launch_pdl(bwd_pool_tokens_kernel, dim3(1), dim3(1024), 0, c.stream, (const uint8_t *)c.tau, s.T, pool_tok, pool_n);
+        if (err != cudaSuccess) return err;
         const int chunks = (std::max(both_pools ? s.E_pub : 0, s.E_priv) + kPT - 1) / kPT;
         const dim3 grid((s.T + kPT - 1) / kPT, chunks * ksplit, both_pools ? 2 : 1);
-        bwd_pool_logits_kernel<<<grid, 256, 0, c.stream>>>(c.hidden, c.router_pub, c.router_priv, pool_tok, pool_n,
-                                                             s.T, s.H, s.E_pub, s.E_priv, both_pools ? 0 : 1, ksplit, ld,
-                                                             logit_part);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+        err = launch_pdl(bwd_pool_logits_kernel, grid, dim3(256), 0, c.stream, c.hidden, c.router_pub, c.router_priv,
+                         (const int32_t *)pool_tok, (const int *)pool_n, s.T, s.H, s.E_pub, s.E_priv, both_pools ? 0 : 1,
+                         ksplit, ld, logit_part);
+        if (err != cudaSuccess) return err;
     }
-    bwd_router_kernel<<<c.num_sms * 4, 256, 0, c.stream>>>(c.tau, c.idx, c.w, c.slot_of, gw_part, s.I / 128, s.T,
-                                                           s.E_pub, s.E_priv, s.k, s.renorm, both_pools, ld, logit_part,
-                                                           ksplit, dz);
-    return cudaGetLastError();
+    return launch_pdl(bwd_router_kernel, dim3(c.num_sms * 4), dim3(256), 0, c.stream, (const uint8_t *)c.tau,
+                      (const int32_t *)c.idx, (const float *)c.w, (const int32_t *)c.slot_of, gw_part, s.I / 128, s.T,
+                      s.E_pub, s.E_priv, s.k, s.renorm, both_pools, ld, (const float *)logit_part, ksplit, dz);
 }
 
 cudaError_t launch_router_term(const Ctx &c, const float *dz, int ld, const int32_t *pool_tok, const int *pool_n,
@@ -468,9 +473,8 @@ cudaError_t launch_router_term(const Ctx &c, const float *dz, int ld, const int3
 {
     const Shape &s = c.s;
     const dim3 grid((s.T + kPT - 1) / kPT, s.H / kPT, 2);
-    bwd_pool_router_term_kernel<<<grid, 256, 0, c.stream>>>(dz, ld, c.router_pub, c.router_priv, pool_tok, pool_n,
-                                                              s.H, s.E_pub, s.E_priv, d_hidden);
-    return cudaGetLastError();
+    return launch_pdl(bwd_pool_router_term_kernel, grid, dim3(256), 0, c.stream, dz, ld, c.router_pub, c.router_priv,
+                      pool_tok, pool_n, s.H, s.E_pub, s.E_priv, d_hidden);
 }
 
 struct BwdScratch {
@@ -520,8 +524,7 @@ cudaError_t launch_backward_private(const Ctx &c, const bf16 *dout, float *d_rou
     const int E = s.E();
     cudaStream_t st = c.stream;
 
-    launch_gather_rows(dout, c.tok_of_slot, c.offsets, s.E_pub, E, R, H, b.dout_rows, c.num_sms, st);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_gather_rows(dout, c.tok_of_slot, c.offsets, s.E_pub, E, R, H, b.dout_rows, c.num_sms, st);
     if (err != cudaSuccess) return err;
     if ((err = launch_backward_rows(c, b.dout_rows, b.zpad, b.dgu, b.wact, b.gw_part)) != cudaSuccess) return err;
     if ((err = launch_router_dz(c, b.gw_part, 0, s.E_priv, b.dz, b.pool_tok, b.pool_n, b.logit_part)) != cudaSuccess) return err;
@@ -541,14 +544,12 @@ cudaError_t launch_router_wgrad(const Ctx &c, const float *dz, int ld, float *pa
     int per = 32;
     const int nsplit = router_splits(s, c.num_sms, &per);
     dim3 grid((s.H + 127) / 128, (s.E_priv + 31) / 32, nsplit);
-    bwd_router_wgrad_kernel<<<grid, 256, 0, c.stream>>>(dz, ld, c.hidden, c.tau, s.T, s.H, s.E_priv, per, part,
-                                                        active);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_pdl(bwd_router_wgrad_kernel, grid, dim3(256), 0, c.stream, dz, ld, c.hidden,
+                                 (const uint8_t *)c.tau, s.T, s.H, s.E_priv, per, part, active);
     if (err != cudaSuccess) return err;
     const int n = s.E_priv * s.H;
-    bwd_router_reduce_kernel<<<std::min((n + 255) / 256, c.num_sms * 4), 256, 0, c.stream>>>(part, active, nsplit,
-                                                                                              n, d_router);
-    return cudaGetLastError();
+    return launch_pdl(bwd_router_reduce_kernel, dim3(std::min((n + 255) / 256, c.num_sms * 4)), dim3(256), 0, c.stream,
+                      (const float *)part, (const int *)active, nsplit, n, d_router);
 }
 
 }  // namespace pmpe

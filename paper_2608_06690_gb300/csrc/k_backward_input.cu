@@ -209,8 +209,7 @@ cudaError_t launch_backward_input(const Ctx &c, const bf16 *dout, float *d_hidde
 
     // routed experts: the upstream gradient of every dispatch row, then Z,
     // [dG | dU] (and dL/dw partials) and dA over all E experts
-    launch_gather_rows(dout, c.tok_of_slot, c.offsets, 0, E, R, H, b.dout_rows, c.num_sms, st);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_gather_rows(dout, c.tok_of_slot, c.offsets, 0, E, R, H, b.dout_rows, c.num_sms, st);
     if (err != cudaSuccess) return err;
     const RowsGroups g{0, E, 0, b.rp};
     if ((err = launch_rows_z(c, g, b.dout_rows, (uint64_t)R + 64, 1, b.zpad)) != cudaSuccess) return err;
@@ -278,8 +277,7 @@ cudaError_t launch_backward_step(const Ctx &c, const bf16 *dout, float *d_router
     const InScratch &b = st.in;
     cudaStream_t stream = c.stream;
 
-    launch_gather_rows(dout, c.tok_of_slot, c.offsets, 0, E, R, H, b.dout_rows, c.num_sms, stream);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_gather_rows(dout, c.tok_of_slot, c.offsets, 0, E, R, H, b.dout_rows, c.num_sms, stream);
     if (err != cudaSuccess) return err;
     const RowsGroups g{0, E, 0, b.rp};
     if ((err = launch_rows_z(c, g, b.dout_rows, (uint64_t)R + 64, 1, b.zpad)) != cudaSuccess) return err;

@@ -189,6 +189,7 @@ struct RowsParams {
     const bf16 *zpad;     // gate/up: Z in the padded row layout [RP][I]
     float *gw_part;       // gate/up (routed, may be null): [R][I / 128] dL/dw partial per 128-column tile
     int wact;             // gate/up: 1 to write w act to out1 for the private experts' rows
+    int gemm_next;        // 1: another of these launches follows (see pdl_trigger's use)
     int reverse;          // 1: walk the tiles from the last group to the first
     uint32_t *status;
     uint32_t idesc;
@@ -308,6 +309,11 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    // An early start of the next launch pays only when it is another of these
+    // GEMMs (private gradients at T = 1000 437 -> 429 us): a small kernel's CTAs
+    // that started beside a GEMM's ran with the L1 its shared memory left over
+    // (the T = 4096 step 1086 -> 1110 us with every launch triggering).
+    if (kMode == kRowsGU || p.gemm_next) pdl_trigger();
     if (warp == 1) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
     const int nt = p.N / p.bn;
@@ -511,6 +517,7 @@ __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams 
                                                                bf16 *wact)
 {
     __shared__ GroupTable gt;
+    pdl_trigger();
     pdl_wait();
     const int nt = p.I / 128;
     build_groups(gt, p.offsets, p.g0, p.G, p.R, p.shared_T, nt, 0);
@@ -904,6 +911,7 @@ cudaError_t launch_rows_z(const Ctx &c, const RowsGroups &g, const bf16 *d, uint
     p.kb_rows = s.H; p.k_split = s.H / BK;
     p.a_rows = tight ? kArowsTight : kArowsSlot;
     p.idesc = make_idesc_major(BM, p.bn, false, true);
+    p.gemm_next = c.saved_gu == nullptr;
     bool ok = encode_2d(&maps.a, d, s.H, d_rows, BM);
     for (int q = 0; q < (g.shared_T ? 1 : 2); ++q) {
         uint64_t rows;

@@ -123,6 +123,8 @@ __global__ void __launch_bounds__(256) gather_dispatch_rows_kernel(const bf16 *h
                                                                     const uint32_t *offsets, int g0, int g1, int R,
                                                                     int T, int H, bf16 *rows)
 {
+    pdl_trigger();
+    pdl_wait();
     const uint32_t p0 = min(offsets[g0], (uint32_t)R), p1 = min(max(offsets[g1], p0), (uint32_t)R);
     const int nv = H / 8;
     const int lane = threadIdx.x & 31;
@@ -395,9 +397,8 @@ cudaError_t launch_combine(const Ctx &c)
 cudaError_t launch_gather_dispatch_rows(const Ctx &c, int g0, int g1)
 {
     const Shape &s = c.s;
-    gather_dispatch_rows_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.hidden, c.tok_of_slot, c.offsets, g0, g1,
-                                                                     s.T * s.k, s.T, s.H, c.a_perm);
-    return cudaGetLastError();
+    return launch_pdl(gather_dispatch_rows_kernel, dim3(c.num_sms * 8), dim3(256), 0, c.stream, c.hidden,
+                      (const int32_t *)c.tok_of_slot, (const uint32_t *)c.offsets, g0, g1, s.T * s.k, s.T, s.H, c.a_perm);
 }
 
 }  // namespace pmpe

@@ -98,7 +98,7 @@ cudaError_t launch_backward_private(const Ctx &c, const bf16 *dout, float *d_rou
 // router's softmax gradient from the dL/dw partials per slot (both_pools = 0:
 // the private pool, zero for DENY tokens; 1: each token's own pool), dz [T][ld]
 // (pool softmax: the pools' token lists go to pool_tok [T] and pool_n [2]).
-void launch_gather_rows(const bf16 *dout, const int32_t *tok_of_slot, const uint32_t *offsets, int g0, int g1, int R,
+cudaError_t launch_gather_rows(const bf16 *dout, const int32_t *tok_of_slot, const uint32_t *offsets, int g0, int g1, int R,
                         int H, bf16 *rows, int num_sms, cudaStream_t st);
 cudaError_t launch_router_dz(const Ctx &c, const float *gw_part, int both_pools, int ld, float *dz, int32_t *pool_tok,
                              int *pool_n, float *logit_part);
