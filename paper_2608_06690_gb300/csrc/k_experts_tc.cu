@@ -676,7 +676,10 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
     auto tq_empty_bar = [&](int i) { return bar0 + 8u * (3 * kMaxStages + 5 + kTQ + i); };
     // Entry i of the pair's tile sequence, for a consumer role (a whole warp).
     // False at the end of the list or after an abort.
-    auto next_tile = [&](int i, Tile &t) -> bool {
+    // With gather_only (the gather warps) also at the first tile that is not
+    // gathered, after which none is: the warp then leaves every entry's
+    // barrier, so that it no longer polls beside the down tiles.
+    auto next_tile = [&](int i, Tile &t, bool gather_only = false) -> bool {
         const int slot = i % kTQ;
         int ok = 1;
         if (lane == 0) ok = mbar_wait(tq_full_bar(slot), (uint32_t)(i / kTQ) & 1u, &s_abort, p.status) ? 1 : 0;
@@ -687,6 +690,10 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
         t.n0 = (int)y.x; t.rows = (int)y.y; t.row_base = (int)y.z; t.nkb = (int)y.w;
         // (the vote needs every lane's entry: it is read before its slot is handed back)
         const bool live = !__any_sync(~0u, t.flags & kTileEnd) && __all_sync(~0u, t.rows > 0 && t.nkb > 0);
+        if (gather_only && !t.gather()) {
+            if (lane < kTQ) mbar_arrive_drop(dsmem_addr(tq_empty_bar(lane), 0));
+            return false;
+        }
         if (lane == 0) {
             if (rank == 0) mbar_arrive(tq_empty_bar(slot));
             else mbar_arrive_remote(dsmem_addr(tq_empty_bar(slot), 0));
@@ -1369,8 +1376,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
         bool ok = true;
         bool synced = false;                 // wait_dispatch has returned (every lane acquires)
         Tile t;
-        for (int qi = 0; ok && next_tile(qi, t); ++qi) {
-            if (!t.gather()) continue;  // rows through TMA; no gathered tile follows one
+        for (int qi = 0; ok && next_tile(qi, t, true); ++qi) {
             if (!synced && !(synced = __all_sync(~0u, wait_dispatch()))) break;
             // this thread's rows: their token rows in the hidden states
             const int nj = t.n() / 32, first = rank * (t.n() / 2);

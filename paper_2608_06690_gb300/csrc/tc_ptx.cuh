@@ -41,6 +41,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// The last arrival of a participant (address from dsmem_addr): it counts in the
+// current phase, and later phases expect one arrival less.
+__device__ __forceinline__ void mbar_arrive_drop(uint32_t remote_bar)
+{
+    asm volatile("mbarrier.arrive_drop.shared::cluster.b64 _, [%0];\n" ::"r"(remote_bar) : "memory");
+}
 // The phase's state now, without waiting.
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
 {
@@ -59,6 +65,18 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
     return t;
 }
 
+// mbar_try_wait for a longer wait: the thread may sleep up to 20 us (it wakes
+// when the phase completes), so that waiting roles poll less beside busy ones.
+__device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(20000u)
+        : "memory");
+    return ok != 0;
+}
 // Wait for the phase of `bar` with parity `parity`, for at most limit_ns
 // (kWaitLimitNs for the layer's kernels) or until another role raised the
 // abort flag.  On expiry it raises the abort flag, records
@@ -75,7 +93,7 @@ __device__ __noinline__ static bool mbar_wait_for(uint32_t bar, uint32_t parity,
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < kWaitTries; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
+            if (mbar_try_wait_hint(bar, parity)) return true;
         if (*abort_flag) return false;
         const unsigned long long now = globaltimer_ns();
         if (t0 == 0) {
