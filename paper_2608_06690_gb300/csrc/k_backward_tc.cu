@@ -4,10 +4,10 @@
 // TMA -> shared memory -> tcgen05.mma -> TMEM -> epilogue pipeline of the
 // forward's expert GEMMs:
 //
-//   bwd_rows_tc_kernel<kRowsMN>   rows of an expert as M, K = H:
+//   bwd_rows_pair_kernel   K = H (weights as M, an expert's rows as N):
 //     Z = D W_down                  (D: the rows' upstream gradients; W_down read
 //                                    MN-major; so dL/da = w Z) -> BF16
-//   bwd_rows_tc_kernel<kRowsGU>   rows of an expert as M, K = H:
+//   bwd_rows_tc_kernel     rows of an expert as M, K = H:
 //     G = A W_gate^T, U = A W_up^T  (A: the expert's dispatched rows; recomputed)
 //   and in the epilogue, with Z read back, per row and column:
 //     act = bf16(silu(G) U) (the forward's activation), dL/dw partial = sum Z act,
@@ -23,12 +23,11 @@
 //   expert's rows.  FP32 outputs.
 //
 // The same two row kernels, over all routed experts and the shared experts,
-// and an MN-mode launch dA = [dG | dU] [W_gate; W_up] give the gradient of
+// and the pair launch dA = [dG | dU] [W_gate; W_up] give the gradient of
 // the layer's input (launch_rows_z, launch_rows_gu, launch_rows_da).
 //
-// Every launch keeps four 48 KB operand stages in flight (a 128 x 256 x 64 MMA
-// block each) and two 128 x 256 FP32 accumulators, so the epilogue of one tile
-// overlaps the MMAs of the next.  CTA roles (224 threads): warps 0 and 6 issue
+// Every launch keeps 160 to 192 KB of operand stages in flight and two FP32
+// accumulators, so the epilogue of one tile overlaps the MMAs of the next.  CTA roles (224 threads): warps 0 and 6 issue
 // the TMA loads of the first and the second operand, warp 1 allocates TMEM and
 // issues the MMAs, warps 2-5 drain TMEM (one tile row per thread).  Warps 0, 1
 // and 6 run their loops as whole warps, with one elected lane issuing (elect_one).  Every wait
@@ -169,19 +168,18 @@ __device__ __forceinline__ void drain_stages(uint32_t bar0, int stages, int issu
 
 // ------------------------------------------------------------- rows
 
-enum { kRowsMN = 0, kRowsGU = 1 };
 enum { kArowsTight = 0, kArowsSlot = 1, kArowsPad = 2 };
 
-// One launch of the row GEMMs.  Mode kRowsMN: C = A B with A K-major rows
-// (K = K) and B read MN-major from a weight tensor of the group's expert
-// (K blocks below k_split from b0, the rest from b1; kb_rows rows of K per
-// expert in those tensors), C -> BF16 [padded rows][N].  Mode kRowsGU: the
-// gate/up recompute (K = H) and the SwiGLU backward epilogue.
+// One launch of the row GEMMs: C = A B on CTA pairs (A K-major rows of K, B
+// read MN-major from a weight tensor of the group's expert: K blocks below
+// k_split from w0, the rest from w1; kb_rows rows of K per expert in those
+// tensors; C BF16 [padded rows][N]), or the gate/up recompute (K = H) with the
+// SwiGLU backward epilogue.
 struct RowsParams {
     int E_pub, H, I, R;
     int g0, G, shared_T;  // the groups (see build_groups)
     int K, N, bn;         // contracted size, output columns, output columns per tile
-    int kb_rows, k_split; // MN mode: K rows of B per expert; first K block taken from b1
+    int kb_rows, k_split; // C = A B: K rows of B per expert; first K block taken from w1
     int a_rows;           // A row of a tile row: kArowsTight (relative to expert g0's first slot),
                           // kArowsSlot (the dispatch slot; the token for shared groups), kArowsPad
     const uint32_t *offsets;
@@ -197,9 +195,8 @@ struct RowsParams {
 
 struct RowsMaps {
     CUtensorMap a;           // A rows, 64 x 128 box (K-major)
-    CUtensorMap b0[2], b1[2];  // per weight pool (public, private; shared groups use [0]): MN mode:
-                             // 64 x 64 x bn/64 3-D boxes (MN-major); gate/up: gate, up, 64 x 128 (K-major)
-    CUtensorMap out0;        // MN: C [RP][N]; gate/up: [dG | dU] [RP][2I]  (32 x 32 BF16 boxes, 64-byte swizzle)
+    CUtensorMap b0[2], b1[2];  // per weight pool (public, private; shared groups use [0]): gate, up, 64 x 128 (K-major)
+    CUtensorMap out0;        // [dG | dU] [RP][2I]  (32 x 32 BF16 boxes, 64-byte swizzle)
     CUtensorMap out1;        // gate/up: w act [RP][I]
 };
 
@@ -284,7 +281,6 @@ __device__ __forceinline__ float chunk_tree_sum(const float (&q)[32])
     return __fadd_rn(__fadd_rn(t0, t1), __fadd_rn(t2, t3));
 }
 
-template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsParams p, const __grid_constant__ RowsMaps maps)
 {
     extern __shared__ uint8_t dsmem[];
@@ -313,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
     // GEMMs (private gradients at T = 1000 437 -> 429 us): a small kernel's CTAs
     // that started beside a GEMM's ran with the L1 its shared memory left over
     // (the T = 4096 step 1086 -> 1110 us with every launch triggering).
-    if (kMode == kRowsGU || p.gemm_next) pdl_trigger();
+    pdl_trigger();
     if (warp == 1) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
     const int nt = p.N / p.bn;
@@ -334,9 +330,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------ TMA producers
-        // warp 0: the tile's 128 rows x 64 K of A (16 KB).  Warp 6, gate/up: the
-        // 128 gate and the 128 up rows (16 KB each); MN mode: the bn / 64 MN
-        // blocks of B as one 3-D box (8 KB per block).
+        // warp 0: the tile's 128 rows x 64 K of A (16 KB); warp 6: the 128 gate
+        // and the 128 up rows (16 KB each)
         int stage = 0, issued = 0;
         uint32_t phase = 0;
         bool ok = true;
@@ -353,19 +348,10 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
                         mbar_expect_tx(full_bar(stage), kABytes);
                         tma_load_2d(sA, &maps.a, full_bar(stage), kx, arow);
                     }
-                } else if (kMode == kRowsGU) {
-                    if (elect_one()) {
-                        mbar_expect_tx(full_bar(stage), 2 * kABytes);
-                        tma_load_2d(sB, &maps.b0[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
-                        tma_load_2d(sB + kABytes, &maps.b1[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
-                    }
-                } else {
-                    const bool second = kb >= p.k_split;
-                    const int krow = wq.y * p.kb_rows + (second ? kx - p.k_split * BK : kx);
-                    if (elect_one()) {
-                        mbar_expect_tx(full_bar(stage), (uint32_t)(p.bn / 64 * kMnBlockBytes));
-                        tma_load_3d(sB, second ? &maps.b1[wq.x] : &maps.b0[wq.x], full_bar(stage), 0, krow, t.n0 / 64);
-                    }
+                } else if (elect_one()) {
+                    mbar_expect_tx(full_bar(stage), 2 * kABytes);
+                    tma_load_2d(sB, &maps.b0[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
+                    tma_load_2d(sB + kABytes, &maps.b1[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
                 }
                 ++issued;
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -374,8 +360,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
         drain_stages(bar0, kStages, issued, stage, phase);
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        // gate/up: one N = 256 MMA over the gate and up rows, G in accumulator
-        // columns [0, 128) and U in [128, 256); Z: N = bn, W_down MN-major.
+        // one N = 256 MMA over the gate and up rows, G in accumulator columns
+        // [0, 128) and U in [128, 256)
         int stage = 0, it = 0;
         uint32_t phase = 0;
         bool ok = true;
@@ -391,17 +377,13 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
                 tc_fence_after();
                 const uint32_t eb = empty_bar(stage);
                 const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
-                const uint64_t ad = sw128_desc(sA);
+                const uint64_t ad = sw128_desc(sA), bd = sw128_desc(sB);
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 ready = mbar_test_wait(full_bar(stage), phase);
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
-                        // K-major: +32 bytes of K per step inside the swizzle row;
-                        // MN-major: 16 K rows = 2048 bytes per step
-                        const uint64_t bd = kMode == kRowsGU ? sw128_desc(sB) + 2 * k
-                                                             : mn_sw128_desc(sB + k * 2048, kMnBlockBytes);
-                        tc_mma(d_tmem, ad + 2 * k, bd, p.idesc, (kb | k) != 0);
+                        tc_mma(d_tmem, ad + 2 * k, bd + 2 * k, p.idesc, (kb | k) != 0);
                     }
                     tc_commit(eb);
                     if (kb == nkb - 1) tc_commit(tfull_bar(buf));
@@ -434,18 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
             const bool valid = r < t.rows;
             const int orow = gt.pad[t.q] + t.m0 + quarter * 32;  // this warp's 32 rows in the padded layout
             const uint32_t tb = tmem_base + (uint32_t)(buf * kAccCols) + ((uint32_t)(quarter * 32) << 16);
-            if (kMode == kRowsMN) {
-#pragma unroll 1
-                for (int c = 0; c < p.bn / 32; ++c) {
-                    float v[32];
-                    tmem_ld32(tb + c * 32, v);
-                    tmem_ld_wait();
-                    uint32_t pk[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
-                    out.put(lane, pk, &maps.out0, t.n0 + c * 32, orow);
-                }
-            } else {
+            {
                 const int prow = gt.off[t.q] + t.m0 + r;  // row relative to expert g0's first slot (shared: token)
                 const float w = valid ? (p.shared_T ? 1.f : p.w_of_slot[p0 + prow]) : 0.f;
                 const uint4 *zrow = reinterpret_cast<const uint4 *>(p.zpad + (size_t)(orow + lane) * p.I + t.n0);
@@ -503,6 +474,305 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
     }
 }
 
+// ------------------------------------------------------------- rows, CTA pairs
+
+// Z and dA on CTA pairs with the weights as M and the tokens as N, as the
+// forward's expert GEMMs: a tile is 256 output columns (128 a CTA) x up to 256
+// rows of an expert (N a multiple of 32, half staged by each CTA), so that a
+// K step stages 32 KB a CTA for what a single CTA's 128 x 256 tile stages 48 KB,
+// and an expert's rows are padded to 32 instead of 128: Z 145 -> 101 us and dA
+// 201 -> 180 us at the DeepSeek shape, T = 3000 (its shared experts 45 -> 28 and
+// 53 -> 47), 119 -> 112 and 222 -> 199 us at Qwen3 T = 4096, where the weights'
+// DRAM reads bound them.  The weights are read
+// MN-major as stored.  Pair i takes tiles i, i + pairs, ...: tiles of all sizes,
+// and the row tiles of a weight block at the same time.  (Contiguous runs split
+// by the tiles' N took 318 us for dA at Qwen3 T = 4096: a tile of few tokens
+// costs its weights' DRAM time, as much as a full one.)
+constexpr int kPairMaxN = 256;
+constexpr int kPairRing = 6 * 2 * kABytes;      // 6 stages at N = 256
+constexpr int kPairMaxStages = 10;              // at N = 32
+constexpr int kPairOutBytes = 4096;             // per epilogue warp: two 2 KB transpose buffers
+constexpr int kPairDynSmem = kPairRing + 4 * kPairOutBytes + 1024;
+constexpr int kTokBoxes = 4;                    // token row boxes: 128, 64, 32, 16 rows
+
+struct PairMaps {
+    CUtensorMap tok[kTokBoxes];  // the contracted rows' operand (K-major), by box rows
+    CUtensorMap w0[2], w1[2];    // per weight pool, 64 x 64 x 2 3-D boxes (MN-major)
+};
+
+struct PairTable {
+    int tiles[kMaxGroups + 1];   // tiles of the groups before q
+    int rows[kMaxGroups], off[kMaxGroups], pad[kMaxGroups];  // as GroupTable
+    int nmax;                    // bit b: some tile has N = 32 (b + 1)
+};
+
+struct PairTile {
+    int q, m0, n0, n, rows;
+};
+
+__device__ __forceinline__ int pair_row_tiles(int rows) { return (rows + kPairMaxN - 1) / kPairMaxN; }
+__device__ __forceinline__ int pair_row_size(int rows, int mt) { return ((rows + mt - 1) / mt + 31) & ~31; }
+
+// The last entry of a nondecreasing prefix that is <= x, by a whole warp.
+__device__ __forceinline__ int prefix_find(const int *pre, int G, int x, int lane)
+{
+    int n = 0;
+    for (int b = 0; b < G; b += 32) n += __popc(__ballot_sync(~0u, b + lane < G && pre[b + lane] <= x));
+    return n - 1;
+}
+
+__device__ __forceinline__ PairTile decode_pair(const PairTable &pt, int G, int tile, int lane)
+{
+    PairTile t;
+    t.q = prefix_find(pt.tiles, G, tile, lane);
+    const int rows = pt.rows[t.q], mt = pair_row_tiles(rows), bm = pair_row_size(rows, mt);
+    const int local = tile - pt.tiles[t.q], block = local / mt;  // block major: its row tiles share the weights
+    t.m0 = (local - block * mt) * bm;
+    t.n0 = block * 256;
+    t.rows = min(bm, rows - t.m0);
+    t.n = (t.rows + 31) & ~31;
+    return t;
+}
+
+// All threads: the table of a launch over `blocks` 256-column blocks a group.
+__device__ void build_pairs(PairTable &pt, const uint32_t *offsets, int g0, int G, int R, int shared_T, int blocks)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int p0 = shared_T ? 0 : (int)min(offsets[g0], (uint32_t)R);
+    if (tid == 0) pt.nmax = 0;
+    __syncthreads();
+    int nmax = 0;
+    for (int q = tid; q < G; q += blockDim.x) {
+        int b = 0, e = shared_T;
+        if (!shared_T) {
+            b = min(max((int)offsets[g0 + q], p0), R);
+            e = min(max((int)offsets[g0 + q + 1], b), R);
+        }
+        const int rows = e - b, mt = pair_row_tiles(rows), bm = mt ? pair_row_size(rows, mt) : 0;
+        if (mt) nmax |= 1 << (bm / 32 - 1);
+        pt.rows[q] = rows;
+        pt.off[q] = b - p0;
+        pt.tiles[q + 1] = mt * blocks;
+        pt.pad[q] = (rows + kPad - 1) / kPad * kPad;  // made exclusive prefix below
+    }
+    if (nmax) atomicOr(&pt.nmax, nmax);
+    __syncthreads();
+    if (warp < 2) {  // inclusive scan of tiles, exclusive scan of padded rows
+        int *arr = warp == 0 ? pt.tiles + 1 : pt.pad;
+        int carry = 0;
+        for (int b = 0; b < G; b += 32) {
+            const int q = b + lane;
+            const int v = q < G ? arr[q] : 0;
+            int x = v;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(~0u, x, off);
+                if (lane >= off) x += y;
+            }
+            if (q < G) arr[q] = carry + (warp == 1 ? x - v : x);
+            carry += __shfl_sync(~0u, x, 31);
+        }
+        if (warp == 0 && lane == 0) arr[-1] = 0;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsParams p, bf16 *out,
+                                                                    const __grid_constant__ PairMaps maps)
+{
+    extern __shared__ uint8_t dsmem[];
+    __shared__ PairTable pt;
+    __shared__ __align__(8) uint64_t bars[2 * kPairMaxStages + 5];
+    __shared__ uint32_t s_tmem;
+    __shared__ volatile int s_abort;
+
+    const int tid = threadIdx.x, warp = __shfl_sync(~0u, tid >> 5, 0), lane = tid & 31;
+    const int rank = (int)cluster_ctarank();  // 0: the leader, whose warp 1 issues the pair's MMAs
+    const uint32_t sbase = (smem_u32(dsmem) + 1023u) & ~1023u;
+    const uint32_t bar0 = smem_u32(bars);
+    // full (both CTAs' copies) and tempty (both CTAs' epilogues) are the
+    // leader's; empty and tfull are signalled in both CTAs by the commits
+    auto full_bar = [&](int s) { return bar0 + 8u * s; };
+    auto empty_bar = [&](int s) { return bar0 + 8u * (kPairMaxStages + s); };
+    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kPairMaxStages + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kPairMaxStages + 2 + b); };
+    const uint32_t done_bar = bar0 + 8u * (2 * kPairMaxStages + 4);
+
+    if (tid == 0) {
+        for (int s = 0; s < kPairMaxStages; ++s) { mbar_init(full_bar(s), kLoaders); mbar_init(empty_bar(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
+        mbar_init(done_bar, 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (p.gemm_next) pdl_trigger();
+    if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
+    pdl_wait();
+    build_pairs(pt, p.offsets, p.g0, p.G, p.R, p.shared_T, (p.N + 255) / 256);
+    tc_fence_before();
+    cluster_sync_all();  // both CTAs' barriers and TMEM are ready
+    tc_fence_after();
+    const uint32_t tmem_base = s_tmem;
+    const int first = blockIdx.x >> 1, pairs = gridDim.x >> 1, last = pt.tiles[p.G];
+    const int nkb = p.K / BK;
+    const int p0 = p.shared_T ? 0 : (int)min(p.offsets[p.g0], (uint32_t)p.R);
+    const int stage_bytes = kABytes + (pt.nmax ? 32 - __clz(pt.nmax) : 1) * (16 * BK * 2);
+    const int nst = min(kPairMaxStages, kPairRing / stage_bytes);
+    // A barrier wait by a whole warp, with one answer.
+    auto warp_wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        return __all_sync(~0u, mbar_wait(bar, parity, &s_abort, p.status));
+    };
+
+    if (warp == 0 || warp == 6) {
+        // ------------------------------------------------ TMA producers
+        // warp 0: this CTA's half of the tile's token rows (at most three boxes
+        // of 128 to 16 rows); warp 6: its 128 columns of the weights (16 KB).
+        // Every copy completes on the leader's barrier, where the leader's
+        // warps announce both CTAs' bytes.
+        int stage = 0, issued = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = first; tile < last && ok; tile += pairs) {
+            const PairTile t = decode_pair(pt, p.G, tile, lane);
+            if (warp == 0) {
+                const int trows = t.n / 2;
+                const int y = (p.a_rows == kArowsPad ? pt.pad[t.q] : (p.a_rows == kArowsSlot ? p0 : 0) + pt.off[t.q]) +
+                              t.m0 + rank * trows;
+                const int b0 = __clz(trows) - 24, r0 = 128 >> b0;  // the boxes, largest first (trows is 16 .. 128)
+                const int b1 = trows > r0 ? __clz(trows - r0) - 24 : -1, r1 = b1 < 0 ? 0 : r0 + (128 >> b1);
+                const int b2 = b1 >= 0 && trows > r1 ? __clz(trows - r1) - 24 : -1;
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = false; break; }
+                    if (elect_one()) {
+                        const uint32_t sT = sbase + stage * stage_bytes + kABytes;
+                        const uint32_t fb = dsmem_addr(full_bar(stage), 0);
+                        if (rank == 0) mbar_expect_tx(full_bar(stage), (uint32_t)(t.n * BK * 2));
+                        tma_load_2d_pair(sT, &maps.tok[b0], fb, kb * BK, y);
+                        if (b1 >= 0) tma_load_2d_pair(sT + r0 * 128, &maps.tok[b1], fb, kb * BK, y + r0);
+                        if (b2 >= 0) tma_load_2d_pair(sT + r1 * 128, &maps.tok[b2], fb, kb * BK, y + r1);
+                    }
+                    ++issued;
+                    if (++stage == nst) { stage = 0; phase ^= 1u; }
+                }
+            } else {
+                const int2 wq = group_weights(p, t.q);
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = false; break; }
+                    const bool second = kb >= p.k_split;
+                    const int krow = wq.y * p.kb_rows + (second ? kb - p.k_split : kb) * BK;
+                    if (elect_one()) {
+                        if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * kABytes);
+                        tma_load_3d_pair(sbase + stage * stage_bytes, second ? &maps.w1[wq.x] : &maps.w0[wq.x],
+                                         dsmem_addr(full_bar(stage), 0), 0, krow, (t.n0 + rank * 128) / 64);
+                    }
+                    ++issued;
+                    if (++stage == nst) { stage = 0; phase ^= 1u; }
+                }
+            }
+        }
+        if (rank == 0) drain_stages(bar0, nst, issued, stage, phase);  // both CTAs' copies
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        int stage = 0, it = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = first; rank == 0 && tile < last && ok; tile += pairs, ++it) {
+            const PairTile t = decode_pair(pt, p.G, tile, lane);
+            const uint32_t idesc = p.idesc | ((uint32_t)(t.n >> 3) << 17);
+            const int buf = it & 1;
+            const uint32_t use = (uint32_t)(it >> 1) & 1u;
+            if (!warp_wait(tempty_bar(buf), use ^ 1u)) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * kAccCols);
+            bool ready = false;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!__all_sync(~0u, ready || mbar_wait(full_bar(stage), phase, &s_abort, p.status))) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t eb = empty_bar(stage);
+                const uint32_t sW = sbase + stage * stage_bytes;
+                const uint64_t bd = sw128_desc(sW + kABytes);
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+                ready = mbar_test_wait(full_bar(stage), phase);
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_pair(d_tmem, mn_sw128_desc(sW + k * 2048, kMnBlockBytes), bd + 2 * k, idesc, (kb | k) != 0);
+                    tc_commit_pair(eb);
+                    if (kb == nkb - 1) tc_commit_pair(tfull_bar(buf));
+                }
+                __syncwarp();
+            }
+        }
+        // the leader's last commit: its MMAs and every commit before (whose
+        // arrivals reach both CTAs) are done before either CTA exits
+        if (elect_one()) {
+            if (rank == 0) tc_commit_pair(done_bar);
+            const unsigned long long t0 = globaltimer_ns();
+            while (!mbar_try_wait(done_bar, 0))
+                if (globaltimer_ns() - t0 > kWaitLimitNs) break;
+        }
+    } else {
+        // ------------------------------------------------ epilogue
+        // A warp's 32 TMEM lanes are 32 output columns; chunks of 32 tokens are
+        // turned into rows of 64 bytes through shared memory (see the forward's
+        // down projection).  Only the expert's rows are written.
+        const int quarter = warp & 3;
+        const uint32_t own = sbase + kPairRing + quarter * kPairOutBytes;
+        const int srow = lane & 7, scol = lane >> 3;
+        int it = 0;
+        for (int tile = first; tile < last; tile += pairs, ++it) {
+            const PairTile t = decode_pair(pt, p.G, tile, lane);
+            const int buf = it & 1;
+            if (!warp_wait(tfull_bar(buf), (uint32_t)(it >> 1) & 1u)) break;
+            tc_fence_after();
+            const int col = t.n0 + rank * 128 + quarter * 32;
+            const uint32_t tb = tmem_base + (uint32_t)(buf * kAccCols) + ((uint32_t)(quarter * 32) << 16);
+            bf16 *orow = out + (size_t)(pt.pad[t.q] + t.m0) * p.N + col + (lane & 3) * 8;
+#pragma unroll 1
+            for (int c = 0; c < t.n / 32 && col < p.N; ++c) {  // (a last block's second half may lie past N)
+                const uint32_t xo = own + (uint32_t)((c & 1) * 2048);
+                float v[2][16];
+                tmem_frag16(tb + c * 32, v[0]);
+                tmem_frag16(tb + c * 32 + (16u << 16), v[1]);
+                tmem_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int r = 8 * j + srow;
+                    stmatrix_x4_trans(xo + r * 64 + ((scol ^ ((r >> 1) & 3)) << 4), pack_bf16x2(v[0][4 * j], v[0][4 * j + 1]),
+                                      pack_bf16x2(v[0][4 * j + 2], v[0][4 * j + 3]), pack_bf16x2(v[1][4 * j], v[1][4 * j + 1]),
+                                      pack_bf16x2(v[1][4 * j + 2], v[1][4 * j + 3]));
+                }
+                __syncwarp();
+                uint4 f[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const int r = 8 * h + (lane >> 2);
+                    f[h] = ld_shared_v4(xo + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
+                }
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const int tok = c * 32 + 8 * h + (lane >> 2);
+                    if (tok < t.rows) *reinterpret_cast<uint4 *>(orow + (size_t)tok * p.N) = f[h];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                if (rank == 0) mbar_arrive(tempty_bar(buf));
+                else mbar_arrive_remote(dsmem_addr(tempty_bar(buf), 0));
+            }
+        }
+    }
+
+    __syncwarp();
+    tc_fence_before();
+    cluster_sync_all();  // the pair's MMAs, copies and barrier arrivals are done
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, kTmemCols);
+    }
+}
+
 // ------------------------------------------------------------- saved G | U
 
 // The gate/up launch's outputs from the forward's saved accumulators G | U
@@ -510,7 +780,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsPara
 // 128-column tile, four columns per lane (coalesced rows), with the
 // epilogue's per-element arithmetic and its dL/dw summation order
 // (chunk_tree_sum, then the four 32-column chunks in order), so [dG | dU],
-// w act and the dL/dw partials are bitwise those of kRowsGU.  Tiles and the
+// w act and the dL/dw partials are bitwise those of bwd_rows_tc_kernel.  Tiles and the
 // padded layout come from the same group table; padded tail rows are written
 // as zeros.
 __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams p, const float *saved_gu, bf16 *dgu,
@@ -890,13 +1160,25 @@ const bf16 *pool_tensor(const Ctx &c, const RowsGroups &g, const bf16 *const *w,
     return g.shared_T ? w[2] : w[q];
 }
 
-cudaError_t run_rows(int mode, const Ctx &c, const RowsParams &p, const RowsMaps &maps)
+cudaError_t run_rows(const Ctx &c, const RowsParams &p, const RowsMaps &maps)
 {
-    static std::atomic<int> smem_limit[2][64];
-    auto kernel = mode == kRowsMN ? bwd_rows_tc_kernel<kRowsMN> : bwd_rows_tc_kernel<kRowsGU>;
-    cudaError_t err = ensure_dynamic_smem(kernel, kDynSmem, smem_limit[mode]);
+    static std::atomic<int> smem_limit[64];
+    cudaError_t err = ensure_dynamic_smem(bwd_rows_tc_kernel, kDynSmem, smem_limit);
     if (err != cudaSuccess) return err;
-    return launch_pdl(kernel, dim3(c.num_sms), dim3(kThreads), kDynSmem, c.stream, p, maps);
+    return launch_pdl(bwd_rows_tc_kernel, dim3(c.num_sms), dim3(kThreads), kDynSmem, c.stream, p, maps);
+}
+
+// C = A B on CTA pairs: A [a_rows][K] K-major, the weights' maps filled in.
+cudaError_t run_pairs(const Ctx &c, RowsParams &p, PairMaps &maps, const bf16 *a, uint64_t a_rows, bf16 *out)
+{
+    for (int b = 0; b < kTokBoxes; ++b)
+        if (!encode_2d(&maps.tok[b], a, p.K, a_rows, 128u >> b)) return cudaErrorInvalidValue;
+    p.idesc = make_idesc_major(2 * BM, 0, true, false);  // N added per tile
+    static std::atomic<int> smem_limit[64];
+    cudaError_t err = ensure_dynamic_smem(bwd_rows_pair_kernel, kPairDynSmem, smem_limit);
+    if (err != cudaSuccess) return err;
+    return launch_cluster_pdl(bwd_rows_pair_kernel, 2, dim3(c.num_sms / 2 * 2), dim3(kThreads), kPairDynSmem, c.stream, p,
+                              out, maps);
 }
 
 }  // namespace
@@ -905,22 +1187,19 @@ cudaError_t launch_rows_z(const Ctx &c, const RowsGroups &g, const bf16 *d, uint
 {
     const Shape &s = c.s;
     RowsParams p = rows_params(c, g);
-    RowsMaps maps;
+    PairMaps maps;
     memset(&maps, 0, sizeof(maps));
-    p.K = s.H; p.N = s.I; p.bn = s.I % 256 == 0 ? 256 : 128;
+    p.K = s.H; p.N = s.I;
     p.kb_rows = s.H; p.k_split = s.H / BK;
     p.a_rows = tight ? kArowsTight : kArowsSlot;
-    p.idesc = make_idesc_major(BM, p.bn, false, true);
     p.gemm_next = c.saved_gu == nullptr;
-    bool ok = encode_2d(&maps.a, d, s.H, d_rows, BM);
+    bool ok = true;
     for (int q = 0; q < (g.shared_T ? 1 : 2); ++q) {
         uint64_t rows;
         const bf16 *w = pool_tensor(c, g, c.down, q, s.H, &rows);
-        ok &= encode_3d_blocks(&maps.b0[q], w, s.I, rows, 64, p.bn / 64);
+        ok &= encode_3d_blocks(&maps.w0[q], w, s.I, rows, 64, 2);
     }
-    ok &= encode_2d_box(&maps.out0, zpad, s.I, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    if (!ok) return cudaErrorInvalidValue;
-    return run_rows(kRowsMN, c, p, maps);
+    return ok ? run_pairs(c, p, maps, d, d_rows, zpad) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_rows_gu(const Ctx &c, const RowsGroups &g, const bf16 *a, uint64_t a_rows, const bf16 *zpad,
@@ -959,30 +1238,27 @@ cudaError_t launch_rows_gu(const Ctx &c, const RowsGroups &g, const bf16 *a, uin
     ok &= encode_2d_box(&maps.out0, dgu, 2 * (uint64_t)s.I, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     if (wact) ok &= encode_2d_box(&maps.out1, wact, s.I, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     if (!ok) return cudaErrorInvalidValue;
-    return run_rows(kRowsGU, c, p, maps);
+    return run_rows(c, p, maps);
 }
 
 cudaError_t launch_rows_da(const Ctx &c, const RowsGroups &g, const bf16 *dgu, bf16 *da)
 {
     const Shape &s = c.s;
     RowsParams p = rows_params(c, g);
-    RowsMaps maps;
+    PairMaps maps;
     memset(&maps, 0, sizeof(maps));
-    p.K = 2 * s.I; p.N = s.H; p.bn = s.H % 256 == 0 ? 256 : 128;
+    p.K = 2 * s.I; p.N = s.H;
     p.kb_rows = s.I; p.k_split = s.I / BK;  // K blocks of dG take W_gate, those of dU take W_up
     p.a_rows = kArowsPad;
-    p.idesc = make_idesc_major(BM, p.bn, false, true);
-    bool ok = encode_2d(&maps.a, dgu, 2 * (uint64_t)s.I, g.padded_rows, BM);
+    bool ok = true;
     for (int q = 0; q < (g.shared_T ? 1 : 2); ++q) {
         uint64_t rows;
         const bf16 *wg = pool_tensor(c, g, c.gate, q, s.I, &rows);
         const bf16 *wu = pool_tensor(c, g, c.up, q, s.I, &rows);
-        ok &= encode_3d_blocks(&maps.b0[q], wg, s.H, rows, 64, p.bn / 64);
-        ok &= encode_3d_blocks(&maps.b1[q], wu, s.H, rows, 64, p.bn / 64);
+        ok &= encode_3d_blocks(&maps.w0[q], wg, s.H, rows, 64, 2);
+        ok &= encode_3d_blocks(&maps.w1[q], wu, s.H, rows, 64, 2);
     }
-    ok &= encode_2d_box(&maps.out0, da, s.H, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    if (!ok) return cudaErrorInvalidValue;
-    return run_rows(kRowsMN, c, p, maps);
+    return ok ? run_pairs(c, p, maps, dgu, g.padded_rows, da) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_backward_rows(const Ctx &c, const bf16 *dout_rows, bf16 *zpad, bf16 *dgu, bf16 *wact,

@@ -424,6 +424,15 @@ __device__ __forceinline__ void tma_load_3d_pair_hint(uint32_t dst, const CUtens
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+        "[%2];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
+        : "memory");
+}
+
 // One warp of each CTA of the pair executes the allocation and the release.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem_addr, uint32_t ncols)
 {

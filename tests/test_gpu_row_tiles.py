@@ -46,3 +46,36 @@ def test_gate_and_up_tensors(layout, T):
     gpu = run_gpu_layer(shape, wd, hd, pd)
     check_against_oracle(shape, w, h, pol, gpu)
     check_audit(shape, pol, gpu)
+
+
+@pytest.mark.parametrize("T", [33, 130, 257, 300, 520])
+def test_backward_rows_of_one_expert(T):
+    """The backward's row tiles over one expert's rows per pool and one shared
+    expert: both gradients against the oracle, and the same bits from the
+    forward's saved accumulators as from the recompute."""
+    import numpy as np
+
+    import oracle
+    from paper_2608_06690_gb300 import pmpe
+    shape = LayerShape(T=T, H=384, I=256, E_pub=1, E_priv=1, E_sh=1, k=1, renormalize=False)
+    w, h, _ = make_layer(shape, 90 + T)
+    pol = torch.ones(T, dtype=torch.uint8)
+    pol[T // 2:T // 2 + 40] = 0
+    dout = torch.randn((T, shape.H), generator=torch.Generator().manual_seed(T)).to(torch.bfloat16)
+    wd, hd, pd = to_device(w, h, pol)
+    layer = pmpe.MoeLayer(shape, wd)
+    got = []
+    for saved in (False, True):
+        layer.forward(hd, pd, save_for_backward=saved)
+        got.append(layer.backward(hd, pd, dout.cuda()))
+    torch.cuda.synchronize()
+    (g, dh), (g2, dh2) = got
+    assert torch.equal(dh, dh2)
+    L = oracle.Layer(shape, dict(w, hidden=h), pol.numpy())
+    ref = dict(oracle.backward_private(L, dout.double().numpy()),
+               d_hidden=oracle.backward_input(L, dout.double().numpy()))
+    for n, v in dict(g, d_hidden=dh).items():
+        assert n == "d_hidden" or torch.equal(v, g2[n]), n
+        err = np.abs(v.cpu().double().numpy() - ref[n])  # twice the forward's tolerance, as in the backward's tests
+        assert err.max() <= 2e-2 * max(np.abs(ref[n]).max(), 1e-30), n
+        assert err.sum() <= 1e-2 * max(np.abs(ref[n]).sum(), 1e-30), n
