@@ -272,7 +272,10 @@ __global__ void bwd_router_kernel(const uint8_t *tau, const int32_t *idx, const 
             pe = idx[(size_t)t * k + lane] - e_base;
             const int slot = slot_of[(size_t)t * k + lane];
             const float *gp = gw_part + (size_t)slot * n_part;
-            for (int j = 0; j < n_part; ++j) g += gp[j];  // the per-tile partials of dL/dw, in order
+            for (int j = 0; j < n_part; j += 4) {  // the per-32-column partials of dL/dw, in order, 128 columns at a time
+                const float4 c = *reinterpret_cast<const float4 *>(gp + j);
+                g += ((c.x + c.y) + c.z) + c.w;
+            }
             wj = wts[(size_t)t * k + lane];
         }
         float sum = wj * g;
@@ -431,7 +434,7 @@ int router_splits(const Shape &s, int num_sms, int *tok_per_split)
 
 // Scratch of the backward, in order: dout rows [R + 64][H], Z, [dG | dU] and
 // w act in the padded row layout ([RP][I], [RP][2I], [RP][I], BF16), the dL/dw
-// partials [R][I / 128], dz [T][E_priv] and the router weight-gradient
+// partials [R][I / 32], dz [T][E_priv] and the router weight-gradient
 // partials [splits][E_priv][H] (FP32).
 cudaError_t launch_gather_rows(const bf16 *dout, const int32_t *tok_of_slot, const uint32_t *offsets, int g0, int g1, int R,
                         int H, bf16 *rows, int num_sms, cudaStream_t st)
@@ -464,7 +467,7 @@ cudaError_t launch_router_dz(const Ctx &c, const float *gw_part, int both_pools,
         if (err != cudaSuccess) return err;
     }
     return launch_pdl(bwd_router_kernel, dim3(c.num_sms * 4), dim3(256), 0, c.stream, (const uint8_t *)c.tau,
-                      (const int32_t *)c.idx, (const float *)c.w, (const int32_t *)c.slot_of, gw_part, s.I / 128, s.T,
+                      (const int32_t *)c.idx, (const float *)c.w, (const int32_t *)c.slot_of, gw_part, s.I / 32, s.T,
                       s.E_pub, s.E_priv, s.k, s.renorm, both_pools, ld, (const float *)logit_part, ksplit, dz);
 }
 
@@ -497,7 +500,7 @@ static BwdScratch backward_scratch(const Shape &s, uint8_t *base)
     b.zpad = (bf16 *)(base + o);      o += al(RP * I * 2);
     b.dgu = (bf16 *)(base + o);       o += al(RP * 2 * I * 2);
     b.wact = (bf16 *)(base + o);      o += al(RP * I * 2);
-    b.gw_part = (float *)(base + o);  o += al(R * (I / 128) * 4);
+    b.gw_part = (float *)(base + o);  o += al(R * (I / 32) * 4);
     b.dz = (float *)(base + o);       o += al((size_t)s.T * s.E_priv * 4);
     b.part = (float *)(base + o);     o += al(router_wgrad_part_bytes(s));
     b.active = (int *)(base + o);     o += al(kMaxRouterSplits * 4);

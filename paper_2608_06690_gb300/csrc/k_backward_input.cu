@@ -167,7 +167,7 @@ static InScratch input_scratch(const Shape &s, uint8_t *base)
     b.zpad_sh = (bf16 *)(base + o);   o += al(b.rp_sh * I * 2);
     b.dgu_sh = (bf16 *)(base + o);    o += al(b.rp_sh * 2 * I * 2);
     b.da_sh = (bf16 *)(base + o);     o += al(b.rp_sh * H * 2);
-    b.gw_part = (float *)(base + o);  o += al(R * (I / 128) * 4);
+    b.gw_part = (float *)(base + o);  o += al(R * (I / 32) * 4);
     b.dz = (float *)(base + o);       o += al((size_t)s.T * std::max(s.E_pub, s.E_priv) * 4);
     b.pool_tok = (int32_t *)(base + o); o += al((size_t)s.T * 4);
     b.pool_n = (int *)(base + o);     o += al(2 * 4);

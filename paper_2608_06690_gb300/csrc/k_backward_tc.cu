@@ -4,10 +4,10 @@
 // TMA -> shared memory -> tcgen05.mma -> TMEM -> epilogue pipeline of the
 // forward's expert GEMMs:
 //
-//   bwd_rows_pair_kernel   K = H (weights as M, an expert's rows as N):
+//   bwd_rows_pair_kernel<C = A B>   K = H (weights as M, an expert's rows as N):
 //     Z = D W_down                  (D: the rows' upstream gradients; W_down read
 //                                    MN-major; so dL/da = w Z) -> BF16
-//   bwd_rows_tc_kernel     rows of an expert as M, K = H:
+//   bwd_rows_pair_kernel<gate/up>   the same form, K = H:
 //     G = A W_gate^T, U = A W_up^T  (A: the expert's dispatched rows; recomputed)
 //   and in the epilogue, with Z read back, per row and column:
 //     act = bf16(silu(G) U) (the forward's activation), dL/dw partial = sum Z act,
@@ -47,19 +47,11 @@ namespace {
 constexpr int BM = 128;                        // MMA M (rows of a tile)
 constexpr int BK = 64;                         // K per stage
 constexpr int kABytes = BM * BK * 2;           // 16 KB
-constexpr int kBBytes = 256 * BK * 2;          // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kMnBlockBytes = 64 * BK * 2;     // one 64-element MN block of an MN-major operand: 8 KB
 constexpr int kThreads = 224;
 constexpr int kLoaders = 2;                    // loader warps 0 and 6: one operand each
 constexpr int kPad = 128;                      // padded row layout: each expert starts at a multiple of 128
 
-// Four operand stages; outputs staged per epilogue warp in two 2 KB boxes of
-// 32 rows x 64 bytes (32 BF16 or 16 FP32 columns, 64-byte swizzle).
-constexpr int kStages = 4;
-constexpr int kOutBoxBytes = 32 * 64;
-constexpr int kOutBufs = 2;
-constexpr int kDynSmem = kStages * kStageBytes + 4 * kOutBufs * kOutBoxBytes + 1024;
 constexpr int kAccCols = 256;
 constexpr int kTmemCols = 2 * kAccCols;
 
@@ -119,41 +111,6 @@ __device__ void build_groups(GroupTable &gt, const uint32_t *offsets, int g0, in
     __syncthreads();
 }
 
-// This lane's 64-byte row of a staged output box: 16-byte chunk j of row r at
-// chunk j ^ ((r >> 1) & 3), the TMA 64-byte swizzle (conflict-free for these
-// 16-byte writes).
-__device__ __forceinline__ void store_box_row(uint32_t sbuf, int lane, const uint32_t *w16)
-{
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t addr = sbuf + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(w16[4 * j]), "r"(w16[4 * j + 1]),
-                     "r"(w16[4 * j + 2]), "r"(w16[4 * j + 3])
-                     : "memory");
-    }
-}
-
-// One epilogue warp's output path: stage a 32 x 64-byte box in one of two
-// shared buffers and store it with TMA.
-struct OutStager {
-    uint32_t base;
-    int ob;
-    __device__ __forceinline__ void put(int lane, const uint32_t *w16, const CUtensorMap *map, int x, int y)
-    {
-        const uint32_t sbuf = base + (uint32_t)(ob * kOutBoxBytes);
-        if (lane == 0) bulk_wait_read<kOutBufs - 1>();  // the store that used this buffer has read it
-        __syncwarp();
-        store_box_row(sbuf, lane, w16);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-            tma_store_2d(map, sbuf, x, y);
-            bulk_commit();
-        }
-        ob ^= 1;
-    }
-};
-
 // Bounded wait for the drain at exit: every copy a loader issued has landed
 // (the last use of each stage, after `issued` stages up to `stage` in `phase`).
 __device__ __forceinline__ void drain_stages(uint32_t bar0, int stages, int issued, int stage, uint32_t phase)
@@ -178,26 +135,18 @@ enum { kArowsTight = 0, kArowsSlot = 1, kArowsPad = 2 };
 struct RowsParams {
     int E_pub, H, I, R;
     int g0, G, shared_T;  // the groups (see build_groups)
-    int K, N, bn;         // contracted size, output columns, output columns per tile
+    int K, N;             // contracted size, output columns
     int kb_rows, k_split; // C = A B: K rows of B per expert; first K block taken from w1
     int a_rows;           // A row of a tile row: kArowsTight (relative to expert g0's first slot),
                           // kArowsSlot (the dispatch slot; the token for shared groups), kArowsPad
     const uint32_t *offsets;
     const float *w_of_slot;  // gate/up: routing weights per slot (shared groups: weight 1)
     const bf16 *zpad;     // gate/up: Z in the padded row layout [RP][I]
-    float *gw_part;       // gate/up (routed, may be null): [R][I / 128] dL/dw partial per 128-column tile
-    int wact;             // gate/up: 1 to write w act to out1 for the private experts' rows
+    float *gw_part;       // gate/up (routed, may be null): [R][I / 32] dL/dw partial per 32 columns
+    int wact;             // saved gate/up: 1 to write w act for the private experts' rows
     int gemm_next;        // 1: another of these launches follows (see pdl_trigger's use)
-    int reverse;          // 1: walk the tiles from the last group to the first
     uint32_t *status;
     uint32_t idesc;
-};
-
-struct RowsMaps {
-    CUtensorMap a;           // A rows, 64 x 128 box (K-major)
-    CUtensorMap b0[2], b1[2];  // per weight pool (public, private; shared groups use [0]): gate, up, 64 x 128 (K-major)
-    CUtensorMap out0;        // [dG | dU] [RP][2I]  (32 x 32 BF16 boxes, 64-byte swizzle)
-    CUtensorMap out1;        // gate/up: w act [RP][I]
 };
 
 struct RowsTile {
@@ -219,18 +168,6 @@ __device__ __forceinline__ RowsTile rows_tile(const GroupTable &gt, int lo, int 
     return t;
 }
 
-// By a whole warp: the group is the last one whose tile prefix is <= tile
-// (empty groups are passed).
-__device__ __forceinline__ RowsTile decode_rows(const GroupTable &gt, int G, int bn, int tile, int reverse)
-{
-    const int lane = threadIdx.x & 31;
-    if (reverse) tile = gt.tiles[G] - 1 - tile;
-    int n = 0;
-    for (int b = 0; b < G; b += 32) n += __popc(__ballot_sync(~0u, b + lane < G && gt.tiles[b + lane] <= tile));
-    return rows_tile(gt, n - 1, bn, tile);
-}
-
-// By one thread (fewer instructions where every warp of a CTA decodes).
 __device__ __forceinline__ RowsTile decode_rows_thread(const GroupTable &gt, int G, int bn, int tile)
 {
     int lo = 0, hi = G - 1;
@@ -265,215 +202,6 @@ __device__ __forceinline__ void swiglu_bwd(float g, float u, float z, float w, f
     wa = w * a;
 }
 
-// dL/dw over 32 columns of a row: the products z a of four consecutive
-// columns summed pairwise, then those eight sums pairwise.  The order is the
-// butterfly of eight lanes holding four columns each, so a thread holding all
-// 32 (the gate/up epilogue) and a warp holding the row's columns four per
-// lane (bwd_swiglu_saved_kernel) get the same bits.
-__device__ __forceinline__ float chunk_tree_sum(const float (&q)[32])
-{
-    float s[8];
-#pragma unroll
-    for (int l = 0; l < 8; ++l)
-        s[l] = __fadd_rn(__fadd_rn(q[4 * l], q[4 * l + 1]), __fadd_rn(q[4 * l + 2], q[4 * l + 3]));
-    const float t0 = __fadd_rn(s[0], s[1]), t1 = __fadd_rn(s[2], s[3]);
-    const float t2 = __fadd_rn(s[4], s[5]), t3 = __fadd_rn(s[6], s[7]);
-    return __fadd_rn(__fadd_rn(t0, t1), __fadd_rn(t2, t3));
-}
-
-__global__ void __launch_bounds__(kThreads, 1) bwd_rows_tc_kernel(const RowsParams p, const __grid_constant__ RowsMaps maps)
-{
-    extern __shared__ uint8_t dsmem[];
-    __shared__ GroupTable gt;
-    __shared__ __align__(8) uint64_t bars[2 * kStages + 5];
-    __shared__ uint32_t s_tmem;
-    __shared__ volatile int s_abort;
-
-    const int tid = threadIdx.x, warp = __shfl_sync(~0u, tid >> 5, 0), lane = tid & 31;
-    const uint32_t sbase = (smem_u32(dsmem) + 1023u) & ~1023u;
-    const uint32_t bar0 = smem_u32(bars);
-    auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
-    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
-    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kStages + 2 + b); };
-    const uint32_t done_bar = bar0 + 8u * (2 * kStages + 4);
-
-    if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), kLoaders); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 4); }
-        mbar_init(done_bar, 1);
-        s_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    // An early start of the next launch pays only when it is another of these
-    // GEMMs (private gradients at T = 1000 437 -> 429 us): a small kernel's CTAs
-    // that started beside a GEMM's ran with the L1 its shared memory left over
-    // (the T = 4096 step 1086 -> 1110 us with every launch triggering).
-    pdl_trigger();
-    if (warp == 1) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
-    pdl_wait();
-    const int nt = p.N / p.bn;
-    build_groups(gt, p.offsets, p.g0, p.G, p.R, p.shared_T, nt, 0);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = s_tmem;
-    const int total = gt.tiles[p.G];
-    const int nkb = p.K / BK;
-    const int p0 = p.shared_T ? 0 : (int)min(p.offsets[p.g0], (uint32_t)p.R);
-
-    // A barrier wait by a whole warp: every lane waits, and the vote keeps the
-    // warp together and gives one answer.
-    auto warp_wait = [&](uint32_t bar, uint32_t parity) -> bool {
-        return __all_sync(~0u, mbar_wait(bar, parity, &s_abort, p.status));
-    };
-
-    if (warp == 0 || warp == 6) {
-        // ------------------------------------------------ TMA producers
-        // warp 0: the tile's 128 rows x 64 K of A (16 KB); warp 6: the 128 gate
-        // and the 128 up rows (16 KB each)
-        int stage = 0, issued = 0;
-        uint32_t phase = 0;
-        bool ok = true;
-        for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
-            const RowsTile t = decode_rows(gt, p.G, p.bn, tile, p.reverse);
-            const int2 wq = group_weights(p, t.q);
-            const int arow = (p.a_rows == kArowsPad ? gt.pad[t.q] : (p.a_rows == kArowsSlot ? p0 : 0) + gt.off[t.q]) + t.m0;
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = false; break; }
-                const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
-                const int kx = kb * BK;
-                if (warp == 0) {
-                    if (elect_one()) {
-                        mbar_expect_tx(full_bar(stage), kABytes);
-                        tma_load_2d(sA, &maps.a, full_bar(stage), kx, arow);
-                    }
-                } else if (elect_one()) {
-                    mbar_expect_tx(full_bar(stage), 2 * kABytes);
-                    tma_load_2d(sB, &maps.b0[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
-                    tma_load_2d(sB + kABytes, &maps.b1[wq.x], full_bar(stage), kx, wq.y * p.I + t.n0);
-                }
-                ++issued;
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
-            }
-        }
-        drain_stages(bar0, kStages, issued, stage, phase);
-    } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer
-        // one N = 256 MMA over the gate and up rows, G in accumulator columns
-        // [0, 128) and U in [128, 256)
-        int stage = 0, it = 0;
-        uint32_t phase = 0;
-        bool ok = true;
-        for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, ++it) {
-            const int buf = it & 1;
-            const uint32_t use = (uint32_t)(it >> 1) & 1u;
-            if (!warp_wait(tempty_bar(buf), use ^ 1u)) break;
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * kAccCols);
-            bool ready = false;
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!__all_sync(~0u, ready || mbar_wait(full_bar(stage), phase, &s_abort, p.status))) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t eb = empty_bar(stage);
-                const uint32_t sA = sbase + stage * kStageBytes, sB = sA + kABytes;
-                const uint64_t ad = sw128_desc(sA), bd = sw128_desc(sB);
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                ready = mbar_test_wait(full_bar(stage), phase);
-                if (elect_one()) {
-#pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {
-                        tc_mma(d_tmem, ad + 2 * k, bd + 2 * k, p.idesc, (kb | k) != 0);
-                    }
-                    tc_commit(eb);
-                    if (kb == nkb - 1) tc_commit(tfull_bar(buf));
-                }
-                __syncwarp();
-            }
-        }
-        if (elect_one()) {
-            tc_commit(done_bar);
-            const unsigned long long t0 = globaltimer_ns();
-            while (!mbar_try_wait(done_bar, 0))
-                if (globaltimer_ns() - t0 > kWaitLimitNs) break;
-        }
-    } else {
-        // ------------------------------------------------ epilogue
-        const int quarter = warp & 3;
-        OutStager out{sbase + kStages * kStageBytes + (uint32_t)((warp - 2) * kOutBufs * kOutBoxBytes), 0};
-        int it = 0;
-        for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++it) {
-            const RowsTile t = decode_rows(gt, p.G, p.bn, tile, p.reverse);
-            const int buf = it & 1;
-            const uint32_t use = (uint32_t)(it >> 1) & 1u;
-            int ok = 1;
-            if (lane == 0) ok = mbar_wait(tfull_bar(buf), use, &s_abort, p.status) ? 1 : 0;
-            ok = __shfl_sync(~0u, ok, 0);
-            if (!ok) break;
-            __syncwarp();
-            tc_fence_after();
-            const int r = quarter * 32 + lane;
-            const bool valid = r < t.rows;
-            const int orow = gt.pad[t.q] + t.m0 + quarter * 32;  // this warp's 32 rows in the padded layout
-            const uint32_t tb = tmem_base + (uint32_t)(buf * kAccCols) + ((uint32_t)(quarter * 32) << 16);
-            {
-                const int prow = gt.off[t.q] + t.m0 + r;  // row relative to expert g0's first slot (shared: token)
-                const float w = valid ? (p.shared_T ? 1.f : p.w_of_slot[p0 + prow]) : 0.f;
-                const uint4 *zrow = reinterpret_cast<const uint4 *>(p.zpad + (size_t)(orow + lane) * p.I + t.n0);
-                float gw = 0.f;
-#pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
-                    uint4 zq[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) zq[i] = valid ? zrow[c * 4 + i] : make_uint4(0u, 0u, 0u, 0u);
-                    float g[32], u[32];
-                    tmem_ld32(tb + c * 32, g);
-                    tmem_ld32(tb + 128 + c * 32, u);
-                    tmem_ld_wait();
-                    const __nv_bfloat162 *zb = reinterpret_cast<const __nv_bfloat162 *>(zq);
-                    uint32_t pg[16], pu[16], pa[16];
-                    float zq_a[32];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float2 z2 = __bfloat1622float2(zb[i]);
-                        float dg[2], du[2], wa[2];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int j = 2 * i + h;
-                            float a;
-                            const float z = h ? z2.y : z2.x;
-                            swiglu_bwd(g[j], u[j], z, w, a, dg[h], du[h], wa[h]);
-                            zq_a[j] = __fmul_rn(z, a);
-                            if (!valid) dg[h] = du[h] = wa[h] = 0.f;
-                        }
-                        pg[i] = pack_bf16x2(dg[0], dg[1]);
-                        pu[i] = pack_bf16x2(du[0], du[1]);
-                        pa[i] = pack_bf16x2(wa[0], wa[1]);
-                    }
-                    gw = __fadd_rn(gw, chunk_tree_sum(zq_a));
-                    out.put(lane, pg, &maps.out0, t.n0 + c * 32, orow);
-                    out.put(lane, pu, &maps.out0, p.I + t.n0 + c * 32, orow);
-                    if (p.wact && !p.shared_T && p.g0 + t.q >= p.E_pub)
-                        out.put(lane, pa, &maps.out1, t.n0 + c * 32, orow);
-                }
-                if (valid && p.gw_part) p.gw_part[(size_t)(p0 + prow) * nt + t.n_tile] = gw;
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(buf));
-        }
-        if (lane == 0) bulk_wait_all();
-    }
-
-    __syncwarp();
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
-    }
-}
-
 // ------------------------------------------------------------- rows, CTA pairs
 
 // Z and dA on CTA pairs with the weights as M and the tokens as N, as the
@@ -492,12 +220,22 @@ constexpr int kPairMaxN = 256;
 constexpr int kPairRing = 6 * 2 * kABytes;      // 6 stages at N = 256
 constexpr int kPairMaxStages = 10;              // at N = 32
 constexpr int kPairOutBytes = 4096;             // per epilogue warp: two 2 KB transpose buffers
-constexpr int kPairDynSmem = kPairRing + 4 * kPairOutBytes + 1024;
+constexpr int kPairRowWBytes = kPairMaxN * 4;   // per epilogue warp: the tile's routing weights
+constexpr int kPairDynSmem = kPairRing + 4 * (kPairOutBytes + kPairRowWBytes) + 1024;
 constexpr int kTokBoxes = 4;                    // token row boxes: 128, 64, 32, 16 rows
 
 struct PairMaps {
     CUtensorMap tok[kTokBoxes];  // the contracted rows' operand (K-major), by box rows
-    CUtensorMap w0[2], w1[2];    // per weight pool, 64 x 64 x 2 3-D boxes (MN-major)
+    CUtensorMap w0[2], w1[2];    // per weight pool, 64 x 64 x 2 3-D boxes (MN-major); gate/up: 64-row boxes of
+                                 // the gate and the up rows, where one box cannot hold both
+    CUtensorMap gu[2];           // gate/up: 64 gate and 64 up rows (encode_3d_two)
+};
+
+// The gate/up recompute's outputs (GuOut) or C.
+struct PairOut {
+    bf16 *c;              // C [padded rows][N], or [dG | dU] [padded rows][2I]
+    bf16 *wact;           // gate/up: w act [padded rows][I] (private experts' rows), or NULL
+    uint8_t up_first[2], two_boxes[2];  // gate/up, per weight pool: the box's order; two boxes
 };
 
 struct PairTable {
@@ -521,20 +259,20 @@ __device__ __forceinline__ int prefix_find(const int *pre, int G, int x, int lan
     return n - 1;
 }
 
-__device__ __forceinline__ PairTile decode_pair(const PairTable &pt, int G, int tile, int lane)
+__device__ __forceinline__ PairTile decode_pair(const PairTable &pt, int G, int width, int tile, int lane)
 {
     PairTile t;
     t.q = prefix_find(pt.tiles, G, tile, lane);
     const int rows = pt.rows[t.q], mt = pair_row_tiles(rows), bm = pair_row_size(rows, mt);
     const int local = tile - pt.tiles[t.q], block = local / mt;  // block major: its row tiles share the weights
     t.m0 = (local - block * mt) * bm;
-    t.n0 = block * 256;
+    t.n0 = block * width;
     t.rows = min(bm, rows - t.m0);
     t.n = (t.rows + 31) & ~31;
     return t;
 }
 
-// All threads: the table of a launch over `blocks` 256-column blocks a group.
+// All threads: the table of a launch over `blocks` column blocks a group.
 __device__ void build_pairs(PairTable &pt, const uint32_t *offsets, int g0, int G, int R, int shared_T, int blocks)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -577,7 +315,181 @@ __device__ void build_pairs(PairTable &pt, const uint32_t *offsets, int g0, int 
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsParams p, bf16 *out,
+// The rows of a 16-token x 32-column tile of BF16 pairs (pk[4 h + 2 j + q]:
+// tokens 8 j + 2 (lane & 3), + 1 of column 16 h + 8 q + lane / 4) through 1 KB
+// of shared memory: f[i] is this lane's 8 columns 8 (lane & 3) of token 8 i + lane / 4.
+__device__ __forceinline__ void rows16(uint32_t buf, int lane, const uint32_t *pk, uint4 *f)
+{
+    const int srow = lane & 7, scol = lane >> 3;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int r = 8 * j + srow;
+        stmatrix_x4_trans(buf + r * 64 + ((scol ^ ((r >> 1) & 3)) << 4), pk[2 * j], pk[2 * j + 1], pk[4 + 2 * j],
+                          pk[5 + 2 * j]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = 8 * h + (lane >> 2);
+        f[h] = ld_shared_v4(buf + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
+    }
+}
+
+// The SwiGLU backward of a gate/up tile by one epilogue warp: per chunk of 32
+// tokens it computes 16 (first 16: warps 0-1) of its 32 columns, from its own
+// accumulators and its partner's (exchanged as in the forward), with Z read
+// row by row and turned into the accumulators' layout by ldmatrix.  dL/dw is
+// summed over the 32 columns in the order of bwd_swiglu_saved_kernel (pairs of
+// neighbouring columns, then pairs of pairs, ...), by a butterfly that halves
+// the values it carries.  Rows past the expert's, to the end of its padded
+// rows, are written as zeros.
+__device__ __forceinline__ void gu_epilogue(const RowsParams &p, const PairOut &out, const PairTable &pt, const PairTile &t,
+                                            uint32_t tb, uint32_t own, uint32_t partner, uint32_t roww, int rank,
+                                            int quarter, int lane, int prow, int p0)
+{
+    const bool first = quarter < 2;
+    const int2 wq = group_weights(p, t.q);
+    const bool gate = first != (out.up_first[wq.x] != 0);
+    const int col = t.n0 + rank * 64 + (quarter & 1) * 32, half = first ? 0 : 16;
+    const int I = p.I, ch8 = (lane & 3) * 8, r4 = lane >> 2;
+    const bool wa_out = out.wact != nullptr && !p.shared_T && p.g0 + t.q >= p.E_pub;
+    bf16 *drow = out.c + (size_t)prow * 2 * I + col + ch8;
+    bf16 *arow = wa_out ? out.wact + (size_t)prow * I + col + ch8 : nullptr;
+    const bf16 *zrow = p.zpad + (size_t)prow * I + col + ch8;
+    const int nch = t.n / 32;
+    uint4 z[2];
+    auto load_z = [&](int c) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int tok = c * 32 + half + 8 * h + r4;
+            z[h] = c < nch && tok < t.rows ? *reinterpret_cast<const uint4 *>(zrow + (size_t)tok * I)
+                                           : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    load_z(0);
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+        const uint32_t xo = own + (uint32_t)((c & 1) * 2048), xp = partner + (uint32_t)((c & 1) * 2048);
+        float v[2][16];
+        tmem_frag16(tb + c * 32, v[0]);
+        tmem_frag16(tb + c * 32 + (16u << 16), v[1]);
+        tmem_ld_wait();
+        float mine[16], other[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float *s = &v[i >> 1][(i & 1) * 4];  // tokens 0-15; + 8: tokens 16-31
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mine[4 * i + q] = first ? s[q] : s[8 + q];
+            st_shared_v4(xo + i * 512 + lane * 16,
+                         make_uint4(__float_as_uint(first ? s[8] : s[0]), __float_as_uint(first ? s[9] : s[1]),
+                                    __float_as_uint(first ? s[10] : s[2]), __float_as_uint(first ? s[11] : s[3])));
+        }
+        named_barrier_sync(1 + (quarter & 1), 64);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint4 f = ld_shared_v4(xp + i * 512 + lane * 16);
+            other[4 * i] = __uint_as_float(f.x); other[4 * i + 1] = __uint_as_float(f.y);
+            other[4 * i + 2] = __uint_as_float(f.z); other[4 * i + 3] = __uint_as_float(f.w);
+        }
+        __syncwarp();
+        // Z through the partner's buffer, which this warp has read (and the
+        // partner fills again only after their next barrier)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = 8 * h + r4;
+            st_shared_v4(xp + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4), z[h]);
+        }
+        __syncwarp();
+        uint32_t zf[2][4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int r = 8 * j + (lane & 7);
+            ldmatrix_x4_trans(zf[j][0], zf[j][1], zf[j][2], zf[j][3], xp + r * 64 + (((lane >> 3) ^ ((r >> 1) & 3)) << 4));
+        }
+        load_z(c + 1);
+        uint32_t pg[8], pu[8], pa[8];  // [4 h + 2 j + q / 2]
+        float s[16];                   // z a: [8 j + 4 (token parity) + 2 h + q / 2]
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 w2 = ld_shared_f32x2(roww + (c * 32 + half + 8 * j + 2 * (lane & 3)) * 4);
+            const int tok = c * 32 + half + 8 * j + 2 * (lane & 3);
+            const bool v0 = tok < t.rows, v1 = tok + 1 < t.rows;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {  // column group 8 a: h = a / 2, q / 2 = a & 1
+                const int i = 4 * (2 * (a >> 1) + j) + 2 * (a & 1);
+                const float2 zz = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&zf[j][a]));
+                float act, dg[2], du[2], wa[2];
+                swiglu_bwd(gate ? mine[i] : other[i], gate ? other[i] : mine[i], zz.x, w2.x, act, dg[0], du[0], wa[0]);
+                s[8 * j + a] = __fmul_rn(zz.x, act);
+                swiglu_bwd(gate ? mine[i + 1] : other[i + 1], gate ? other[i + 1] : mine[i + 1], zz.y, w2.y, act, dg[1],
+                           du[1], wa[1]);
+                s[8 * j + 4 + a] = __fmul_rn(zz.y, act);
+                if (!v0) dg[0] = du[0] = wa[0] = 0.f;
+                if (!v1) dg[1] = du[1] = wa[1] = 0.f;
+                const int o = 4 * (a >> 1) + 2 * j + (a & 1);
+                pg[o] = pack_bf16x2(dg[0], dg[1]);
+                pu[o] = pack_bf16x2(du[0], du[1]);
+                pa[o] = pack_bf16x2(wa[0], wa[1]);
+            }
+        }
+        __syncwarp();  // Z has been read
+        uint4 f[2], f2[2];
+        rows16(xp, lane, pg, f);
+        rows16(xp + 1024, lane, pu, f2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            bf16 *d = drow + (size_t)(c * 32 + half + 8 * h + r4) * 2 * I;
+            *reinterpret_cast<uint4 *>(d) = f[h];
+            *reinterpret_cast<uint4 *>(d + I) = f2[h];
+        }
+        if (wa_out) {
+            __syncwarp();
+            rows16(xp, lane, pa, f);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                *reinterpret_cast<uint4 *>(arow + (size_t)(c * 32 + half + 8 * h + r4) * I) = f[h];
+        }
+        if (p.gw_part) {
+            // over the 8 columns of each group (lane / 4): at each level a lane
+            // keeps the half of its values that its bit names
+            float a8[8], a4[4], a2[2];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {  // keep token octet j = bit 2
+                const float keep = (lane & 4) ? s[8 + i] : s[i], give = (lane & 4) ? s[i] : s[8 + i];
+                a8[i] = __fadd_rn(keep, __shfl_xor_sync(~0u, give, 4));
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {  // keep token parity = bit 3
+                const float keep = (lane & 8) ? a8[4 + i] : a8[i], give = (lane & 8) ? a8[i] : a8[4 + i];
+                a4[i] = __fadd_rn(keep, __shfl_xor_sync(~0u, give, 8));
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {  // keep column groups 0-1 or 2-3 = bit 4
+                const float keep = (lane & 16) ? a4[2 + i] : a4[i], give = (lane & 16) ? a4[i] : a4[2 + i];
+                a2[i] = __fadd_rn(keep, __shfl_xor_sync(~0u, give, 16));
+            }
+            const float b = __fadd_rn(a2[0], a2[1]);
+            const float gw = __fadd_rn(b, __shfl_xor_sync(~0u, b, 16));
+            const int tok = c * 32 + half + ((lane & 4) ? 8 : 0) + 2 * (lane & 3) + ((lane & 8) ? 1 : 0);
+            if (lane < 16 && tok < t.rows)
+                p.gw_part[(size_t)(p0 + pt.off[t.q] + t.m0 + tok) * (I / 32) + col / 32] = gw;
+        }
+    }
+    if (t.m0 + t.rows == pt.rows[t.q]) {  // the expert's last rows: zeros to the end of its padded rows
+        const int end = (pt.rows[t.q] + kPad - 1) / kPad * kPad - t.m0;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        for (int r = t.n + r4 + (first ? 0 : 8); r < end; r += 16) {
+            *reinterpret_cast<uint4 *>(drow + (size_t)r * 2 * I) = zero;
+            *reinterpret_cast<uint4 *>(drow + (size_t)r * 2 * I + I) = zero;
+            if (wa_out) *reinterpret_cast<uint4 *>(arow + (size_t)r * I) = zero;
+        }
+    }
+}
+
+// kGU: the gate/up recompute with the SwiGLU backward (tiles of 128 columns: each
+// CTA 64 gate and the same 64 up columns, as the forward's); else C = A B.
+template <bool kGU>
+__global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsParams p, const PairOut out,
                                                                     const __grid_constant__ PairMaps maps)
 {
     extern __shared__ uint8_t dsmem[];
@@ -605,10 +517,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (p.gemm_next) pdl_trigger();
+    // An early start of the next launch pays only when it is another of these
+    // GEMMs (private gradients at T = 1000 437 -> 429 us): a small kernel's CTAs
+    // that started beside a GEMM's ran with the L1 its shared memory left over
+    // (the T = 4096 step 1086 -> 1110 us with every launch triggering).
+    if (kGU || p.gemm_next) pdl_trigger();
     if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
-    build_pairs(pt, p.offsets, p.g0, p.G, p.R, p.shared_T, (p.N + 255) / 256);
+    const int width = kGU ? 128 : 256;  // output columns of a tile
+    build_pairs(pt, p.offsets, p.g0, p.G, p.R, p.shared_T, (p.N + width - 1) / width);
     tc_fence_before();
     cluster_sync_all();  // both CTAs' barriers and TMEM are ready
     tc_fence_after();
@@ -633,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
         uint32_t phase = 0;
         bool ok = true;
         for (int tile = first; tile < last && ok; tile += pairs) {
-            const PairTile t = decode_pair(pt, p.G, tile, lane);
+            const PairTile t = decode_pair(pt, p.G, width, tile, lane);
             if (warp == 0) {
                 const int trows = t.n / 2;
                 const int y = (p.a_rows == kArowsPad ? pt.pad[t.q] : (p.a_rows == kArowsSlot ? p0 : 0) + pt.off[t.q]) +
@@ -658,12 +575,26 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
                 const int2 wq = group_weights(p, t.q);
                 for (int kb = 0; kb < nkb; ++kb) {
                     if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = false; break; }
-                    const bool second = kb >= p.k_split;
-                    const int krow = wq.y * p.kb_rows + (second ? kb - p.k_split : kb) * BK;
-                    if (elect_one()) {
-                        if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * kABytes);
-                        tma_load_3d_pair(sbase + stage * stage_bytes, second ? &maps.w1[wq.x] : &maps.w0[wq.x],
-                                         dsmem_addr(full_bar(stage), 0), 0, krow, (t.n0 + rank * 128) / 64);
+                    const uint32_t sW = sbase + stage * stage_bytes, fb = dsmem_addr(full_bar(stage), 0);
+                    if (kGU) {
+                        const int y = wq.y * p.I + t.n0 + rank * 64;
+                        if (elect_one()) {
+                            if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * kABytes);
+                            if (!out.two_boxes[wq.x]) {
+                                tma_load_3d_pair(sW, &maps.gu[wq.x], fb, kb * BK, y, 0);
+                            } else {
+                                tma_load_2d_pair(sW, &maps.w0[wq.x], fb, kb * BK, y);
+                                tma_load_2d_pair(sW + kABytes / 2, &maps.w1[wq.x], fb, kb * BK, y);
+                            }
+                        }
+                    } else {
+                        const bool second = kb >= p.k_split;
+                        const int krow = wq.y * p.kb_rows + (second ? kb - p.k_split : kb) * BK;
+                        if (elect_one()) {
+                            if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * kABytes);
+                            tma_load_3d_pair(sW, second ? &maps.w1[wq.x] : &maps.w0[wq.x], fb, 0, krow,
+                                             (t.n0 + rank * 128) / 64);
+                        }
                     }
                     ++issued;
                     if (++stage == nst) { stage = 0; phase ^= 1u; }
@@ -677,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
         uint32_t phase = 0;
         bool ok = true;
         for (int tile = first; rank == 0 && tile < last && ok; tile += pairs, ++it) {
-            const PairTile t = decode_pair(pt, p.G, tile, lane);
+            const PairTile t = decode_pair(pt, p.G, width, tile, lane);
             const uint32_t idesc = p.idesc | ((uint32_t)(t.n >> 3) << 17);
             const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1) & 1u;
@@ -696,7 +627,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        tc_mma_pair(d_tmem, mn_sw128_desc(sW + k * 2048, kMnBlockBytes), bd + 2 * k, idesc, (kb | k) != 0);
+                        tc_mma_pair(d_tmem, kGU ? sw128_desc(sW) + 2 * k : mn_sw128_desc(sW + k * 2048, kMnBlockBytes),
+                                    bd + 2 * k, idesc, (kb | k) != 0);
                     tc_commit_pair(eb);
                     if (kb == nkb - 1) tc_commit_pair(tfull_bar(buf));
                 }
@@ -715,44 +647,67 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
         // ------------------------------------------------ epilogue
         // A warp's 32 TMEM lanes are 32 output columns; chunks of 32 tokens are
         // turned into rows of 64 bytes through shared memory (see the forward's
-        // down projection).  Only the expert's rows are written.
+        // epilogues, whose exchange of gate and up values this one shares).
         const int quarter = warp & 3;
-        const uint32_t own = sbase + kPairRing + quarter * kPairOutBytes;
+        const uint32_t stage0 = sbase + kPairRing;
+        const uint32_t own = stage0 + quarter * kPairOutBytes, partner = stage0 + (quarter ^ 2) * kPairOutBytes;
+        const uint32_t roww = stage0 + 4 * kPairOutBytes + quarter * kPairRowWBytes;
         const int srow = lane & 7, scol = lane >> 3;
         int it = 0;
         for (int tile = first; tile < last; tile += pairs, ++it) {
-            const PairTile t = decode_pair(pt, p.G, tile, lane);
+            const PairTile t = decode_pair(pt, p.G, width, tile, lane);
             const int buf = it & 1;
-            if (!warp_wait(tfull_bar(buf), (uint32_t)(it >> 1) & 1u)) break;
-            tc_fence_after();
-            const int col = t.n0 + rank * 128 + quarter * 32;
-            const uint32_t tb = tmem_base + (uint32_t)(buf * kAccCols) + ((uint32_t)(quarter * 32) << 16);
-            bf16 *orow = out + (size_t)(pt.pad[t.q] + t.m0) * p.N + col + (lane & 3) * 8;
-#pragma unroll 1
-            for (int c = 0; c < t.n / 32 && col < p.N; ++c) {  // (a last block's second half may lie past N)
-                const uint32_t xo = own + (uint32_t)((c & 1) * 2048);
-                float v[2][16];
-                tmem_frag16(tb + c * 32, v[0]);
-                tmem_frag16(tb + c * 32 + (16u << 16), v[1]);
-                tmem_ld_wait();
+            const int prow = pt.pad[t.q] + t.m0;  // the tile's first row of the padded layout
+            if (kGU) {  // the rows' routing weights, ahead of the accumulator
+                const int slot0 = p0 + pt.off[t.q] + t.m0;
+                float w[kPairMaxN / 32];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int r = 8 * j + srow;
-                    stmatrix_x4_trans(xo + r * 64 + ((scol ^ ((r >> 1) & 3)) << 4), pack_bf16x2(v[0][4 * j], v[0][4 * j + 1]),
-                                      pack_bf16x2(v[0][4 * j + 2], v[0][4 * j + 3]), pack_bf16x2(v[1][4 * j], v[1][4 * j + 1]),
-                                      pack_bf16x2(v[1][4 * j + 2], v[1][4 * j + 3]));
+                for (int c = 0; c < kPairMaxN / 32; ++c) {
+                    const int r = c * 32 + lane;
+                    w[c] = r < t.rows ? (p.shared_T ? 1.f : p.w_of_slot[slot0 + r]) : 0.f;
                 }
                 __syncwarp();
-                uint4 f[4];
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    const int r = 8 * h + (lane >> 2);
-                    f[h] = ld_shared_v4(xo + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
-                }
+                for (int c = 0; c < kPairMaxN / 32; ++c) st_shared_f32(roww + (c * 32 + lane) * 4, w[c]);
+                __syncwarp();
+            }
+            const bool ok = warp_wait(tfull_bar(buf), (uint32_t)(it >> 1) & 1u);
+            // (gate/up: the four warps, which meet at barriers inside a tile, go on or stop together)
+            if (kGU ? !named_barrier_all(3, 128, ok) : !ok) break;
+            tc_fence_after();
+            const uint32_t tb = tmem_base + (uint32_t)(buf * kAccCols) + ((uint32_t)(quarter * 32) << 16);
+            if (kGU) {
+                gu_epilogue(p, out, pt, t, tb, own, partner, roww, rank, quarter, lane, prow, p0);
+            } else {
+                const int col = t.n0 + rank * 128 + quarter * 32;
+                bf16 *orow = out.c + (size_t)prow * p.N + col + (lane & 3) * 8;
+#pragma unroll 1
+                for (int c = 0; c < t.n / 32 && col < p.N; ++c) {  // (a last block's second half may lie past N)
+                    const uint32_t xo = own + (uint32_t)((c & 1) * 2048);
+                    float v[2][16];
+                    tmem_frag16(tb + c * 32, v[0]);
+                    tmem_frag16(tb + c * 32 + (16u << 16), v[1]);
+                    tmem_ld_wait();
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    const int tok = c * 32 + 8 * h + (lane >> 2);
-                    if (tok < t.rows) *reinterpret_cast<uint4 *>(orow + (size_t)tok * p.N) = f[h];
+                    for (int j = 0; j < 4; ++j) {
+                        const int r = 8 * j + srow;
+                        stmatrix_x4_trans(xo + r * 64 + ((scol ^ ((r >> 1) & 3)) << 4), pack_bf16x2(v[0][4 * j], v[0][4 * j + 1]),
+                                          pack_bf16x2(v[0][4 * j + 2], v[0][4 * j + 3]),
+                                          pack_bf16x2(v[1][4 * j], v[1][4 * j + 1]),
+                                          pack_bf16x2(v[1][4 * j + 2], v[1][4 * j + 3]));
+                    }
+                    __syncwarp();
+                    uint4 f[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int r = 8 * h + (lane >> 2);
+                        f[h] = ld_shared_v4(xo + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
+                    }
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int tok = c * 32 + 8 * h + (lane >> 2);
+                        if (tok < t.rows) *reinterpret_cast<uint4 *>(orow + (size_t)tok * p.N) = f[h];
+                    }
                 }
             }
             tc_fence_before();
@@ -780,7 +735,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
 // 128-column tile, four columns per lane (coalesced rows), with the
 // epilogue's per-element arithmetic and its dL/dw summation order
 // (chunk_tree_sum, then the four 32-column chunks in order), so [dG | dU],
-// w act and the dL/dw partials are bitwise those of bwd_rows_tc_kernel.  Tiles and the
+// w act and the dL/dw partials are bitwise those of bwd_rows_pair_kernel.  Tiles and the
 // padded layout come from the same group table; padded tail rows are written
 // as zeros.
 __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams p, const float *saved_gu, bf16 *dgu,
@@ -834,22 +789,18 @@ __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams 
             if (wa_out)
                 *reinterpret_cast<uint2 *>(wact + (size_t)orow * p.I + col) =
                     make_uint2(pack_bf16x2(wa[0], wa[1]), pack_bf16x2(wa[2], wa[3]));
-            // the 32-column chunk sums in chunk_tree_sum's order: four columns in
-            // the lane, then the butterfly over the chunk's eight lanes
+            // the 32-column chunk sums: pairs of neighbouring columns, then pairs of
+            // those, and so on (four columns in the lane, then a butterfly over
+            // the chunk's eight lanes)
             float sum = __fadd_rn(__fadd_rn(q[0], q[1]), __fadd_rn(q[2], q[3]));
             sum = __fadd_rn(sum, __shfl_xor_sync(~0u, sum, 1));
             sum = __fadd_rn(sum, __shfl_xor_sync(~0u, sum, 2));
             sum = __fadd_rn(sum, __shfl_xor_sync(~0u, sum, 4));
             const float c0 = __shfl_sync(~0u, sum, 0), c1 = __shfl_sync(~0u, sum, 8);
             const float c2 = __shfl_sync(~0u, sum, 16), c3 = __shfl_sync(~0u, sum, 24);
-            if (lane == 0 && valid && p.gw_part) {
-                float gw = 0.f;
-                gw = __fadd_rn(gw, c0);
-                gw = __fadd_rn(gw, c1);
-                gw = __fadd_rn(gw, c2);
-                gw = __fadd_rn(gw, c3);
-                p.gw_part[(size_t)(p0 + prow) * nt + t.n_tile] = gw;
-            }
+            if (lane == 0 && valid && p.gw_part)
+                *reinterpret_cast<float4 *>(p.gw_part + (size_t)(p0 + prow) * (p.I / 32) + t.n0 / 32) =
+                    make_float4(c0, c1, c2, c3);
         }
     }
 }
@@ -1160,25 +1111,19 @@ const bf16 *pool_tensor(const Ctx &c, const RowsGroups &g, const bf16 *const *w,
     return g.shared_T ? w[2] : w[q];
 }
 
-cudaError_t run_rows(const Ctx &c, const RowsParams &p, const RowsMaps &maps)
-{
-    static std::atomic<int> smem_limit[64];
-    cudaError_t err = ensure_dynamic_smem(bwd_rows_tc_kernel, kDynSmem, smem_limit);
-    if (err != cudaSuccess) return err;
-    return launch_pdl(bwd_rows_tc_kernel, dim3(c.num_sms), dim3(kThreads), kDynSmem, c.stream, p, maps);
-}
-
-// C = A B on CTA pairs: A [a_rows][K] K-major, the weights' maps filled in.
-cudaError_t run_pairs(const Ctx &c, RowsParams &p, PairMaps &maps, const bf16 *a, uint64_t a_rows, bf16 *out)
+// A launch on CTA pairs: the rows' operand A [a_rows][K] K-major, the
+// weights' maps filled in.
+template <bool kGU>
+cudaError_t run_pairs(const Ctx &c, RowsParams &p, PairMaps &maps, const bf16 *a, uint64_t a_rows, const PairOut &out)
 {
     for (int b = 0; b < kTokBoxes; ++b)
         if (!encode_2d(&maps.tok[b], a, p.K, a_rows, 128u >> b)) return cudaErrorInvalidValue;
-    p.idesc = make_idesc_major(2 * BM, 0, true, false);  // N added per tile
+    p.idesc = kGU ? make_idesc(2 * BM, 0) : make_idesc_major(2 * BM, 0, true, false);  // N added per tile
     static std::atomic<int> smem_limit[64];
-    cudaError_t err = ensure_dynamic_smem(bwd_rows_pair_kernel, kPairDynSmem, smem_limit);
+    cudaError_t err = ensure_dynamic_smem(bwd_rows_pair_kernel<kGU>, kPairDynSmem, smem_limit);
     if (err != cudaSuccess) return err;
-    return launch_cluster_pdl(bwd_rows_pair_kernel, 2, dim3(c.num_sms / 2 * 2), dim3(kThreads), kPairDynSmem, c.stream, p,
-                              out, maps);
+    return launch_cluster_pdl(bwd_rows_pair_kernel<kGU>, 2, dim3(c.num_sms / 2 * 2), dim3(kThreads), kPairDynSmem, c.stream,
+                              p, out, maps);
 }
 
 }  // namespace
@@ -1199,7 +1144,7 @@ cudaError_t launch_rows_z(const Ctx &c, const RowsGroups &g, const bf16 *d, uint
         const bf16 *w = pool_tensor(c, g, c.down, q, s.H, &rows);
         ok &= encode_3d_blocks(&maps.w0[q], w, s.I, rows, 64, 2);
     }
-    return ok ? run_pairs(c, p, maps, d, d_rows, zpad) : cudaErrorInvalidValue;
+    return ok ? run_pairs<false>(c, p, maps, d, d_rows, PairOut{zpad, nullptr, {}, {}}) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_rows_gu(const Ctx &c, const RowsGroups &g, const bf16 *a, uint64_t a_rows, const bf16 *zpad,
@@ -1207,38 +1152,32 @@ cudaError_t launch_rows_gu(const Ctx &c, const RowsGroups &g, const bf16 *a, uin
 {
     const Shape &s = c.s;
     RowsParams p = rows_params(c, g);
-    if (c.saved_gu) {  // the forward saved the G | U accumulators of these rows
-        p.K = s.H; p.N = s.I; p.bn = 128;
-        p.zpad = zpad;
-        p.gw_part = gw_part;
-        p.wact = wact ? 1 : 0;
-        return launch_pdl(bwd_swiglu_saved_kernel, dim3(c.num_sms * 8), dim3(256), 0, c.stream, p,
-                          (const float *)c.saved_gu, dgu, wact);
-    }
-    RowsMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    p.K = s.H; p.N = s.I; p.bn = 128;
-    p.a_rows = kArowsSlot;
-    // last group first: the Z launch before ended on the last groups, whose
-    // rows are still in L2, and the launch after starts on the first groups,
-    // whose operands this one read last
-    p.reverse = 1;
+    p.K = s.H; p.N = s.I;
     p.zpad = zpad;
     p.gw_part = gw_part;
     p.wact = wact ? 1 : 0;
-    p.idesc = make_idesc(BM, 256);
-    bool ok = encode_2d(&maps.a, a, s.H, a_rows, BM);
+    if (c.saved_gu)  // the forward saved the G | U accumulators of these rows
+        return launch_pdl(bwd_swiglu_saved_kernel, dim3(c.num_sms * 8), dim3(256), 0, c.stream, p,
+                          (const float *)c.saved_gu, dgu, wact);
+    PairMaps maps;
+    memset(&maps, 0, sizeof(maps));
+    p.a_rows = kArowsSlot;
+    PairOut out{dgu, wact, {}, {}};
+    bool ok = true;
     for (int q = 0; q < (g.shared_T ? 1 : 2); ++q) {
         uint64_t rows;
         const bf16 *wg = pool_tensor(c, g, c.gate, q, s.I, &rows);
         const bf16 *wu = pool_tensor(c, g, c.up, q, s.I, &rows);
-        ok &= encode_2d(&maps.b0[q], wg, s.H, rows, 128);
-        ok &= encode_2d(&maps.b1[q], wu, s.H, rows, 128);
+        bool up_first;
+        if (encode_gate_up(&maps.gu[q], wg, wu, s.H, rows, &up_first)) {
+            out.up_first[q] = up_first;
+        } else {
+            out.two_boxes[q] = 1;
+            ok &= encode_2d(&maps.w0[q], wg, s.H, rows, 64);
+            ok &= encode_2d(&maps.w1[q], wu, s.H, rows, 64);
+        }
     }
-    ok &= encode_2d_box(&maps.out0, dgu, 2 * (uint64_t)s.I, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    if (wact) ok &= encode_2d_box(&maps.out1, wact, s.I, g.padded_rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    if (!ok) return cudaErrorInvalidValue;
-    return run_rows(c, p, maps);
+    return ok ? run_pairs<true>(c, p, maps, a, a_rows, out) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_rows_da(const Ctx &c, const RowsGroups &g, const bf16 *dgu, bf16 *da)
@@ -1258,7 +1197,7 @@ cudaError_t launch_rows_da(const Ctx &c, const RowsGroups &g, const bf16 *dgu, b
         ok &= encode_3d_blocks(&maps.w0[q], wg, s.H, rows, 64, 2);
         ok &= encode_3d_blocks(&maps.w1[q], wu, s.H, rows, 64, 2);
     }
-    return ok ? run_pairs(c, p, maps, dgu, g.padded_rows, da) : cudaErrorInvalidValue;
+    return ok ? run_pairs<false>(c, p, maps, dgu, g.padded_rows, PairOut{da, nullptr, {}, {}}) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_backward_rows(const Ctx &c, const bf16 *dout_rows, bf16 *zpad, bf16 *dgu, bf16 *wact,

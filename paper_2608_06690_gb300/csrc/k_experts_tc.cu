@@ -1495,12 +1495,9 @@ bool fill_phase(const Ctx &c, int mode, TcParams &p, TcMaps &maps)
             ok &= encode_2d(&maps.down[q], c.down[q], s.I, n * s.H, 128);
             continue;
         }
-        p.up_first[q] = c.up[q] < c.gate[q];
-        const bf16 *lo = p.up_first[q] ? c.up[q] : c.gate[q], *hi = p.up_first[q] ? c.gate[q] : c.up[q];
-        const uint64_t apart = (uint64_t)((uintptr_t)hi - (uintptr_t)lo);
-        // a tensor map's strides are below 2^40 bytes (one tensor as both: two boxes)
-        p.gu_two_boxes[q] = apart == 0 || apart >= (1ull << 40) ||
-                            !encode_3d_two(&maps.gu[q], lo, s.H, n * s.I, apart, 64);
+        bool up_first;
+        p.gu_two_boxes[q] = !encode_gate_up(&maps.gu[q], c.gate[q], c.up[q], s.H, n * s.I, &up_first);
+        p.up_first[q] = up_first;
         if (p.gu_two_boxes[q]) {
             p.up_first[q] = 0;
             ok &= encode_2d(&maps.gate[q], c.gate[q], s.H, n * s.I, 64);
@@ -1775,15 +1772,18 @@ bool encode_3d_blocks(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t r
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool encode_3d_two(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows, uint64_t apart, uint32_t box_rows)
+bool encode_gate_up(CUtensorMap *m, const bf16 *gate, const bf16 *up, uint64_t cols, uint64_t rows, bool *up_first)
 {
+    *up_first = up < gate;
+    const bf16 *lo = *up_first ? up : gate, *hi = *up_first ? gate : up;
+    const uint64_t apart = (uint64_t)((uintptr_t)hi - (uintptr_t)lo);
     auto fn = encode_fn();
-    if (!fn) return false;
+    if (!fn || apart == 0 || apart >= (1ull << 40)) return false;  // a map's strides are below 2^40 bytes
     const cuuint64_t dims[3] = {cols, rows, 2};
     const cuuint64_t strides[2] = {cols * 2, apart};
-    const cuuint32_t box[3] = {64, box_rows, 2};
+    const cuuint32_t box[3] = {64, 64, 2};
     const cuuint32_t estr[3] = {1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, estr,
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16 *>(lo), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

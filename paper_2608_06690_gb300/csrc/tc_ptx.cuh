@@ -172,6 +172,15 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uin
                  "r"(c), "r"(d)
                  : "memory");
 }
+// The reverse: four 8 x 8 BF16 matrices read by 16-byte rows and transposed into
+// the mma fragment layout.
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(addr)
+                 : "memory");
+}
 // 16 bytes to global memory with an L2 cache policy.
 __device__ __forceinline__ void st_global_hint(void *ptr, const uint4 &v, uint64_t policy)
 {
@@ -505,10 +514,12 @@ bool encode_2d_f32(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows
 // [box_rows][64] tiles one after another (the layout of an MN-major operand
 // whose MN blocks are box_rows * 128 bytes apart).
 bool encode_3d_blocks(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows, uint32_t box_rows, uint32_t nblocks);
-// 3-D BF16 tensor map over two row-major [rows, cols] matrices `apart` bytes
-// apart (the first at ptr): a box of 64 columns x box_rows rows of both, one
-// after the other, 128-byte swizzle.
-bool encode_3d_two(CUtensorMap *m, const void *ptr, uint64_t cols, uint64_t rows, uint64_t apart, uint32_t box_rows);
+// 3-D BF16 tensor map over the gate and up weights, two row-major [rows, cols]
+// matrices anywhere in memory (one dimension steps from the lower to the
+// higher): a box of 64 columns x 64 rows of both, one after the other, 128-byte
+// swizzle, the up rows first when *up_first.  False where a map cannot hold
+// both (one tensor as both, or 2^40 bytes apart).
+bool encode_gate_up(CUtensorMap *m, const bf16 *gate, const bf16 *up, uint64_t cols, uint64_t rows, bool *up_first);
 // tcgen05 instruction descriptor: BF16 x BF16 -> FP32, both operands K-major.
 uint32_t make_idesc(int M, int N);
 // The same with either operand MN-major (transpose bits 15 for A, 16 for B).
