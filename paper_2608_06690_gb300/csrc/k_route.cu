@@ -607,7 +607,7 @@ constexpr int kCMaxStages = 6;
 
 struct ClusterRouterParams {
     int T, H, E_pub, E_priv, k, renorm;
-    int nq;              // CTAs per cluster: H is split into nq ranges
+    int nq;              // CTAs per cluster: H is split into nq ranges (1: two ranges of one CTA)
     int slots4;
     uint32_t idesc;      // M = 128, N = 128
     const uint8_t *policy;
@@ -951,55 +951,63 @@ __global__ void __launch_bounds__(kCThreads, 1) router_cluster_kernel(const Clus
     tc_fence_after();
     const uint32_t tmem = s_tmem;
 
-    if (warp == 0) {
-        if (lane < (contiguous ? 2 : 1)) {
-            // ---- TMA: lane 0 the router rows of this CTA's range of H, lane 1
-            // the token rows when the tile's tokens are consecutive (a thread's
-            // boxes are processed one after another: two lanes, two streams)
-            const uint32_t tx = lane == 0 ? a_bytes : 16384u;
-            uint32_t filled = 0, last_parity = 0;
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int st = kb % stages;
-                const uint32_t ph = (uint32_t)(kb / stages) & 1u;
-                if (!mbar_wait(empty_bar(st), ph ^ 1u, &s_abort, p.status)) break;
-                const uint32_t sA = sbase + st * stage_bytes, sB = sA + a_bytes;
+    // ---- TMA: warp 0 the router rows of this CTA's range of H; warp 2 the token
+    // rows when the tile's tokens are consecutive (two issuing warps, two streams)
+    auto load_tiles = [&](bool router) {
+        const uint32_t tx = router ? a_bytes : 16384u;
+        int kb = 0;
+        for (; kb < nkb; ++kb) {
+            const int st = kb % stages;
+            if (!__all_sync(~0u, mbar_wait(empty_bar(st), ((uint32_t)(kb / stages) & 1u) ^ 1u, &s_abort, p.status))) break;
+            const uint32_t sA = sbase + st * stage_bytes;
+            if (elect_one()) {
                 mbar_expect_tx(full_bar(st), tx);
-                if (lane == 0) {
+                if (router) {
                     for (int mi = 0; mi < nm; ++mi)
                         tma_load_2d(sA + mi * 16384u, &maps.router[pool], full_bar(st), k0 + kb * 64, mi * 128);
                 } else {
-                    tma_load_2d(sB, &maps.hidden, full_bar(st), k0 + kb * 64, s_tok[0]);
+                    tma_load_2d(sA + a_bytes, &maps.hidden, full_bar(st), k0 + kb * 64, s_tok[0]);
                 }
-                filled |= 1u << st;
-                last_parity = (last_parity & ~(1u << st)) | (ph << st);
             }
-            for (int st = 0; st < stages; ++st)
-                if ((filled >> st) & 1u) {
-                    const unsigned long long w0 = globaltimer_ns();
-                    while (!mbar_try_wait(full_bar(st), (last_parity >> st) & 1u))
-                        if (globaltimer_ns() - w0 > kWaitLimitNs) break;
-                }
         }
+        for (int b = max(0, kb - stages); b < kb; ++b) {  // the last use of each stage has landed
+            const unsigned long long w0 = globaltimer_ns();
+            while (!mbar_try_wait(full_bar(b % stages), (uint32_t)(b / stages) & 1u))
+                if (globaltimer_ns() - w0 > kWaitLimitNs) break;
+        }
+    };
+
+    if (warp == 0) {
+        load_tiles(true);
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---- MMA: logits[128 experts, 128 tokens] += router x rows^T per stage
-            bool ok = true;
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int st = kb % stages;
-                const uint32_t ph = (uint32_t)(kb / stages) & 1u;
-                if (!mbar_wait(full_bar(st), ph, &s_abort, p.status)) { ok = false; break; }
-                tc_fence_after();
-                fence_proxy_async_smem();  // gathered rows (generic proxy) read by the tensor cores
-                const uint32_t sA = sbase + st * stage_bytes, sB = sA + a_bytes;
-                const uint64_t bd = sw128_desc(sB);
+        // ---- MMA: logits[128 experts, 128 tokens] += router x rows^T per stage
+        // (one CTA alone: the second half of H into columns of its own)
+        const int half = p.nq == 1 ? nkb / 2 : nkb;
+        bool ok = true;
+        for (int kb = 0; kb < nkb; ++kb) {
+            const int st = kb % stages;
+            if (!__all_sync(~0u, mbar_wait(full_bar(st), (uint32_t)(kb / stages) & 1u, &s_abort, p.status))) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            fence_proxy_async_smem();  // gathered rows (generic proxy) read by the tensor cores
+            const uint32_t acc = tmem + (kb >= half ? 128u : 0u);
+            const uint32_t sA = sbase + st * stage_bytes;
+            const uint64_t bd = sw128_desc(sA + a_bytes);
+            const uint32_t add = kb != 0 && kb != half;
+            if (elect_one()) {
                 for (int mi = 0; mi < nm; ++mi) {
                     const uint64_t ad = sw128_desc(sA + mi * 16384u);
 #pragma unroll
                     for (int k4 = 0; k4 < 4; ++k4)
-                        tc_mma(tmem + (uint32_t)(mi * 128), ad + 2 * k4, bd + 2 * k4, p.idesc, (kb | k4) != 0);
+                        tc_mma(acc + (uint32_t)(mi * 128), ad + 2 * k4, bd + 2 * k4, p.idesc, add | (k4 != 0));
                 }
                 tc_commit(empty_bar(st));
             }
+            __syncwarp();
+        }
+        if (elect_one()) {
             if (ok) tc_commit(tfull_bar);
             tc_commit(done_bar);
             const unsigned long long w0 = globaltimer_ns();
@@ -1037,6 +1045,8 @@ __global__ void __launch_bounds__(kCThreads, 1) router_cluster_kernel(const Clus
                 cp_async_arrive_noinc(full_bar(st));
             }
             cp_async_wait<0>();
+        } else if (warp == 2) {
+            load_tiles(false);
         }
         // ---- epilogue: the partial logits to shared memory, [token][expert]
         // FP32 (chunks of 32 experts at a stride of kChunkPitch; the ring is
@@ -1053,8 +1063,17 @@ __global__ void __launch_bounds__(kCThreads, 1) router_cluster_kernel(const Clus
                 const int e = mi * 128 + quarter * 32 + lane;
                 for (int cc = 0; cc < kCTile / 32; ++cc) {
                     float v[32];
-                    tmem_ld32(tmem + (uint32_t)(mi * 128 + cc * 32) + ((uint32_t)(quarter * 32) << 16), v);
-                    tmem_ld_wait();
+                    const uint32_t ta = tmem + (uint32_t)(mi * 128 + cc * 32) + ((uint32_t)(quarter * 32) << 16);
+                    tmem_ld32(ta, v);
+                    if (p.nq == 1) {
+                        float v2[32];
+                        tmem_ld32(ta + 128, v2);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] += v2[i];
+                    } else {
+                        tmem_ld_wait();
+                    }
 #pragma unroll
                     for (int i = 0; i < 32; ++i) S[(cc * 32 + i) * pitch + chunk_pos(e)] = v[i];
                 }
@@ -1324,9 +1343,13 @@ static cudaError_t launch_route_chunked(const Ctx &c)
 // once, so that each CTA's share of H fits its ring in one round; else 4 (2
 // when H is not a multiple of 256); and 2 when clusters of 4 would not fit
 // the GPU in one wave (one wave of clusters of 2 measured faster than two
-// waves of clusters of 4: 35 vs 57 us at T = 8192).
-static int cluster_router_nq(int H, int T, int num_sms)
+// waves of clusters of 4: 35 vs 57 us at T = 8192).  When clusters of 2 would
+// not either, one CTA takes the tile and adds the two halves of H that a
+// cluster of 2 adds, in the same order (T = 16384: the router alone 63 -> 49 us); for pools of at
+// most 128, whose two accumulators fit the CTA's TMEM.
+static int cluster_router_nq(int H, int T, int P, int num_sms)
 {
+    if (router_slots(T) * 2 > num_sms && P <= 128) return 1;
     if (H % 512 == 0 && router_slots(T) * 8 <= num_sms) return 8;
     if (router_slots(T) * 4 > num_sms) return 2;
     return H % 256 == 0 ? 4 : 2;
@@ -1338,7 +1361,7 @@ bool route_uses_cluster_kernel(const Shape &s, int unmasked, int num_sms)
 {
     if (unmasked) return false;
     const int P = s.E_pub > s.E_priv ? s.E_pub : s.E_priv;
-    return cluster_router_smem(P, s.k, cluster_router_nq(s.H, s.T, num_sms)) <= kCMaxDynSmem;
+    return cluster_router_smem(P, s.k, cluster_router_nq(s.H, s.T, P, num_sms)) <= kCMaxDynSmem;
 }
 
 bool route_writes_dispatch(const Ctx &c)
@@ -1355,7 +1378,8 @@ cudaError_t launch_route(const Ctx &c, bool write_dispatch)
     memset(&p, 0, sizeof(p));
     memset(&maps, 0, sizeof(maps));
     p.T = s.T; p.H = s.H; p.E_pub = s.E_pub; p.E_priv = s.E_priv; p.k = s.k; p.renorm = s.renorm;
-    p.nq = cluster_router_nq(s.H, s.T, c.num_sms);
+    const int P = s.E_pub > s.E_priv ? s.E_pub : s.E_priv;
+    p.nq = cluster_router_nq(s.H, s.T, P, c.num_sms);
     p.slots4 = router_slots4(s.T);
     p.idesc = make_idesc(128, kCTile);
     p.policy = c.policy;
@@ -1384,7 +1408,6 @@ cudaError_t launch_route(const Ctx &c, bool write_dispatch)
     ok &= encode_2d(&maps.router[0], c.router_pub, s.H, s.E_pub, 128);
     ok &= encode_2d(&maps.router[1], c.router_priv, s.H, s.E_priv, 128);
     if (!ok) return cudaErrorInvalidValue;
-    const int P = s.E_pub > s.E_priv ? s.E_pub : s.E_priv;
     const int smem = cluster_router_smem(P, s.k, p.nq);
     static std::atomic<int> smem_limit[64];
     cudaError_t err = ensure_dynamic_smem(router_cluster_kernel, smem, smem_limit);
