@@ -48,12 +48,14 @@
 // each thread's copies of a stage arrive on a barrier when they complete
 // (cp.async.mbarrier.arrive): the leader's on the stage's full barrier; the
 // other CTA's on one of its own, where its warp 0 waits, fences the async proxy
-// and arrives on the leader's.
+// and arrives on the leader's.  With in-launch routing (at most 128 tokens) TMA
+// gather4 copies of four rows take their place, which complete on the leader's
+// full barrier like any other (see kGatherGroups).
 //
-// CTA roles (480 threads):
+// CTA roles (480 threads; 256 with in-launch routing):
 //   warp 0       hands out the tiles (leader) and loads the token rows that
 //                come through TMA (activations or, for the shared group, hidden
-//                states), completing on the leader's barrier
+//                states; with in-launch routing half of the gathered ones)
 //   warp 1       allocates 512 TMEM columns (two accumulators of 256 columns,
 //                so the epilogue of one tile overlaps the MMAs of the next);
 //                the leader's issues tcgen05.mma M = 256, K = 16
@@ -66,9 +68,10 @@
 //                mode the tiles of weight block 0 also write the execution audit,
 //                each row checked against the route log of its token
 //   warps 6..13  the row gather of the routed gate/up tiles (cp.async), two
-//                groups of four warps taking turns
-//   warp 14      the weights through TMA, two 64-row boxes a stage
-// Warps 0, 1 and 14 run their loops as whole warps and issue TMA and MMA
+//                groups of four warps taking turns; with in-launch routing
+//                warp 6 alone, the other half of the rows by gather4
+//   the last     the weights through TMA
+// The issuing warps run their loops as whole warps and issue TMA and MMA
 // instructions from one elected lane.
 // Expert weights that only one tile reads stream through L2 (evict first);
 // the hidden states and activations, read again by other tiles of the launch,
@@ -97,12 +100,20 @@ constexpr int kRingBytes = 6 * 2 * kWBytes;   // 6 stages at N = 256
 constexpr int kMaxStages = 10;                // at N = 32: 18 KB each
 constexpr int kAccCols = kMaxN;               // FP32 TMEM columns per accumulator
 constexpr int kTmemCols = 2 * kAccCols;
-constexpr int kGatherGroups = 2;              // the row gather: groups of four warps, every other stage each
-constexpr int kGatherWarps = 4 * kGatherGroups;  // warps 6..13
-constexpr int kWeightWarp = 6 + kGatherWarps;
-constexpr int kThreads = 192 + 32 * kGatherWarps + 32;
-constexpr int kGatherThreads = 128;           // of a group: the arrivals of a gathered stage
-constexpr int kFullArrivals = 3 + kGatherThreads;  // the leader's token and weight loaders and gather, the other CTA's gather
+// The row gather of the routed gate/up tiles: with in-launch routing (at most
+// 128 tokens) TMA gather4 copies of four rows, issued by warp 0 and one more;
+// else groups of four warps with cp.async, every other stage each.  (gather4
+// takes about 43 clocks for four rows: one token's step 48 -> 44.5 us and a
+// decode step of 96 tokens 224 -> 220 us with it, but 32 of them a stage
+// took the gate/up GEMM at T = 16384 from 527 to 1,037 us.)
+constexpr int kGatherGroups = 2;
+constexpr int kGatherWarp = 6;                // the first of the gather's warps
+template <bool kRoute> constexpr int kGatherWarps = kRoute ? 1 : 4 * kGatherGroups;
+template <bool kRoute> constexpr int kTcThreads = 192 + 32 * kGatherWarps<kRoute> + 32;
+constexpr int kGatherThreads = 128;           // of a cp.async group: the arrivals of a gathered stage
+// Arrivals of a ring stage: the leader's token and weight loaders; with cp.async
+// the leader's gather and the other CTA's.
+template <bool kRoute> constexpr int kFullArrivals = kRoute ? 2 : 3 + kGatherThreads;
 constexpr int kMaxGroups = 2 * kMaxPool + 1;
 constexpr int kPrefetchTiles = 96;            // gate/up tiles (1 MB of weights each) prefetched into L2 at small batches
 // Large batches, the launch following the router: the gate and up weights of
@@ -114,8 +125,9 @@ constexpr int kPrefillPrefetchExperts = 16;
 constexpr unsigned long long kPrefillPrefetchDelayNs = 14000;
 constexpr int kTQ = 8;                        // tile queue entries (tile indices handed to the pair's roles)
 constexpr int kHandOutStages = 8;             // K steps before a tile's last at which the next tile is handed out
-constexpr int kTQConsumers = 2 + 4 + kGatherWarps       // leader: MMA, weight, epilogue and gather warps (one lane each)
-                             + 2 + 4 + kGatherWarps;    // other CTA: both loaders, epilogue, gather
+// Readers of a queue entry (one lane each): the leader's MMA, weight, epilogue
+// and gather warps; the other CTA's token, weight, epilogue and gather warps.
+template <bool kRoute> constexpr int kTQConsumers = 2 * (2 + 4 + kGatherWarps<kRoute>);
 constexpr int kStageOutBytes = 4096;          // per epilogue warp: two 2 KB exchange / transpose buffers
 constexpr int kRowWBytes = kMaxN * 4;         // per epilogue warp: the tile's routing weights
 constexpr int kDynSmem = kRingBytes + 4 * (kStageOutBytes + kRowWBytes) + 1024 /* alignment slack */;
@@ -201,6 +213,7 @@ struct TcMaps {
     // 3-D box of both tensors (one dimension steps from one to the other), or
     // (p.gu_two_boxes) 64-row boxes of each; down, 128-row boxes
     CUtensorMap gu[3], gate[3], up[3], down[3];
+    CUtensorMap hidden;        // the hidden states, one-row boxes (gather4)
     CUtensorMap tok[2][kTokBoxes];     // per GEMM, by box rows: the shared group's hidden states; the activations
     CUtensorMap tok_sh[kTokBoxes];     // the shared group's activations
 };
@@ -405,7 +418,7 @@ __device__ bool route_in_launch(const TcParams &p, uint8_t *ring, TileTable &tt,
     __shared__ uint8_t s_tau[kRouteMaxTokens];
     __shared__ int s_nd;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    constexpr int kWarps = kThreads / 32;
+    constexpr int kThreads = kTcThreads<true>, kWarps = kThreads / 32;
     const int T = p.T, K = p.k, E = p.E, E_priv = p.E - p.E_pub, R = p.R;
     // ---- tau per token (Sec. 2.1) and the logit work items: (token, block
     // of bs experts of its pool), bs the least size from 32 up that gives
@@ -647,8 +660,9 @@ constexpr size_t fused_dispatch_smem(int E, int slots) { return (size_t)E * (siz
 // kRoute: the instantiation that can route the tokens itself (p.fuse_route);
 // the other one carries none of that code (fewer registers, a smaller body).
 template <bool kRoute>
-__global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcParams p, const __grid_constant__ TcMaps maps)
+__global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(const TcParams p, const __grid_constant__ TcMaps maps)
 {
+    constexpr int kThreads = kTcThreads<kRoute>, kWeightWarp = kGatherWarp + kGatherWarps<kRoute>;
     extern __shared__ uint8_t dsmem[];
     __shared__ TileTable tt;
     __shared__ __align__(8) uint64_t bars[3 * kMaxStages + 5 + 2 * kTQ];
@@ -715,13 +729,13 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
 
     if (tid == 0) {
         for (int s = 0; s < kMaxStages; ++s) {
-            mbar_init(full_bar(s), kFullArrivals);
+            mbar_init(full_bar(s), kFullArrivals<kRoute>);
             mbar_init(empty_bar(s), 1);
             mbar_init(gfull_bar(s), kGatherThreads);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
         mbar_init(done_bar, 1);
-        for (int i = 0; i < kTQ; ++i) { mbar_init(tq_full_bar(i), 1); mbar_init(tq_empty_bar(i), kTQConsumers); }
+        for (int i = 0; i < kTQ; ++i) { mbar_init(tq_full_bar(i), 1); mbar_init(tq_empty_bar(i), kTQConsumers<kRoute>); }
         s_abort = 0;
         s_pdl_done = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -906,6 +920,30 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
         return __all_sync(~0u, mbar_wait(bar, parity, &s_abort, p.status));
     };
 
+    // gather4 (kRoute): this CTA's half of a gathered tile's token rows, half
+    // `part` of that by warp 0 (0) and by the gather warp (1).  load_rows keeps the
+    // rows' token ids (rows past the tile's read token 0, whose columns are not
+    // stored).
+    __shared__ __align__(16) int s_rows[kRoute ? 2 : 1][kRoute ? kMaxN / 4 : 4];
+    auto load_rows = [&](const Tile &t, int part) {
+        const int n4 = t.n() / 4, first = rank * (t.n() / 2) + part * n4;
+        __syncwarp();
+        for (int i = lane; i < n4; i += 32) {
+            const int tok = first + i < t.rows ? p.tok_of_slot[t.row_base + t.m0 + first + i] : 0;
+            s_rows[part][i] = (unsigned)tok < (unsigned)p.T ? tok : 0;
+        }
+        __syncwarp();
+    };
+    auto gather_stage = [&](int stage, int kb, int ng, int part) {
+        const uint32_t dst = sbase + stage * stage_bytes + kWBytes + part * ng * 512;
+        const uint32_t fb = dsmem_addr(full_bar(stage), 0), ids = smem_u32(s_rows[part]);
+#pragma unroll 4
+        for (int g = 0; g < ng; ++g) {
+            const uint4 r = ld_shared_v4(ids + g * 16);
+            tma_gather4_pair(dst + g * 512, &maps.hidden, fb, kb * BK, (int)r.x, (int)r.y, (int)r.z, (int)r.w, pol_keep);
+        }
+    };
+
     if (warp == 0) {
         // ------------------------------------------------ tile hand-out, token rows through TMA
         // This CTA's half of the tile's token rows when they come through TMA
@@ -963,6 +1001,10 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
             const int tn = t.n(), trows = tn / 2;  // this CTA's token rows
             const int trow = t.row_base + t.m0 + rank * trows;
             int ok = 1;
+            if (kRoute && gather && lane == 0) {  // the slot maps are read here
+                if (!synced) synced = wait_dispatch();
+                ok = synced;
+            }
             if (t.down() && p.has_gu && lane == 0) {
                 // a down tile after the gate/up tiles of the same launch: its
                 // activation rows are complete once every gate/up epilogue
@@ -996,6 +1038,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
             const int b1 = trows > r0 ? __clz(trows - r0) - 24 : -1, r1 = b1 < 0 ? 0 : r0 + (128 >> b1);
             const int b2 = b1 >= 0 && trows > r1 ? __clz(trows - r1) - 24 : -1;
             const int hand_out = max(t.nkb - kHandOutStages, 1);
+            if (kRoute && gather) load_rows(t, 0);
             int kb = 0;
 #pragma unroll 1
             for (int part = 0; part < 2 && ok; ++part) {
@@ -1004,7 +1047,15 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
                     next = decode_tile(p, tt, G, (int)min(__shfl_sync(~0u, ahead, 0), (uint32_t)total), total, lane);
                     push(qi + 1, next);
                 }
-                if (gather && rank == 1) {
+                if (kRoute && gather) {
+                    for (; kb < end; ++kb, advance()) {
+                        if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = 0; break; }
+                        if (elect_one()) {
+                            if (rank == 0) mbar_expect_tx(full_bar(stage), (uint32_t)(tn * BK * 2));
+                            gather_stage(stage, kb, tn / 16, 0);
+                        }
+                    }
+                } else if (gather && rank == 1) {
                     for (; kb < end; ++kb, advance()) {
                         if (!warp_wait(gfull_bar(stage), phase)) { ok = 0; break; }
                         if (elect_one()) {
@@ -1025,7 +1076,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
                             const uint32_t fb = dsmem_addr(full_bar(stage), 0);
                             if (rank == 0) {
                                 mbar_expect_tx(full_bar(stage), (uint32_t)(tn * BK * 2));
-                                mbar_arrive_count(full_bar(stage), 1 + kGatherThreads);  // nothing is gathered
+                                if (!kRoute) mbar_arrive_count(full_bar(stage), 1 + kGatherThreads);  // nothing is gathered
                             }
                             tma_load_2d_pair_hint(sT, &tmap[b0], fb, kb * BK, trow, pol_keep);
                             if (b1 >= 0) tma_load_2d_pair_hint(sT + r0 * 128, &tmap[b1], fb, kb * BK, trow + r0, pol_keep);
@@ -1050,9 +1101,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
     } else if (warp == kWeightWarp) {
         // ------------------------------------------------ weights through TMA
         // One 16 KB box a stage: 64 gate and 64 up rows, or 128 output columns'
-        // rows.  (A box costs the TMA unit about 180 clocks whatever its rows:
-        // as two boxes beside the tokens' one, a stage took 540 clocks even
-        // with every operand in L2.  The drain above covers these copies.)
+        // rows.  (The drain above covers these copies.)
         int stage = 0;
         uint32_t phase = 0;
         int ok = 1;
@@ -1112,7 +1161,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
                 // rows this CTA's gather warps copied (generic proxy, complete
                 // when the barrier's phase completed) are read by the tensor
                 // cores through the async proxy
-                if (gather) fence_proxy_async_smem();
+                if (!kRoute && gather) fence_proxy_async_smem();
                 tc_fence_after();
                 const uint32_t eb = empty_bar(stage);
                 const uint32_t sW = sbase + stage * stage_bytes;
@@ -1356,7 +1405,23 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
                 __syncwarp();
             }
         }
-    } else if (warp >= 6 && warp < kWeightWarp) {
+    } else if (kRoute && warp == kGatherWarp) {
+        // ------------------------------------------------ gather4 of the second half of the rows
+        int stage = 0;
+        uint32_t phase = 0;
+        int ok = 1;
+        bool synced = false;  // wait_dispatch has returned (every lane acquires)
+        Tile t;
+        for (int qi = 0; ok && next_tile(qi, t, true); ++qi) {
+            if (!synced && !(synced = __all_sync(~0u, wait_dispatch()))) break;
+            load_rows(t, 1);
+            for (int kb = 0; kb < t.nkb; ++kb) {
+                if (!warp_wait(empty_bar(stage), phase ^ 1u)) { ok = 0; break; }
+                if (elect_one()) gather_stage(stage, kb, t.n() / 16, 1);
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+            }
+        }
+    } else if (warp >= kGatherWarp && warp < kWeightWarp) {
         // ------------------------------------------------ token row gather
         // This CTA's half of a routed gate/up tile's token rows: thread i of
         // a group's 128 copies 16-byte chunk (i & 7) of rows (i >> 3) + 16 j of
@@ -1367,7 +1432,7 @@ __global__ void __launch_bounds__(kThreads, 1) expert_gemm_tc_kernel(const TcPar
         // thread's copies of a stage arrive on the leader's full barrier, or the
         // other CTA's gfull barrier, when they complete (cp.async.mbarrier.arrive), so the threads never wait for
         // their own copies: up to the whole ring is in flight.
-        const int gi = (tid - 192) & 127, group = (warp - 6) >> 2;
+        const int gi = (tid - 192) & 127, group = (warp - kGatherWarp) >> 2;
         const int chunk = gi & 7, row0 = gi >> 3;
         int stage = 0;
         uint32_t phase = 0;
@@ -1504,6 +1569,7 @@ bool fill_phase(const Ctx &c, int mode, TcParams &p, TcMaps &maps)
             ok &= encode_2d(&maps.up[q], c.up[q], s.H, n * s.I, 64);
         }
     }
+    if (gu) ok &= encode_2d(&maps.hidden, c.hidden, s.H, T, 1);
     if (gu && s.E_sh > 0) ok &= encode_tokens(maps.tok[kGateUp], c.hidden, s.H, T);
     if (!gu) ok &= encode_tokens(maps.tok[kDown], c.act, s.I, R);
     if (!gu && s.E_sh > 0) ok &= encode_tokens(maps.tok_sh, c.act_sh, s.E_sh * s.I, T);
@@ -1618,9 +1684,9 @@ cudaError_t launch_tc(const Ctx &c, bool gu, bool down, bool fuse_dispatch = fal
     const cudaError_t err = fuse_route ? ensure_tc_smem<true>() : ensure_tc_smem<false>();
     if (err != cudaSuccess) return err;
     if (fuse_route)
-        return launch_cluster_pdl(expert_gemm_tc_kernel<true>, 2, dim3(tc_grid(c)), dim3(kThreads), kDynSmem, c.stream, p,
+        return launch_cluster_pdl(expert_gemm_tc_kernel<true>, 2, dim3(tc_grid(c)), dim3(kTcThreads<true>), kDynSmem, c.stream, p,
                                   maps);
-    return launch_cluster_pdl(expert_gemm_tc_kernel<false>, 2, dim3(tc_grid(c)), dim3(kThreads), kDynSmem, c.stream, p,
+    return launch_cluster_pdl(expert_gemm_tc_kernel<false>, 2, dim3(tc_grid(c)), dim3(kTcThreads<false>), kDynSmem, c.stream, p,
                               maps);
 }
 
@@ -1633,7 +1699,7 @@ bool pairs_fit(const Ctx &c)
     if (ensure_tc_smem<kRoute>() != cudaSuccess) return false;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(tc_grid(c));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kTcThreads<kRoute>);
     cfg.dynamicSmemBytes = kDynSmem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;

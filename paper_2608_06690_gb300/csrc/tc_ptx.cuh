@@ -442,6 +442,19 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+// Four rows (y0 .. y3) of a 2-D tensor, 64 columns from x, into four consecutive
+// 128-byte rows of this CTA's shared memory (a map with one-row boxes),
+// completing on the leader's barrier.
+__device__ __forceinline__ void tma_gather4_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y0, int y1,
+                                                 int y2, int y3, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes.cta_group::2.L2::"
+        "cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "l"(policy)
+        : "memory");
+}
+
 // One warp of each CTA of the pair executes the allocation and the release.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem_addr, uint32_t ncols)
 {
