@@ -239,7 +239,8 @@ struct PairOut {
 };
 
 struct PairTable {
-    int tiles[kMaxGroups + 1];   // tiles of the groups before q
+    int tiles[kMaxGroups + 1];   // tiles of the places before L
+    uint16_t order[kMaxGroups];  // the group at place L (all routed experts: pool_place; else L)
     int rows[kMaxGroups], off[kMaxGroups], pad[kMaxGroups];  // as GroupTable
     int nmax;                    // bit b: some tile has N = 32 (b + 1)
 };
@@ -262,9 +263,10 @@ __device__ __forceinline__ int prefix_find(const int *pre, int G, int x, int lan
 __device__ __forceinline__ PairTile decode_pair(const PairTable &pt, int G, int width, int tile, int lane)
 {
     PairTile t;
-    t.q = prefix_find(pt.tiles, G, tile, lane);
+    const int L = prefix_find(pt.tiles, G, tile, lane);
+    t.q = pt.order[L];
     const int rows = pt.rows[t.q], mt = pair_row_tiles(rows), bm = pair_row_size(rows, mt);
-    const int local = tile - pt.tiles[t.q], block = local / mt;  // block major: its row tiles share the weights
+    const int local = tile - pt.tiles[L], block = local / mt;  // block major: its row tiles share the weights
     t.m0 = (local - block * mt) * bm;
     t.n0 = block * width;
     t.rows = min(bm, rows - t.m0);
@@ -273,7 +275,7 @@ __device__ __forceinline__ PairTile decode_pair(const PairTable &pt, int G, int 
 }
 
 // All threads: the table of a launch over `blocks` column blocks a group.
-__device__ void build_pairs(PairTable &pt, const uint32_t *offsets, int g0, int G, int R, int shared_T, int blocks)
+__device__ void build_pairs(PairTable &pt, const uint32_t *offsets, int g0, int G, int E_pub, int R, int shared_T, int blocks)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int p0 = shared_T ? 0 : (int)min(offsets[g0], (uint32_t)R);
@@ -290,7 +292,9 @@ __device__ void build_pairs(PairTable &pt, const uint32_t *offsets, int g0, int 
         if (mt) nmax |= 1 << (bm / 32 - 1);
         pt.rows[q] = rows;
         pt.off[q] = b - p0;
-        pt.tiles[q + 1] = mt * blocks;
+        const int L = !shared_T && g0 == 0 && interleave_pools(R, G) ? pool_place(q, E_pub, G - E_pub) : q;
+        pt.order[L] = (uint16_t)q;
+        pt.tiles[L + 1] = mt * blocks;
         pt.pad[q] = (rows + kPad - 1) / kPad * kPad;  // made exclusive prefix below
     }
     if (nmax) atomicOr(&pt.nmax, nmax);
@@ -525,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
     if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
     const int width = kGU ? 128 : 256;  // output columns of a tile
-    build_pairs(pt, p.offsets, p.g0, p.G, p.R, p.shared_T, (p.N + width - 1) / width);
+    build_pairs(pt, p.offsets, p.g0, p.G, p.E_pub, p.R, p.shared_T, (p.N + width - 1) / width);
     tc_fence_before();
     cluster_sync_all();  // both CTAs' barriers and TMEM are ready
     tc_fence_after();

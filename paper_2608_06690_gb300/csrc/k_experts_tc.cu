@@ -32,7 +32,8 @@
 //
 // The pairs walk a tile list built on the device from the dispatch offsets:
 // no host sync, and empty experts contribute no tile.  The list holds every
-// gate/up tile, then every down tile, group by group, weight-block major inside
+// gate/up tile, then every down tile, expert by expert with the pools
+// interleaved where it pays (pool_place), weight-block major inside
 // a group, so that the tiles sharing weights are next to each other.  Each pair
 // takes the next tile when its loader is ready for one (an atomic counter);
 // the leader hands it to the roles of both CTAs through a small queue in
@@ -232,7 +233,8 @@ struct __align__(16) Tile {
 };
 
 struct TileTable {
-    int prefix[2][kMaxGroups + 1];  // tiles of the groups before g, per GEMM
+    int prefix[2][kMaxGroups + 1];  // tiles of the places before L, per GEMM
+    uint16_t order[2 * kMaxPool];   // the expert at place L (pool_place, or L)
     int mpre[kMaxGroups + 1];       // row tiles of the groups before g
     int rows[kMaxGroups];
     int base[kMaxGroups];
@@ -261,7 +263,7 @@ __device__ __forceinline__ int total_tiles(const TcParams &p, const TileTable &t
     return (p.has_gu ? tt.prefix[kGateUp][G] : 0) + (p.has_down ? tt.prefix[kDown][G] : 0);
 }
 
-// The down GEMM's order of the groups: with shared experts their group sits
+// The down GEMM's order of the places: with shared experts their group sits
 // after the first half of the routed experts, so that the list ends with
 // routed down tiles (K = I) instead of the shared group's (K = E_sh I, the
 // launch's longest tiles), which otherwise made the last wave uneven; there
@@ -282,8 +284,9 @@ __device__ __forceinline__ int down_place(const TcParams &p, int g)
 }
 
 // Tile `tile` of the list (the end at `total`): the gate/up tiles (when this
-// launch runs them), then the down tiles; inside a GEMM, group by group (the
+// launch runs them), then the down tiles; inside a GEMM, place by place (the
 // down GEMM in down_group order), weight-block major.  By a whole warp.
+template <bool kRoute>
 __device__ __forceinline__ Tile decode_tile(const TcParams &p, const TileTable &tt, int G, int tile, int total, int lane)
 {
     Tile t;
@@ -296,11 +299,12 @@ __device__ __forceinline__ Tile decode_tile(const TcParams &p, const TileTable &
     const int ph = tile < n_gu ? kGateUp : kDown;
     const int local_all = tile - (ph == kDown ? n_gu : 0);
     const int *pre = tt.prefix[ph];
-    int n = 0;  // groups with prefix <= local_all; the last of them holds the tile
+    int n = 0;  // places with prefix <= local_all; the last of them holds the tile
     for (int b = 0; b < G; b += 32) n += __popc(__ballot_sync(~0u, b + lane < G && pre[b + lane] <= local_all));
     const int lo = n - 1;
-    const int g = ph == kDown ? down_group(p, lo) : lo;
-    const bool shared = g >= p.E;
+    const int L = ph == kDown ? down_group(p, lo) : lo;
+    const bool shared = L >= p.E;
+    const int g = shared ? p.E : kRoute ? L : tt.order[L];
     const int rows = tt.rows[g], mt = row_tiles(rows);
     const int local = local_all - pre[lo];
     const int block = local / mt;
@@ -321,11 +325,12 @@ __device__ __forceinline__ Tile decode_tile(const TcParams &p, const TileTable &
 // Weights of gate/up tile blockIdx.x of the list of all experts (the first
 // wave when every expert has one row tile): 128 gate rows and
 // 128 up rows, each block contiguous, prefetched into L2 by one thread.
-__device__ __forceinline__ void prefetch_first_wave(const TcParams &p)
+__device__ __forceinline__ void prefetch_first_wave(const TcParams &p, bool by_place)
 {
     const int nt = p.I / 128;
-    const int e = (int)blockIdx.x / nt, n = (int)blockIdx.x - e * nt;
-    if (e < p.E) {
+    const int L = (int)blockIdx.x / nt, n = (int)blockIdx.x - L * nt;
+    if (L < p.E) {
+        const int e = by_place ? pool_at(L, p.E_pub, p.E - p.E_pub) : L;
         const int q = e < p.E_pub ? 0 : 1;
         const size_t row0 = (size_t)(q ? e - p.E_pub : e) * p.I + (size_t)n * 128;
         const uint32_t bytes = (uint32_t)(128u * (uint32_t)p.H * 2u);
@@ -517,7 +522,7 @@ __device__ bool route_in_launch(const TcParams &p, uint8_t *ring, TileTable &tt,
     if (!grid_barrier(p.bar_a, gridDim.x, s_abort, p.status)) return false;
     // the first wave's weights into L2 while the selection and the dispatch
     // run (not earlier: the prefetch would delay the router rows)
-    if (warp == 2 && lane == 0 && (int)blockIdx.x < p.prefetch_tiles) prefetch_first_wave(p);
+    if (warp == 2 && lane == 0 && (int)blockIdx.x < p.prefetch_tiles) prefetch_first_wave(p, false);
     // ---- 2. selection, one warp per token
     if ((int)blockIdx.x < T && warp == 0) {
         const int t = (int)blockIdx.x, tau = s_tau[t];
@@ -716,6 +721,8 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
     };
 
     const int G = p.E + (p.E_sh > 0 ? 1 : 0);
+    // (in-launch routing: few rows an expert, id order)
+    const bool by_place = !kRoute && interleave_pools(p.R, p.E);
     // expert weights that one tile reads stream through L2 (evict first); the
     // hidden states, activations and per-row outputs are read again by other
     // tiles of this launch (evict last)
@@ -745,15 +752,14 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
     // weights of the first wave into L2 while the routing is computed (in
     // this launch: after this CTA's router rows have landed, which the
     // prefetch would otherwise delay)
-    if (warp == 2 && lane == 0 && (int)blockIdx.x < p.prefetch_tiles && !p.fuse_route) prefetch_first_wave(p);
+    if (warp == 2 && lane == 0 && (int)blockIdx.x < p.prefetch_tiles && !p.fuse_route) prefetch_first_wave(p, by_place);
     if (warp == 2 && lane == 0 && (int)blockIdx.x < p.prefetch_experts) {
-        // the list starts with expert 0's tiles, then expert 1's, ...: the
-        // first wave's weights, after the delay, or at once when the router
+        // the list starts with the first places' tiles: the first wave's weights, after the delay, or at once when the router
         // has already finished (thread 0 passed its wait; bounded spin)
         const unsigned long long t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < kPrefillPrefetchDelayNs && !s_pdl_done) {
         }
-        const int e = (int)blockIdx.x;
+        const int e = by_place ? pool_at((int)blockIdx.x, p.E_pub, p.E - p.E_pub) : (int)blockIdx.x;
         const int q = e < p.E_pub ? 0 : 1;
         const size_t row0 = (size_t)(q ? e - p.E_pub : e) * p.I;
         for (int r = 0; r < p.I; r += 128) {
@@ -878,8 +884,10 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
         tt.rows[g] = rows;
         tt.base[g] = base;
         tt.mpre[g + 1] = mt;
-        tt.prefix[kGateUp][g + 1] = mt * group_blocks(p, kGateUp, shared);
-        tt.prefix[kDown][down_place(p, g) + 1] = mt * group_blocks(p, kDown, shared);
+        const int L = shared ? p.E : by_place ? pool_place(g, p.E_pub, p.E - p.E_pub) : g;
+        if (!kRoute && !shared) tt.order[L] = (uint16_t)g;
+        tt.prefix[kGateUp][L + 1] = mt * group_blocks(p, kGateUp, shared);
+        tt.prefix[kDown][down_place(p, L) + 1] = mt * group_blocks(p, kDown, shared);
     }
     // the same value in every thread of every CTA (all read the same offsets)
     nmax = __reduce_or_sync(~0u, nmax);
@@ -983,7 +991,7 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
             e.flags = __shfl_sync(~0u, e.flags, 0);
         };
         if (rank == 0) {
-            t = decode_tile(p, tt, G, pair, total, lane);
+            t = decode_tile<kRoute>(p, tt, G, pair, total, lane);
             push(0, t);
         }
         for (int qi = 0;; ++qi) {
@@ -1044,7 +1052,7 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
             for (int part = 0; part < 2 && ok; ++part) {
                 const int end = part == 0 ? hand_out : t.nkb;
                 if (part == 1 && rank == 0) {
-                    next = decode_tile(p, tt, G, (int)min(__shfl_sync(~0u, ahead, 0), (uint32_t)total), total, lane);
+                    next = decode_tile<kRoute>(p, tt, G, (int)min(__shfl_sync(~0u, ahead, 0), (uint32_t)total), total, lane);
                     push(qi + 1, next);
                 }
                 if (kRoute && gather) {

@@ -79,3 +79,27 @@ def test_backward_rows_of_one_expert(T):
         err = np.abs(v.cpu().double().numpy() - ref[n])  # twice the forward's tolerance, as in the backward's tests
         assert err.max() <= 2e-2 * max(np.abs(ref[n]).max(), 1e-30), n
         assert err.sum() <= 1e-2 * max(np.abs(ref[n]).sum(), 1e-30), n
+
+
+@pytest.mark.parametrize("E_pub, E_priv", [(2, 2), (7, 3), (3, 7), (8, 1), (5, 4)])
+def test_interleaved_pools(E_pub, E_priv):
+    """At 64 rows an expert and more the GEMMs take the two pools' experts
+    interleaved: the forward and the combined backward of uneven pools against
+    the oracle and the separate passes."""
+    from paper_2608_06690_gb300 import pmpe
+    shape = LayerShape(T=700, H=256, I=128, E_pub=E_pub, E_priv=E_priv, E_sh=1, k=1, renormalize=False)
+    assert shape.T * shape.k >= 64 * shape.E
+    w, h, pol = make_layer(shape, 120 + E_pub)
+    wd, hd, pd = to_device(w, h, pol)
+    gpu = run_gpu_layer(shape, wd, hd, pd)
+    check_against_oracle(shape, w, h, pol, gpu)
+    check_audit(shape, pol, gpu)
+    check_dispatch(shape, h, gpu)
+    layer = pmpe.MoeLayer(shape, wd)
+    dout = torch.randn((shape.T, shape.H), generator=torch.Generator().manual_seed(5)).to(torch.bfloat16).cuda()
+    layer.forward(hd, pd)
+    g_sep = {n: v.clone() for n, v in layer.backward_private(hd, pd, dout).items()}
+    g, _ = layer.backward(hd, pd, dout)
+    torch.cuda.synchronize()
+    for n in g:
+        assert torch.equal(g[n], g_sep[n]), n
