@@ -53,7 +53,7 @@
 // gather4 copies of four rows take their place, which complete on the leader's
 // full barrier like any other (see kGatherGroups).
 //
-// CTA roles (480 threads; 256 with in-launch routing):
+// CTA roles (480 threads; 384 with in-launch routing):
 //   warp 0       hands out the tiles (leader) and loads the token rows that
 //                come through TMA (activations or, for the shared group, hidden
 //                states; with in-launch routing half of the gathered ones)
@@ -71,7 +71,7 @@
 //   warps 6..13  the row gather of the routed gate/up tiles (cp.async), two
 //                groups of four warps taking turns; with in-launch routing
 //                warp 6 alone, the other half of the rows by gather4
-//   the last     the weights through TMA
+//   next         the weights through TMA
 // The issuing warps run their loops as whole warps and issue TMA and MMA
 // instructions from one elected lane.
 // Expert weights that only one tile reads stream through L2 (evict first);
@@ -110,13 +110,15 @@ constexpr int kTmemCols = 2 * kAccCols;
 constexpr int kGatherGroups = 2;
 constexpr int kGatherWarp = 6;                // the first of the gather's warps
 template <bool kRoute> constexpr int kGatherWarps = kRoute ? 1 : 4 * kGatherGroups;
-template <bool kRoute> constexpr int kTcThreads = 192 + 32 * kGatherWarps<kRoute> + 32;
+// (In-launch routing: four more warps, which only take part in the routing and
+// the combine; 207.9 -> 207.0 us at T = 64.)
+template <bool kRoute> constexpr int kTcThreads = 192 + 32 * kGatherWarps<kRoute> + (kRoute ? 160 : 32);
 constexpr int kGatherThreads = 128;           // of a cp.async group: the arrivals of a gathered stage
 // Arrivals of a ring stage: the leader's token and weight loaders; with cp.async
 // the leader's gather and the other CTA's.
 template <bool kRoute> constexpr int kFullArrivals = kRoute ? 2 : 3 + kGatherThreads;
 constexpr int kMaxGroups = 2 * kMaxPool + 1;
-constexpr int kPrefetchTiles = 96;            // gate/up tiles (1 MB of weights each) prefetched into L2 at small batches
+constexpr int kPrefetchTiles = 76;            // gate/up tiles (1 MB of weights each) prefetched into L2 at small batches
 // Large batches, the launch following the router: the gate and up weights of
 // the list's first experts (at most 96 MiB, at most 16 experts) prefetched
 // into L2 while the router runs, by the CTAs that start early, after a delay
@@ -426,7 +428,7 @@ __device__ bool route_in_launch(const TcParams &p, uint8_t *ring, TileTable &tt,
     constexpr int kThreads = kTcThreads<true>, kWarps = kThreads / 32;
     const int T = p.T, K = p.k, E = p.E, E_priv = p.E - p.E_pub, R = p.R;
     // ---- tau per token (Sec. 2.1) and the logit work items: (token, block
-    // of bs experts of its pool), bs the least size from 32 up that gives
+    // of bs experts of its pool), bs the least size from 16 up that gives
     // every CTA at most one item (a CTA's item is a chain of dependent load
     // rounds, so two items on one CTA would double the step)
     __shared__ int s_bs;
@@ -440,7 +442,7 @@ __device__ bool route_in_launch(const TcParams &p, uint8_t *ring, TileTable &tt,
         }
         const int na = T - nd;
         int bs = 256;  // one item per token always fits (T <= the grid)
-        for (int b1 = 32; b1 < 256; b1 += 32) {  // the lanes test 32 sizes at a time
+        for (int b1 = 16; b1 < 256; b1 += 32) {  // the lanes test 32 sizes at a time
             const int c = b1 + lane;
             const bool fits = nd * ((p.E_pub + c - 1) / c) + na * ((E_priv + c - 1) / c) <= (int)gridDim.x;
             const unsigned m = __ballot_sync(~0u, fits);
@@ -1616,9 +1618,12 @@ cudaError_t launch_tc(const Ctx &c, bool gu, bool down, bool fuse_dispatch = fal
     p.hidden = c.hidden;
     p.ready = c.gemm_ready;
     if (gu && s.T <= kRouteMaxTokens && (long long)s.H * s.I >= (1ll << 20)) {
-        // at most T rows per expert: one row tile each (small experts, as in the tiny layer: the launch is too short to
-        // gain from it)
-        p.prefetch_tiles = std::min(s.E() * (s.I / 128), kPrefetchTiles);
+        // at most T rows per expert: one row tile each.  (Not for small experts,
+        // as in the tiny layer: the launch is too short to gain from it; and not
+        // below a pick for every five experts, when most of the prefetched weights
+        // would not be used.  Qwen3 shape: T = 1 42.8 us with it, 41.9 without;
+        // T = 4 63.2 both; T = 8 89.8 and 90.4; T = 64 211.3 and 213.8.)
+        p.prefetch_tiles = 5 * s.T * s.k >= s.E() ? std::min(s.E() * (s.I / 128), kPrefetchTiles) : 0;
         for (int q = 0; q < 2; ++q) {
             p.gate_w[q] = c.gate[q];
             p.up_w[q] = c.up[q];
