@@ -170,7 +170,8 @@ typedef struct pmpe_workspace_layout {
     size_t router_lists; /* float2 [C2*128, k] per 32-expert chunk: each token's best k (score, id) */
     size_t router_meta;  /* float4 [C2*128] per chunk: max score, sum exp(score - max), entries */
     size_t gemm_ready;   /* uint32 [(T*k+127)/128 + E + (T+127)/128 + 1]  gate/up epilogue warps done per
-                          * (expert group, 128-row block), read by the down tiles of the same launch */
+                          * (expert group, row tile of at most 256 rows), read by the down tiles of
+                          * the same launch */
     size_t tile_counts;  /* uint32 [E, S4]  rows of expert e in router tile s (S4 = S rounded up to 4).
                           * With the tiles of a pool in ascending token order, slot
                           * offsets[e] + sum_{s' < s} tile_counts[e, s'] + position gives every expert
@@ -185,7 +186,7 @@ PMPE_API int pmpe_moe_workspace_layout(int T, int H, int I, int E_pub, int E_pri
  *   [1]                  shared_rows      (token, shared expert) pairs executed
  *   [2, 2+E)             route_count[e]   rows the router sent to expert e
  *   [2+E, 2+2E)          exec_rows[e]     rows the expert kernels executed for e
- *   [2+2E, 2+3E)         exec_tiles[e]    row tiles the expert kernels ran for e
+ *   [2+2E, 2+3E)         exec_tiles[e]    128-row blocks of e's rows the expert kernels ran
  *   [2+3E, 2+3E+T)       route_priv_rows[t]  private experts in token t's route
  *   [2+3E+T, 2+3E+2T)    exec_priv_rows[t]   private expert rows executed for token t
  * The route words come from the router; the exec words are written from inside

@@ -10,6 +10,7 @@ namespace pmpe {
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// (Row tiles hold up to 256 rows; the words are counted for 128-row blocks.)
 // Each routed group adds at most one partial 128-row block beyond R/128; the
 // shared-expert group covers the T tokens.  The last two words are the expert
 // kernel's tile counter (the next tile of its list to hand out) and its grid

@@ -53,7 +53,7 @@ struct Ctx {
     float *w_of_slot;
     uint32_t *tile_done;  // [router slots] chunk CTAs finished per router tile
     uint32_t *tile_counts; // [E][router_slots4] rows of each expert per router tile
-    uint32_t *gemm_ready; // [gemm_ready_words] gate/up warps done per (group, 128-row block)
+    uint32_t *gemm_ready; // [gemm_ready_words] gate/up warps done per (group, row tile)
     float2 *router_lists; // [router CTAs * 128, k] per-chunk sorted (score, id)
     float4 *router_meta;  // [router CTAs * 128] per-chunk softmax partials
     bf16 *router_rows;  // [router CTAs * 128, H] copied token rows of non-contiguous router tiles
@@ -71,8 +71,9 @@ int router_chunks(int pool_size);
 int router_slots(int T);
 // router_slots rounded up to a multiple of 4 (the row pitch of tile_counts).
 int router_slots4(int T);
-// Readiness counters of the persistent expert GEMMs: one per (group, 128-row
-// block), an upper bound over all routings.
+// Readiness counters of the persistent expert GEMMs: one per (group, row
+// tile of at most 256 rows); sized for 128-row blocks, an upper bound over all
+// routings.
 size_t gemm_ready_words(const Shape &s);
 
 // Launchers (one per stage); each returns the launch's cudaError_t.
