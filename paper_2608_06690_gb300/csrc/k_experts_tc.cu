@@ -698,8 +698,12 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
     // Entry i of the pair's tile sequence, for a consumer role (a whole warp).
     // False at the end of the list or after an abort.
     // With gather_only (the gather warps) also at the first tile that is not
-    // gathered, after which none is: the warp then leaves every entry's
-    // barrier, so that it no longer polls beside the down tiles.
+    // gathered, after which none is: the warp then leaves the entries' barriers,
+    // so that it no longer polls beside the down tiles.  It leaves slot by slot,
+    // at this entry and the kTQ - 1 after it, once each is published: only then is
+    // its arrival on that slot due.  (A drop is also an arrival; on the slot of an
+    // earlier entry that a slower role has yet to read it would be this warp's
+    // second, and hand the slot back in that role's place.)
     auto next_tile = [&](int i, Tile &t, bool gather_only = false) -> bool {
         const int slot = i % kTQ;
         int ok = 1;
@@ -712,7 +716,15 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
         // (the vote needs every lane's entry: it is read before its slot is handed back)
         const bool live = !__any_sync(~0u, t.flags & kTileEnd) && __all_sync(~0u, t.rows > 0 && t.nkb > 0);
         if (gather_only && !t.gather()) {
-            if (lane < kTQ) mbar_arrive_drop(dsmem_addr(tq_empty_bar(lane), 0));
+            if (lane == 0) {
+                int flags = t.flags;
+                for (int e = i;;) {
+                    mbar_arrive_drop(dsmem_addr(tq_empty_bar(e % kTQ), 0));
+                    if (++e == i + kTQ || (flags & kTileEnd)) break;
+                    if (!mbar_wait(tq_full_bar(e % kTQ), (uint32_t)(e / kTQ) & 1u, &s_abort, p.status)) break;
+                    flags = (int)ld_shared_v4(smem_u32(&s_tq[e % kTQ])).x;
+                }
+            }
             return false;
         }
         if (lane == 0) {

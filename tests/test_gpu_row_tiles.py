@@ -103,3 +103,23 @@ def test_interleaved_pools(E_pub, E_priv):
     torch.cuda.synchronize()
     for n in g:
         assert torch.equal(g[n], g_sep[n]), n
+
+
+@pytest.mark.parametrize("T", [40, 129, 600])
+def test_short_tiles_round_the_queue(T):
+    """Many down tiles of two K steps after gate/up tiles of eight, at 10 stages (no
+    expert above 32 rows): the pairs go round the tile queue several times after
+    the gather warps leave it, with the loader up to five tiles ahead of the MMAs.
+    Same bits as the two GEMMs in separate launches."""
+    from paper_2608_06690_gb300 import pmpe
+    shape = LayerShape(T=T, H=512, I=128, E_pub=256, E_priv=256, E_sh=0, k=1, renormalize=True)
+    w, h, pol = make_layer(shape, 140 + T)
+    wd, hd, pd = to_device(w, h, pol)
+    layer = pmpe.MoeLayer(shape, wd)
+    split = torch.full((T, shape.H), float("nan"), dtype=torch.bfloat16, device="cuda")
+    for st in (pmpe.STAGE_ROUTE | pmpe.STAGE_PERMUTE, pmpe.STAGE_GATEUP, pmpe.STAGE_DOWN, pmpe.STAGE_COMBINE):
+        layer.forward(hd, pd, out=split, stages=st)
+    for _ in range(3):
+        out = layer.forward(hd, pd).clone()
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), split.view(torch.int16))
