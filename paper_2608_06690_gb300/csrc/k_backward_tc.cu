@@ -111,10 +111,13 @@ __device__ void build_groups(GroupTable &gt, const uint32_t *offsets, int g0, in
     __syncthreads();
 }
 
-// Bounded wait for the drain at exit: every copy a loader issued has landed
-// (the last use of each stage, after `issued` stages up to `stage` in `phase`).
+// Bounded wait for the drain at exit, by a whole warp: every copy a loader issued
+// has landed (the last use of each stage, after `issued` stages up to `stage` in
+// `phase`).  The lanes meet first: lanes already polling can keep the elected lane
+// from issuing the last copies that they wait for.
 __device__ __forceinline__ void drain_stages(uint32_t bar0, int stages, int issued, int stage, uint32_t phase)
 {
+    __syncwarp();
     for (int s = 0; s < stages && issued > 0; ++s) {
         if (issued < stages && s >= stage) break;
         const unsigned long long t0 = globaltimer_ns();

@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(kCombTmaThreads, kCombCtasPerSm) combine_tma_k
         }
         // no copy into this CTA's shared memory may still be in flight at its
         // exit (bounded: after an abort the consumers stopped early)
+        __syncwarp();
         if (lane == 0)
             for (int st = 0; st < p.stages; ++st)
                 if ((filled >> st) & 1u) {

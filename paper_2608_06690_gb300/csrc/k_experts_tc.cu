@@ -1112,7 +1112,9 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
             if (rank == 0) t = next;
         }
         // drain: every copy of the pair has landed before its CTAs exit (the
-        // last use of each stage)
+        // last use of each stage).  No lane polls before the elected one has
+        // issued its last copies.
+        __syncwarp();
         for (int s = 0; s < nst && rank == 0 && issued > 0; ++s) {
             if (issued < nst && s >= stage) break;
             const uint32_t last = s < stage ? phase : phase ^ 1u;

@@ -339,7 +339,9 @@ __global__ void __launch_bounds__(kRThreads, 1) router_tc_kernel(const RouterPar
             last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
-        // every copy this thread issued has landed before the CTA exits
+        // every copy this thread issued has landed before the CTA exits (a
+        // stage holds both lanes' copies: neither polls before both are issued)
+        __syncwarp(3u);
         for (int s = 0; s < p.stages; ++s)
             if ((filled >> s) & 1u) {
                 const unsigned long long w0 = globaltimer_ns();
@@ -970,6 +972,7 @@ __global__ void __launch_bounds__(kCThreads, 1) router_cluster_kernel(const Clus
                 }
             }
         }
+        __syncwarp();  // no lane polls before the elected one has issued the last copies
         for (int b = max(0, kb - stages); b < kb; ++b) {  // the last use of each stage has landed
             const unsigned long long w0 = globaltimer_ns();
             while (!mbar_try_wait(full_bar(b % stages), (uint32_t)(b / stages) & 1u))
@@ -1098,6 +1101,7 @@ __global__ void __launch_bounds__(kCThreads, 1) router_cluster_kernel(const Clus
             bulk_copy_to_peer(dsmem_addr(sbase + part_bytes + (uint32_t)q * slice_bytes, (uint32_t)o),
                               sbase + (uint32_t)o * slice_bytes, slice_bytes, dsmem_addr(rcv_bar, (uint32_t)o));
     }
+    __syncwarp();  // thread 0's copies are issued before its warp polls for them
     bool received = true;
     {
         const unsigned long long w0 = globaltimer_ns();

@@ -84,6 +84,26 @@ def test_parity_with_oracle(name):
     assert rep["excused"] <= max(2, shape.T // 50), rep["excused"]
 
 
+@pytest.mark.parametrize("consecutive", [False, True])
+@pytest.mark.parametrize("H, k, renormalize", [(128, 4, True), (384, 9, False)])
+def test_one_cta_router(H, k, renormalize, consecutive):
+    """The cluster router on clusters of one CTA (pools of at most 128 experts, so
+    many tokens that clusters of two would take two waves): both halves of H in
+    one and in three K steps, pools with a remainder, both softmaxes, and tiles of
+    consecutive tokens (loaded by TMA) and of scattered ones (gathered)."""
+    T = 64 * torch.cuda.get_device_properties(0).multi_processor_count + 77
+    shape = LayerShape(T=T, H=H, I=128, E_pub=40, E_priv=9, E_sh=0, k=k, renormalize=renormalize)
+    pol = "iid"
+    if consecutive:
+        pol = torch.zeros(T, dtype=torch.uint8)
+        pol[T // 3:2 * T // 3] = inp.ALLOW
+    w, h, pol = make_layer(shape, 150 + H, policy=pol)
+    gpu = run_gpu_layer(shape, *to_device(w, h, pol))
+    check_against_oracle(shape, w, h, pol, gpu)
+    check_audit(shape, pol, gpu)
+    check_dispatch(shape, h, gpu)
+
+
 def test_expert_loads_0_1_and_152_rows():
     """Empty experts, a single-row expert and a 152-row expert (the shapes of
     the dispatch failures recorded in App. H) in one batch."""
