@@ -341,9 +341,9 @@ __device__ __forceinline__ void prefetch_first_wave(const TcParams &p, bool by_p
     }
 }
 
-// Arrival at a grid barrier: a release add, so that the writes the CTA
-// barrier before it ordered (every thread's) are visible to whoever
-// acquires the count.
+// Arrival at a grid barrier (or on a readiness counter): a release add, so that
+// the writes the barrier before it ordered (of every thread of the CTA, or of the
+// warp) are visible to whoever acquires the count.
 __device__ __forceinline__ void grid_arrive(uint32_t *ctr)
 {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(ctr) : "memory");
@@ -1047,11 +1047,15 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
                     }
                     __nanosleep(128);
                 }
-                // the async proxy (TMA) reads what the generic acquire observed
-                asm volatile("fence.proxy.async.global;\n" ::: "memory");
             }
             ok = __all_sync(~0u, ok);
             if (!ok) break;
+            if (t.down() && p.has_gu) {
+                // the async proxy reads what lane 0's acquire observed: the fence in
+                // every lane, since any may be the one elected to issue the copies
+                __syncwarp();
+                asm volatile("fence.proxy.async.global;\n" ::: "memory");
+            }
             auto advance = [&]() {
                 if (++stage == nst) { stage = 0; phase ^= 1u; }
             };
@@ -1418,13 +1422,13 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
                     atomicAdd(p.shared_rows, (unsigned)t.rows);
             }
             if (gu && p.has_down) {
-                // release this warp's activation columns to the down tiles
-                // that read them (through TMA, after an acquire and a proxy fence)
-                __threadfence();
+                // release this warp's activation columns to the down tiles that read
+                // them (through TMA, after an acquire and a proxy fence): the release
+                // add follows the warp barrier, so it covers every lane's stores
                 __syncwarp();
                 if (lane == 0) {
                     asm volatile("fence.proxy.async.global;\n" ::: "memory");
-                    atomicAdd(p.ready + tt.mpre[t.g] + t.m_tile, 1u);
+                    grid_arrive(p.ready + tt.mpre[t.g] + t.m_tile);
                 }
                 __syncwarp();
             }

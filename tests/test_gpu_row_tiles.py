@@ -123,3 +123,27 @@ def test_short_tiles_round_the_queue(T):
         out = layer.forward(hd, pd).clone()
         torch.cuda.synchronize()
         assert torch.equal(out.view(torch.int16), split.view(torch.int16))
+
+
+@pytest.mark.parametrize("T, E_sh", [(100, 0), (128, 2), (700, 0), (1500, 2)])
+def test_down_tiles_read_this_launchs_activations(T, E_sh):
+    """Forwards of two inputs in turn on one workspace, whose activation rows still
+    hold the other input's values when a launch starts: a down tile that read a row
+    before this launch's gate/up tiles had stored it would show.  Same bits as the
+    two GEMMs in separate launches."""
+    from paper_2608_06690_gb300 import pmpe
+    shape = LayerShape(T=T, H=256, I=256, E_pub=12, E_priv=4, E_sh=E_sh, k=1, renormalize=True)
+    w, h, pol = make_layer(shape, 160 + T)
+    wd, hd, pd = to_device(w, h, pol)
+    layer = pmpe.MoeLayer(shape, wd)
+    ins = [hd, (hd * -0.5).contiguous()]
+    ref = []
+    for x in ins:
+        split = torch.full((T, shape.H), float("nan"), dtype=torch.bfloat16, device="cuda")
+        for st in (pmpe.STAGE_ROUTE | pmpe.STAGE_PERMUTE, pmpe.STAGE_GATEUP, pmpe.STAGE_DOWN, pmpe.STAGE_COMBINE):
+            layer.forward(x, pd, out=split, stages=st)
+        ref.append(split)
+    got = [layer.forward(ins[i & 1], pd).clone() for i in range(40)]
+    torch.cuda.synchronize()
+    for i, out in enumerate(got):
+        assert torch.equal(out.view(torch.int16), ref[i & 1].view(torch.int16)), i
