@@ -856,6 +856,7 @@ __global__ void __launch_bounds__(kTcThreads<kRoute>, 1) expert_gemm_tc_kernel(c
         // each role waits for every CTA's arrival (wait_dispatch) only before
         // it first reads what other CTAs wrote here, so that the tile table,
         // the first weight loads and the other CTAs' arrivals overlap
+        fence_proxy_async_smem();  // this thread's use of the ring, before the GEMM's copies land there
         __syncthreads();
         if (tid == 0) grid_arrive(p.grid_bar);
     }

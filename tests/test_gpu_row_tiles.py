@@ -147,3 +147,23 @@ def test_down_tiles_read_this_launchs_activations(T, E_sh):
     torch.cuda.synchronize()
     for i, out in enumerate(got):
         assert torch.equal(out.view(torch.int16), ref[i & 1].view(torch.int16)), i
+
+
+@pytest.mark.parametrize("T", [500, 16128])
+def test_dispatch_table_in_the_ring(T):
+    """The expert launch derives the dispatch order in the ring's memory before the
+    first copies land there; at T = 16128 its table of 384 experts x 127 router
+    tiles fills the ring.  Same bits as the dispatch and the GEMMs in launches of
+    their own."""
+    from paper_2608_06690_gb300 import pmpe
+    shape = LayerShape(T=T, H=1024, I=1024, E_pub=256, E_priv=128, E_sh=0, k=1, renormalize=True)
+    w, h, pol = make_layer(shape, 170, device="cuda")
+    wd, hd, pd = to_device(w, h, pol)
+    layer = pmpe.MoeLayer(shape, wd)
+    split = torch.full((T, shape.H), float("nan"), dtype=torch.bfloat16, device="cuda")
+    for st in (pmpe.STAGE_ROUTE, pmpe.STAGE_PERMUTE, pmpe.STAGE_GATEUP, pmpe.STAGE_DOWN, pmpe.STAGE_COMBINE):
+        layer.forward(hd, pd, out=split, stages=st)
+    for _ in range(3):
+        out = layer.forward(hd, pd).clone()
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), split.view(torch.int16))
