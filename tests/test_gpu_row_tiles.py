@@ -1,13 +1,27 @@
 """The expert GEMMs' row tiles (N of 32 to 256 tokens, tiles of equal size per
 expert) at the edges of their sizes, for a hidden size whose last 256-row weight
 block is half empty, and the ways the gate and up tensors can lie in memory."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2608_06690_gb300.inputs import LayerShape
 from pmpe_testlib import check_against_oracle, check_audit, check_dispatch, make_layer, run_gpu_layer, to_device
 
 pytestmark = pytest.mark.gpu
+
+
+def check_gradients(shape, w, h, pol, dout, got):
+    """The private gradients and d_hidden of one pass against the oracle, at twice
+    the forward's tolerance, as in the backward's tests."""
+    L = oracle.Layer(shape, dict(w, hidden=h), pol.numpy())
+    d = dout.cpu().double().numpy()
+    ref = dict(oracle.backward_private(L, d), d_hidden=oracle.backward_input(L, d))
+    for n, v in got.items():
+        err = np.abs(v.cpu().double().numpy() - ref[n])
+        assert err.max() <= 2e-2 * max(np.abs(ref[n]).max(), 1e-30), n
+        assert err.sum() <= 1e-2 * max(np.abs(ref[n]).sum(), 1e-30), n
 
 
 @pytest.mark.parametrize("T", [1, 32, 33, 97, 224, 225, 256, 257, 289, 513, 800])
@@ -53,9 +67,6 @@ def test_backward_rows_of_one_expert(T):
     """The backward's row tiles over one expert's rows per pool and one shared
     expert: both gradients against the oracle, and the same bits from the
     forward's saved accumulators as from the recompute."""
-    import numpy as np
-
-    import oracle
     from paper_2608_06690_gb300 import pmpe
     shape = LayerShape(T=T, H=384, I=256, E_pub=1, E_priv=1, E_sh=1, k=1, renormalize=False)
     w, h, _ = make_layer(shape, 90 + T)
@@ -71,14 +82,9 @@ def test_backward_rows_of_one_expert(T):
     torch.cuda.synchronize()
     (g, dh), (g2, dh2) = got
     assert torch.equal(dh, dh2)
-    L = oracle.Layer(shape, dict(w, hidden=h), pol.numpy())
-    ref = dict(oracle.backward_private(L, dout.double().numpy()),
-               d_hidden=oracle.backward_input(L, dout.double().numpy()))
-    for n, v in dict(g, d_hidden=dh).items():
-        assert n == "d_hidden" or torch.equal(v, g2[n]), n
-        err = np.abs(v.cpu().double().numpy() - ref[n])  # twice the forward's tolerance, as in the backward's tests
-        assert err.max() <= 2e-2 * max(np.abs(ref[n]).max(), 1e-30), n
-        assert err.sum() <= 1e-2 * max(np.abs(ref[n]).sum(), 1e-30), n
+    for n in g:
+        assert torch.equal(g[n], g2[n]), n
+    check_gradients(shape, w, h, pol, dout, dict(g, d_hidden=dh))
 
 
 @pytest.mark.parametrize("E_pub, E_priv", [(2, 2), (7, 3), (3, 7), (8, 1), (5, 4)])
@@ -99,10 +105,13 @@ def test_interleaved_pools(E_pub, E_priv):
     dout = torch.randn((shape.T, shape.H), generator=torch.Generator().manual_seed(5)).to(torch.bfloat16).cuda()
     layer.forward(hd, pd)
     g_sep = {n: v.clone() for n, v in layer.backward_private(hd, pd, dout).items()}
-    g, _ = layer.backward(hd, pd, dout)
+    dh_sep = layer.backward_input(hd, pd, dout).clone()
+    g, dh = layer.backward(hd, pd, dout)
     torch.cuda.synchronize()
     for n in g:
         assert torch.equal(g[n], g_sep[n]), n
+    assert torch.equal(dh, dh_sep)
+    check_gradients(shape, w, h, pol, dout, dict(g, d_hidden=dh))
 
 
 @pytest.mark.parametrize("T", [40, 129, 600])
