@@ -69,10 +69,10 @@ struct GroupTable {
 };
 
 // All threads: fill the table (routed groups from the forward's dispatch
-// offsets).  tiles_per_row_block: tiles of a group per 128-row block (0:
-// every group has `fixed_tiles` tiles whatever its rows).
+// offsets).  tiles_per_row_block: tiles of a group per 128-row block (0 where the
+// tiles are not read).
 __device__ void build_groups(GroupTable &gt, const uint32_t *offsets, int g0, int G, int R, int shared_T,
-                             int tiles_per_row_block, int fixed_tiles)
+                             int tiles_per_row_block)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int p0 = shared_T ? 0 : (int)min(offsets[g0], (uint32_t)R);
@@ -85,7 +85,7 @@ __device__ void build_groups(GroupTable &gt, const uint32_t *offsets, int g0, in
         const int rows = e - b;
         gt.rows[q] = rows;
         gt.off[q] = b - p0;
-        gt.tiles[q + 1] = tiles_per_row_block ? ((rows + BM - 1) / BM) * tiles_per_row_block : fixed_tiles;
+        gt.tiles[q + 1] = ((rows + BM - 1) / BM) * tiles_per_row_block;
         gt.pad[q] = (rows + kPad - 1) / kPad * kPad;  // made exclusive prefix below
     }
     __syncthreads();
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams 
     pdl_trigger();
     pdl_wait();
     const int nt = p.I / 128;
-    build_groups(gt, p.offsets, p.g0, p.G, p.R, p.shared_T, nt, 0);
+    build_groups(gt, p.offsets, p.g0, p.G, p.R, p.shared_T, nt);
     const int total = gt.tiles[p.G];
     const int p0 = p.shared_T ? 0 : (int)min(p.offsets[p.g0], (uint32_t)p.R);
     // saved rows: routed [R][2I] (G | U), then shared [T][2 G I] (all G, then all U)
@@ -922,7 +922,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_wgrad_tc_kernel(const WgParam
     }
     if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
-    build_groups(gt, p.offsets, p.g0, p.G, p.R, 0, 0, 0);
+    build_groups(gt, p.offsets, p.g0, p.G, p.R, 0, 0);
     tc_fence_before();
     cluster_sync_all();  // both CTAs' barriers and TMEM are ready
     tc_fence_after();

@@ -198,15 +198,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-// 3-D tile load: box coordinates (x, y, z) of a map made by encode_3d_blocks.
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y, int z)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];\n" ::
-            "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
-        : "memory");
-}
-
 // L2 eviction-priority policies for the cache-hinted copies below: data read
 // once and streamed through L2 (evict_first), and data read again soon by
 // other CTAs or phases of the same kernel (evict_last).
