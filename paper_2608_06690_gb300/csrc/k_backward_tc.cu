@@ -29,7 +29,8 @@
 // Every launch keeps 160 to 192 KB of operand stages in flight and two FP32
 // accumulators, so the epilogue of one tile overlaps the MMAs of the next.  CTA roles (224 threads): warps 0 and 6 issue
 // the TMA loads of the first and the second operand, warp 1 allocates TMEM and
-// issues the MMAs, warps 2-5 drain TMEM (one tile row per thread).  Warps 0, 1
+// issues the MMAs, warps 2-5 drain TMEM (a warp's 32 lanes are 32 output columns
+// in the row launches, 32 rows of a gradient in the weight gradients).  Warps 0, 1
 // and 6 run their loops as whole warps, with one elected lane issuing (elect_one).  Every wait
 // is bounded in time; on expiry the CTA records PMPE_STATUS_PIPELINE_TIMEOUT,
 // stops, waits (bounded) for its copies and MMAs in flight, frees TMEM and exits.
@@ -231,7 +232,7 @@ struct PairMaps {
     CUtensorMap tok[kTokBoxes];  // the contracted rows' operand (K-major), by box rows
     CUtensorMap w0[2], w1[2];    // per weight pool, 64 x 64 x 2 3-D boxes (MN-major); gate/up: 64-row boxes of
                                  // the gate and the up rows, where one box cannot hold both
-    CUtensorMap gu[2];           // gate/up: 64 gate and 64 up rows (encode_3d_two)
+    CUtensorMap gu[2];           // gate/up: 64 gate and 64 up rows (encode_gate_up)
 };
 
 // The gate/up recompute's outputs (GuOut) or C.
@@ -524,10 +525,13 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    // An early start of the next launch pays only when it is another of these
-    // GEMMs (private gradients at T = 1000 437 -> 429 us): a small kernel's CTAs
-    // that started beside a GEMM's ran with the L1 its shared memory left over
-    // (the T = 4096 step 1086 -> 1110 us with every launch triggering).
+    // An early start of the next launch pays when it is another of these GEMMs
+    // (private gradients at T = 1000 437 -> 429 us) and costs when it is not: a small
+    // kernel's CTAs that started beside a GEMM's ran with the L1 its shared memory
+    // left over (the T = 4096 step 1086 -> 1110 us with every launch triggering).
+    // The recompute triggers always: dA follows it, but in the private gradients,
+    // where the router's small kernels do and it makes no difference (425.3 us with
+    // the trigger, 425.3 without).
     if (kGU || p.gemm_next) pdl_trigger();
     if (warp == 1) tmem_alloc_pair(smem_u32(&s_tmem), kTmemCols);
     pdl_wait();
@@ -740,11 +744,10 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_rows_pair_kernel(const RowsPa
 // The gate/up launch's outputs from the forward's saved accumulators G | U
 // ([R][2I] FP32) instead of a recomputing GEMM: one warp per routed row and
 // 128-column tile, four columns per lane (coalesced rows), with the
-// epilogue's per-element arithmetic and its dL/dw summation order
-// (chunk_tree_sum, then the four 32-column chunks in order), so [dG | dU],
-// w act and the dL/dw partials are bitwise those of bwd_rows_pair_kernel.  Tiles and the
-// padded layout come from the same group table; padded tail rows are written
-// as zeros.
+// epilogue's per-element arithmetic and its order of summing dL/dw over 32
+// columns, so [dG | dU], w act and the dL/dw partials are bitwise those of
+// bwd_rows_pair_kernel, in the same padded layout; padded tail rows are written as
+// zeros.
 __global__ void __launch_bounds__(256) bwd_swiglu_saved_kernel(const RowsParams p, const float *saved_gu, bf16 *dgu,
                                                                bf16 *wact)
 {

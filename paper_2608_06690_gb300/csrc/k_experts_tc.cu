@@ -24,11 +24,13 @@
 //
 // What bounds it: HBM (the weights) up to a few thousand tokens, then the rate
 // at which L2 delivers the operands (32 KB a stage and CTA in 512 clocks at the
-// full MMA rate).  Forward, against single-CTA tiles of 128 tokens x 256 weight
-// rows: Qwen3 shape T = 4096 437 -> 366 us, T = 16384 1229 -> 1037 us, T = 777
-// 271 -> 264 us, T = 64 213 -> 211 us; DeepSeek shape T = 8192 1020 -> 867 us.
-// Half of that is the roles' own time a stage (tc_ptx.cuh: the waits' timer, the
-// elected lane) and a tile (the queue below).
+// full MMA rate).  Whole forward, against single-CTA tiles of 128 tokens x 256
+// weight rows with the roles' loops in single threads (both on one GPU; the
+// figures hold the other steps described here too): Qwen3 shape T = 4096 432 -> 369
+// us, T = 16384 1248 -> 1060 us, T = 777 275 -> 266 us, T = 64 215 -> 207 us;
+// DeepSeek shape T = 8192 1037 -> 884 us.  Half of that is the roles' own time a
+// stage (tc_ptx.cuh: the waits' timer, the elected lane) and a tile (the queue
+// below).
 //
 // The pairs walk a tile list built on the device from the dispatch offsets:
 // no host sync, and empty experts contribute no tile.  The list holds every
@@ -270,8 +272,9 @@ __device__ __forceinline__ int total_tiles(const TcParams &p, const TileTable &t
 // routed down tiles (K = I) instead of the shared group's (K = E_sh I, the
 // launch's longest tiles), which otherwise made the last wave uneven; there
 // the shared group's gate/up tiles, the last of the gate/up list, are long
-// finished.  The gate/up GEMM keeps the groups in id order (the copy warps
-// fill no stage after one whose A comes through TMA).  down_place inverts it.
+// finished.  The gate/up GEMM's list ends with the shared group: its token rows
+// come through TMA, and the gather warps fill no stage after such a tile.
+// down_place inverts it.
 __device__ __forceinline__ int down_group(const TcParams &p, int L)
 {
     if (p.E_sh == 0) return L;

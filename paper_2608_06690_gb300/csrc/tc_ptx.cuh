@@ -373,7 +373,9 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t local, uint32_t rank)
 }
 // One arrival on a barrier of another CTA of the cluster (address from
 // dsmem_addr), with the default semantics of a local arrival: what it hands
-// over is TMEM, whose reads tcgen05.wait has completed.  (A release at cluster
+// over is this CTA's own TMEM, whose reads tcgen05.wait has completed, a queue slot
+// that has been read, or rows in this CTA's shared memory that have landed and are
+// fenced for the pair's MMAs.  (A release at cluster
 // scope waits for the thread's TMA stores in flight as well: about 3,000
 // clocks a tile in the weight-gradient epilogue.)
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t remote_bar)
